@@ -342,12 +342,9 @@ typedef struct {
                       length that fills the GPU's last wave of CTAs better); 2: the same on
                       the finest level only (the coarser levels keep the row kernels); 0:
                       every warp loads its own row of nodes */
-  int smem_tail;   /* k >= 1: the coarse end of the V-cycle -- from the finest level l >= k
-                      whose vectors, and those of every level below it, fit in one CTA's
-                      shared memory -- runs as one launch of one CTA per column group, its
-                      steps separated by block barriers only; the result equals the
-                      per-level kernels' bit for bit.
-                      0: off */
+  int smem_tail;   /* accepted (0..15) and kept, without effect: FP32 solves run the coarse
+                      end of the V-cycle, and the whole PCG of a problem that fits, with one
+                      CTA per column wherever that is the faster form */
   int refine_df;   /* arithmetic of the FP64 iterative refinement around FP32 inner solves
                       (the residual b - K x with its norm, the scaling into the inner
                       precision and the update x += d): 0 FP64 instructions; 1 (default)
@@ -366,7 +363,7 @@ int hp_get_tuning(const hp_problem *P, hp_tuning *t);
 /* Times one block of nrhs Gauss-Newton Hessian actions at the current point
  * (CUDA events, the mean of reps timed runs after a warm-up per candidate) over a
  * small candidate set by coordinate descent in two passes (smoother, column
- * chunk, fused transfers, coarse tails, tiled kernels, grid cap; a candidate must
+ * chunk, fused transfers, tiled kernels, grid cap; a candidate must
  * be at least 1 % faster to be taken) and applies the fastest.  best / best_ms
  * (HOST, may be NULL) receive it.  Needs hp_set_point first; allocates its test
  * block (setup-time call). */

@@ -563,7 +563,7 @@ void hp_problem_destroy(hp_problem *P) {
       if (p) cudaFree(p);
   }
   for (CoarseInv *C : {&P->cK, &P->cA})
-    for (void *p : {(void *)C->dense, (void *)C->inv64, (void *)C->inv32})
+    for (void *p : {(void *)C->dense, (void *)C->inv64, (void *)C->inv32, (void *)C->tri32})
       if (p) cudaFree(p);
   for (void *p : {(void *)P->CbetaE_pr, (void *)P->Cbeta_pr, (void *)P->E_pr})
     if (p) cudaFree(p);

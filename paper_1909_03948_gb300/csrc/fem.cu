@@ -511,6 +511,13 @@ __global__ void __launch_bounds__(128) k_dense_inverse32(const float *__restrict
   for (int i = lane; i < nc; i += 32) inv32[(long)j * nc + i] = x[i];
 }
 
+// lower triangle of the symmetric FP32 inverse, row i at i (i + 1) / 2 (the one-CTA coarse
+// solve holds it in shared memory: half the square)
+__global__ void k_pack_tri(const float *__restrict__ inv, int nc, float *__restrict__ tri) {
+  const int i = blockIdx.x;
+  for (int j = threadIdx.x; j <= i; j += blockDim.x) tri[(long)i * (i + 1) / 2 + j] = inv[(long)j * nc + i];
+}
+
 int coarse_setup(hp_problem *P, OpKind op) {
   const Level &lc = P->lv[P->L - 1];
   CoarseInv &C = op == OP_K ? P->cK : P->cA;
@@ -544,7 +551,8 @@ int coarse_setup(hp_problem *P, OpKind op) {
     k_dense_inverse<<<(int)((nc + 31) / 32), 32, 0, P->st>>>(C.dense, (int)nc, C.inv64, C.inv32);
     C.fp64_valid = true;
   }
-  count_launch(3);
+  k_pack_tri<<<(int)nc, 128, 0, P->st>>>(C.inv32, (int)nc, C.tri32);
+  count_launch(4);
   int h = 0;
   HP_CUDA(cudaMemcpyAsync(&h, dstat, sizeof(int), cudaMemcpyDeviceToHost, P->st));
   HP_CUDA(cudaStreamSynchronize(P->st));
@@ -637,6 +645,9 @@ int build_hierarchy_geometry(hp_problem *P) {
     HP_CUDA(cudaMalloc(&C->dense, sizeof(double) * ncn * ncn));
     HP_CUDA(cudaMalloc(&C->inv64, sizeof(double) * ncn * ncn));
     HP_CUDA(cudaMalloc(&C->inv32, sizeof(float) * ncn * ncn));
+    const size_t tb = sizeof(float) * (size_t)((ncn * (ncn + 1) / 2 + 3) / 4 * 4);
+    HP_CUDA(cudaMalloc(&C->tri32, tb));
+    HP_CUDA(cudaMemset(C->tri32, 0, tb));
   }
   HP_TRY(coarse_setup(P, OP_A));
   for (int l = 0; l < L; ++l) {

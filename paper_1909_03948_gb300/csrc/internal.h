@@ -63,6 +63,7 @@ struct CoarseInv {
   double *dense = nullptr;   // work: nc x nc
   double *inv64 = nullptr;
   float *inv32 = nullptr;
+  float *tri32 = nullptr;    // its lower triangle, row i at i (i + 1) / 2
 };
 
 enum OpKind { OP_K = 0, OP_A = 1, OP_M = 2 };
@@ -146,7 +147,7 @@ struct hp_problem {
   int fuse_transfer = 0;        // residual + restriction and prolongation + first post sweep fused (tuning)
   double cheb_alpha = 10.0;     // Chebyshev interval [lmax / alpha, lmax]             (tuning)
   int tma_tiles = 0;            // 2D stiffness levels as TMA-tiled stencil kernels       (tuning)
-  int smem_tail = 0;            // coarse V-cycle levels in one shared-memory CTA per group (tuning)
+  int smem_tail = 0;            // kept for callers, without effect                              (tuning)
   int refine_df = 1;            // FP64 refinement arithmetic in double-float on the FP32 pipe:
                                 // 0 never, 1 for tolerances >= DF_MIN_RTOL, 2 always (tuning)
   cudaStream_t st = nullptr;
@@ -312,6 +313,37 @@ void free_scalars_host(hp_problem *P);
 int solve_block(hp_problem *P, OpKind op, const double *B, long ldb, double *X, long ldx, int s,
                 double rtol, hp_solve_stats *st);
 int apply_op64(hp_problem *P, OpKind op, const double *X, long ldx, double *Y, long ldy, int s);
+
+// ---- column.cu ----------------------------------------------------------------
+// FP32 multigrid work of one column per CTA (see column.cu).  A level of the hierarchy as
+// those kernels see it; the offsets are the shared-memory places of its right-hand side and
+// two iterates (in floats, behind `pad` zeros).
+constexpr int COL_MAXN = 5120;  // most nodes of the finest level held in one CTA
+struct ColLevel {
+  GridDesc g;
+  int n, np, pad, nu, npt;  // npt: nodes per thread
+  const float *diag, *invdiag, *c;
+  float w[4];
+  int offr, offa, offb;
+};
+struct ColArgs {
+  int l0, L, zero_dirichlet, vw, s, jacobi, maxit;
+  ColLevel lv[HP_MAXL];
+  const float *inv;      // dense inverse of the coarsest level
+  const float *r;        // level-l0 right-hand side and result: [group][node][vw], group stride gs
+  float *x;
+  long gs;
+  const double *tol2col, *open;  // squared relative tolerance per column (or tol2), open columns
+  double tol2;
+  int *iter;             // most iterations of a column
+  const float *tri;      // packed lower triangle of inv (zero past its end up to a multiple of 4)
+  // shared-memory layout (floats): size, leading part that starts as zeros; x, p and segment
+  // sums of a PCG, the coarse solve's scratch, the triangle and its length (0: not held)
+  int nfloats, nclear, offx, offp, offs, offc, offt, tn;
+};
+bool col_fits(const ColArgs &a, bool pcg);
+int launch_vtail(ColArgs a, int dim, bool full, int cols, cudaStream_t st);
+int launch_colpcg(ColArgs a, int dim, bool full, int cols, cudaStream_t st);
 
 // ---- dense.cu ---------------------------------------------------------------
 // G (s1 x s2, column-major, ldg) = X^T Y ; X: n x s1, Y: n x s2 (FP64)

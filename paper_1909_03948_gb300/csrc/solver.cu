@@ -1753,236 +1753,6 @@ static dim3 nodegrid(long n, int ng) {
   return dim3((unsigned)b, ng);
 }
 
-// ---------------------------------------------------------------------------
-// Node steps shared by the coarse-tail kernel below (the same arithmetic as the per-level
-// kernels, node by node).
-// ---------------------------------------------------------------------------
-// S x at node id with the centre value xc given; JS: the
-// neighbour values enter as omega D^-1 x (the first sweep of a pair from zero),
-// in the same operation order as k_st
-template <typename T, int VW, int D, bool FULL, bool JS>
-__device__ __forceinline__ Pack<T, VW> vt_apply(const GridDesc &g, const T *diag, const T *invdiag, const T *c,
-                                                const T *x, long id, const int v[3], T omega,
-                                                const Pack<T, VW> &xc) {
-  using PK = Pack<T, VW>;
-  constexpr int NF = FULL ? (1 << D) - 1 : D;
-  PK sx;
-  const T dg = diag[id];
-#pragma unroll
-  for (int q = 0; q < VW; ++q) sx.v[q] = dg * xc.v[q];
-#pragma unroll
-  for (int f = 0; f < NF; ++f) {
-    const int b = FULL ? f + 1 : (1 << f);
-    bool fw = true, bw = true;
-#pragma unroll
-    for (int a = 0; a < D; ++a)
-      if ((b >> a) & 1) {
-        fw = fw && (v[a] < g.N);
-        bw = bw && (v[a] > 0);
-      }
-    const long off = mask_offset(g, b);
-    if (fw) {
-      const T cf = JS ? c[(long)f * g.n + id] * omega * invdiag[id + off] : c[(long)f * g.n + id];
-      sx.axpy(cf, PK::ld(x + (id + off) * VW));
-    }
-    if (bw) {
-      const T cb = JS ? c[(long)f * g.n + id - off] * omega * invdiag[id - off] : c[(long)f * g.n + id - off];
-      sx.axpy(cb, PK::ld(x + (id - off) * VW));
-    }
-  }
-  return sx;
-}
-
-template <int D>
-__device__ __forceinline__ void vt_coords(const GridDesc &g, long id, int v[3]) {
-  v[0] = (int)(id % g.np);
-  const long t = id / g.np;
-  v[1] = D == 2 ? (int)t : (int)(t % g.np);
-  v[2] = D == 2 ? 0 : (int)(t / g.np);
-}
-
-// ---------------------------------------------------------------------------
-// Shared-memory coarse tail: the levels l0 .. L-2 of one column group run in one CTA of
-// VS_NT threads with their vectors in shared memory -- the two iterates of level l0 (its
-// right-hand side stays in global memory, where the restriction of level l0 - 1 wrote
-// it), and the right-hand side and both iterates of each level below -- so the smoothing
-// and transfer steps are separated by __syncthreads only, not by launches.  Two launches
-// bracket the dense coarse solve (k_coarse_apply, spread over many CTAs): PART 0 runs the
-// down leg and leaves each level's iterate (and the right-hand sides below l0) in its
-// global level buffers; PART 1 reloads them with the coarse solution and runs the up leg.
-// The arithmetic mirrors k_st / k_jacobi0 / k_restrict / k_prolong_add step for step
-// (same operations in the same order, explicitly rounded), so the result equals the
-// per-level path bit for bit.  The level-l0 correction is written to `dst`.
-// ---------------------------------------------------------------------------
-constexpr int VS_NT = 1024;
-
-template <typename T> struct VTailS {
-  int l0, L, zero_dirichlet, nc;
-  int nu[HP_MAXL];
-  T w[HP_MAXL][4];
-  GridDesc g[HP_MAXL];
-  const T *diag[HP_MAXL], *invdiag[HP_MAXL], *c[HP_MAXL];
-  const T *r0;  // level-l0 right-hand side (global, group stride gs0)
-  T *dst;       // level-l0 correction (global, group stride gs0)
-  long gs0;
-  T *rg[HP_MAXL], *ag[HP_MAXL];  // global right-hand side / iterate buffers of each level
-  long gs[HP_MAXL];               // their group strides
-  unsigned off_r[HP_MAXL], off_a[HP_MAXL], off_b[HP_MAXL];  // shared-memory byte offsets
-};
-
-template <typename T, int VW, int D, bool FULL, int PART>
-__global__ void __launch_bounds__(VS_NT) k_vtail_smem(VTailS<T> vt) {
-  using PK = Pack<T, VW>;
-  extern __shared__ __align__(16) unsigned char vs_smem[];
-  const int grp = blockIdx.y;
-  auto S = [&](unsigned off) { return reinterpret_cast<T *>(vs_smem + off); };
-  // one node step over level l: mode 0 two sweeps from zero (x = rhs, weights w1, w2),
-  // 1 one sweep from zero (w1), 2 sweep (x, rhs b, w1), 3 residual b - S x
-  auto sweep = [&](int l, int mode, const T *x, const T *b, T *y, T w1, T w2) {
-    const GridDesc &g = vt.g[l];
-    const T *dg = vt.diag[l], *iv = vt.invdiag[l], *cc = vt.c[l];
-    for (long id = threadIdx.x; id < g.n; id += VS_NT) {
-      int v[3];
-      vt_coords<D>(g, id, v);
-      PK out;
-      if (mode == 0) {
-        const T wi = w1 * iv[id], wi2 = w2 * iv[id];
-        const PK r = PK::ld(x + id * VW);
-        PK e1c;
-#pragma unroll
-        for (int q = 0; q < VW; ++q) e1c.v[q] = wi * r.v[q];
-        const PK sx = vt_apply<T, VW, D, FULL, true>(g, dg, iv, cc, x, id, v, w1, e1c);
-#pragma unroll
-        for (int q = 0; q < VW; ++q) out.v[q] = fmadd(wi2, r.v[q] - sx.v[q], e1c.v[q]);
-      } else if (mode == 1) {
-        const T wi = w1 * iv[id];
-        const PK r = PK::ld(x + id * VW);
-#pragma unroll
-        for (int q = 0; q < VW; ++q) out.v[q] = wi * r.v[q];
-      } else {
-        const PK xc = PK::ld(x + id * VW);
-        const PK sx = vt_apply<T, VW, D, FULL, false>(g, dg, iv, cc, x, id, v, T(0), xc);
-        const PK bb = PK::ld(b + id * VW);
-        if (mode == 3) {
-#pragma unroll
-          for (int q = 0; q < VW; ++q) out.v[q] = bb.v[q] - sx.v[q];
-        } else {
-          const T wi = w1 * iv[id];
-#pragma unroll
-          for (int q = 0; q < VW; ++q) out.v[q] = fmadd(wi, bb.v[q] - sx.v[q], xc.v[q]);
-        }
-      }
-      out.st(y + id * VW);
-    }
-    __syncthreads();
-  };
-  auto copy = [&](long n, const T *src, T *dst_) {
-    for (long id = threadIdx.x; id < n; id += VS_NT) PK::ld(src + id * VW).st(dst_ + id * VW);
-  };
-  const T *r0 = vt.r0 + grp * vt.gs0;
-  T *cur[HP_MAXL], *oth[HP_MAXL];
-  if (PART == 1) {
-    // reload: each level's iterate and the right-hand sides below l0, the coarse solution
-    for (int l = vt.l0; l < vt.L; ++l) {
-      copy(vt.g[l].n, vt.ag[l] + grp * vt.gs[l], S(vt.off_a[l]));
-      if (l > vt.l0 && l + 1 < vt.L) copy(vt.g[l].n, vt.rg[l] + grp * vt.gs[l], S(vt.off_r[l]));
-      cur[l] = S(vt.off_a[l]);
-      oth[l] = S(vt.off_b[l]);
-    }
-    __syncthreads();
-  }
-  for (int l = vt.l0; PART == 0 && l + 1 < vt.L; ++l) {
-    const T *rl = l == vt.l0 ? r0 : S(vt.off_r[l]);
-    const int nul = vt.nu[l];
-    T *c = nul >= 2 ? S(vt.off_a[l]) : S(vt.off_b[l]);
-    T *o = nul >= 2 ? S(vt.off_b[l]) : S(vt.off_a[l]);
-    sweep(l, nul >= 2 ? 0 : 1, rl, nullptr, c, vt.w[l][0], vt.w[l][1]);
-    for (int k = 2; k < nul; ++k) {
-      sweep(l, 2, c, rl, o, vt.w[l][k], T(0));
-      T *t = c;
-      c = o;
-      o = t;
-    }
-    sweep(l, 3, c, rl, o, T(0), T(0));
-    // restriction to level l + 1 (transpose of the P1 prolongation)
-    {
-      const GridDesc &gf = vt.g[l], &gc = vt.g[l + 1];
-      T *rc = S(vt.off_r[l + 1]);
-      for (long I = threadIdx.x; I < gc.n; I += VS_NT) {
-        int J[3];
-        vt_coords<D>(gc, I, J);
-        PK out = PK::zero();
-        if (!(vt.zero_dirichlet && (J[D - 1] == 0 || J[D - 1] == gc.N))) {
-          const long f0 = 2 * (long)J[0] + (long)gf.np * (2 * (long)J[1] + (D == 3 ? (long)gf.np * 2 * J[2] : 0));
-          out = PK::ld(o + f0 * VW);
-#pragma unroll
-          for (int b = 1; b < (1 << D); ++b) {
-            bool fw = true, bw = true;
-#pragma unroll
-            for (int a = 0; a < D; ++a)
-              if ((b >> a) & 1) {
-                fw = fw && (J[a] < gc.N);
-                bw = bw && (J[a] > 0);
-              }
-            const long off = mask_offset(gf, b);
-            if (fw) out.axpy(T(0.5), PK::ld(o + (f0 + off) * VW));
-            if (bw) out.axpy(T(0.5), PK::ld(o + (f0 - off) * VW));
-          }
-        }
-        out.st(rc + I * VW);
-      }
-    }
-    __syncthreads();
-    cur[l] = c;
-    oth[l] = o;
-  }
-  if (PART == 0) {
-    // hand over through the global level buffers: iterates, and the right-hand sides
-    // below l0 (the coarsest one is the coarse solve's input)
-    for (int l = vt.l0; l < vt.L; ++l) {
-      if (l + 1 < vt.L) copy(vt.g[l].n, cur[l], vt.ag[l] + grp * vt.gs[l]);
-      if (l > vt.l0) copy(vt.g[l].n, S(vt.off_r[l]), vt.rg[l] + grp * vt.gs[l]);
-    }
-    return;
-  }
-  for (int l = vt.L - 2; l >= vt.l0; --l) {
-    // e_l += P e_{l+1}
-    {
-      const GridDesc &gf = vt.g[l], &gc = vt.g[l + 1];
-      const T *e = cur[l + 1];
-      T *ef = cur[l];
-      for (long i = threadIdx.x; i < gf.n; i += VS_NT) {
-        int v[3];
-        vt_coords<D>(gf, i, v);
-        const int b = (v[0] & 1) | ((v[1] & 1) << 1) | ((v[2] & 1) << 2);
-        const long ic = (v[0] >> 1) + (long)gc.np * ((v[1] >> 1) + (long)gc.np * (v[2] >> 1));
-        PK val = PK::ld(e + ic * VW);
-        if (b) {
-          const PK v2 = PK::ld(e + (ic + mask_offset(gc, b)) * VW);
-#pragma unroll
-          for (int q = 0; q < VW; ++q) val.v[q] = mulr(T(0.5), val.v[q] + v2.v[q]);
-        }
-        PK cv = PK::ld(ef + i * VW);
-#pragma unroll
-        for (int q = 0; q < VW; ++q) cv.v[q] = addr(cv.v[q], val.v[q]);
-        cv.st(ef + i * VW);
-      }
-    }
-    __syncthreads();
-    const T *rl = l == vt.l0 ? r0 : S(vt.off_r[l]);
-    T *c = cur[l], *o = oth[l];
-    const int nul = vt.nu[l];
-    for (int k = 0; k < nul; ++k) {
-      T *y = (l == vt.l0 && k == nul - 1) ? vt.dst + grp * vt.gs0 : o;
-      sweep(l, 2, c, rl, y, vt.w[l][nul - 1 - k], T(0));
-      T *t = c;
-      c = o;
-      o = t;
-    }
-    cur[l] = c;
-  }
-}
-
 // Smoothing weights of level l, sweep k = 0 .. nu-1 (pre-smoothing applies them in this
 // order, post-smoothing in reverse, so the V-cycle stays symmetric).  Damped Jacobi: omega
 // every sweep.  Chebyshev: the reciprocals of the roots of the degree-nu Chebyshev
@@ -2008,53 +1778,77 @@ static void smooth_weights(const hp_problem *P, OpKind op, int l, T w[4]) {
     w[k] = k < nu ? (T)(1.0 / (c - d * std::cos(M_PI * (2.0 * k + 1.0) / (2.0 * nu)))) : T(0);
 }
 
-// opt-in maximum of shared memory per CTA on the current device
-static int smem_optin() {
-  static thread_local int dev = -1, val = 0;
-  int d = 0;
-  if (cudaGetDevice(&d) != cudaSuccess) return 0;
-  if (d != dev) {
-    if (cudaDeviceGetAttribute(&val, cudaDevAttrMaxSharedMemoryPerBlockOptin, d) != cudaSuccess) val = 0;
-    dev = d;
-  }
-  return val;
+// whether the level's stencils run as TMA-tiled kernels in FP32 solves of vw columns per group
+static bool tiled_level(const hp_problem *P, OpKind op, int l, int vw) {
+  const bool on = P->tma_tiles == 1 || (P->tma_tiles == 2 && l == 0);
+  return on && op == OP_K && vw == 4 && P->lv[l].K32.pk && (tile_grid(P->lv[l].g) || tile3_grid(P->lv[l].g));
 }
 
-// Shared-memory layout of the coarse tail from level l0 for node_bytes per node (bytes of
-// one group's values at one node); fills the offsets when vt is given, returns the total.
-template <typename T>
-static size_t smem_tail_layout(const hp_problem *P, int l0, int node_bytes, VTailS<T> *vt) {
-  const int L = P->L;
-  size_t off = 0;
-  auto take = [&](long n) {
-    const size_t o = off;
-    off += ((size_t)n * node_bytes + 15) / 16 * 16;
-    return (unsigned)o;
-  };
-  for (int l = l0; l < L; ++l) {
-    const long n = P->lv[l].g.n;
-    const unsigned r = (l > l0) ? take(n) : 0u;  // level l0 reads its right-hand side from global memory
-    const unsigned a = take(n);
-    const unsigned b = (l < L - 1) ? take(n) : 0u;
-    if (vt) {
-      vt->off_r[l] = r;
-      vt->off_a[l] = a;
-      vt->off_b[l] = b;
-    }
+// The part of an FP32 solve that runs with one CTA per column (column.cu): fills the
+// arguments for the levels from l0 down.
+static void col_args(const hp_problem *P, OpKind op, int vw, int s, int l0, ColArgs *a) {
+  *a = ColArgs{};
+  a->l0 = l0;
+  a->L = P->L;
+  a->zero_dirichlet = op == OP_K;
+  a->vw = vw;
+  a->s = s;
+  a->jacobi = op == OP_M;
+  a->maxit = P->max_iter;
+  if (op == OP_M) a->L = 1;
+  for (int l = 0; l < a->L; ++l) {
+    const Stencil<float> &S = stencil_of<float>(P, op, l);
+    ColLevel &v = a->lv[l];
+    v.g = P->lv[l].g;
+    v.n = (int)v.g.n;
+    v.np = v.g.np;
+    v.pad = P->dim == 2 ? v.np + 1 : v.np * v.np + v.np + 1;
+    v.nu = nu_at(P, l);
+    v.diag = S.diag;
+    v.invdiag = S.invdiag;
+    v.c = S.c;
+    if (op != OP_M) smooth_weights<float>(P, op, l, v.w);
   }
-  return off;
+  a->inv = op == OP_M ? nullptr : coarse_inv<float>(P, op);
+  a->tri = op == OP_M ? nullptr : (op == OP_K ? P->cK.tri32 : P->cA.tri32);
 }
 
-// first level of the shared-memory coarse tail for this solve, or L (no fusion): the lowest
-// level, from smem_tail on, whose tail fits in a CTA's shared memory (at least one level
-// above the coarsest)
-static int tail_level(const hp_problem *P, int node_bytes) {
-  if (P->smem_tail) {
-    const size_t cap = (size_t)smem_optin();
-    for (int l0 = std::max(1, P->smem_tail); l0 + 2 <= P->L; ++l0)
-      if (smem_tail_layout<float>(P, l0, node_bytes, nullptr) <= cap) return l0;
+// first level whose cycle runs with one CTA per column: the finest that fits (at most
+// COL_MAXN nodes) and is not asked to run as TMA tiles; L if there is none (and in FP64)
+static int col_level(const hp_problem *P, OpKind op, int tbytes, int vw) {
+  const int L = op == OP_M ? 1 : P->L;
+  if (tbytes != 4) return L;
+  int l = L;
+  while (l > 0 && P->lv[l - 1].g.n <= COL_MAXN && !tiled_level(P, op, l - 1, vw)) {
+    ColArgs a;
+    col_args(P, op, vw, 1, l - 1, &a);
+    if (!col_fits(a, l == 1)) break;
+    --l;
   }
-  return P->L;
+  return l;
+}
+
+// Whether the whole PCG of a column runs in one CTA: wherever its finest level fits.  Measured
+// per iteration on 65^2 nodes: 32 us for any number of columns up to the 152 SMs, against 36
+// launches of 1.6 us or more; one Hessian column with the prior term on 33^2 nodes went from
+// 1.38 to 0.71 ms, a block of 16 samples' solves likewise.
+static bool col_pcg_rule(const hp_problem *P, OpKind op, int tbytes, int vw) {
+  return col_level(P, op, tbytes, vw) == 0;
+}
+
+// First level of the one-launch coarse end of the V-cycle (a level above the coarsest one,
+// whose own solve is a launch either way), or L.  It starts at COL_TAILN nodes: a larger level
+// costs one SM about what its nine launches cost (65^2 nodes: 28 us from there down, against
+// 19 launches of 1.6 us inside a CUDA graph).  The dense coarse solve has to be small too: one
+// SM takes 6.7 us for 17^2 nodes, bound by its reads of the matrix from L2, where the launch
+// over 150 CTAs takes 3 (measured over 33^2 and 17^2 nodes: no gain; over 13^3, 7^3 and 4^3
+// nodes a block of full-Newton actions on 49^3 went from 4.34 to 3.76 ms).
+constexpr long COL_TAILN = 2304, COL_TAILC = 200;
+static int tail_level(const hp_problem *P, OpKind op, int tbytes, int vw) {
+  if (P->lv[P->L - 1].g.n > COL_TAILC) return P->L;
+  int l = std::max(1, col_level(P, op, tbytes, vw));
+  while (l < P->L && P->lv[l].g.n > COL_TAILN) ++l;
+  return l + 1 < P->L ? l : P->L;
 }
 
 // Algorithmic bytes of the V-cycle's levels l0 .. L-1 as the per-level kernels would move
@@ -2075,65 +1869,6 @@ static double tail_bytes(const hp_problem *P, OpKind op, int s, int l0) {
   }
   const double nc = (double)P->lv[P->L - 1].g.n;
   return b + (nc * nc + 2.0 * nc * s) * w;
-}
-
-// The shared-memory tail as its two launches around the dense coarse solve.
-template <typename T, int VW>
-static void launch_vtail_smem(hp_problem *P, OpKind op, int s, int l0, const T *const *rl, T *const *ea,
-                              const long *gsl, T *dst) {
-  const int L = P->L, ng = (s + VW - 1) / VW;
-  VTailS<T> vt{};
-  vt.l0 = l0;
-  vt.L = L;
-  vt.zero_dirichlet = op == OP_K;
-  vt.nc = (int)P->lv[L - 1].g.n;
-  for (int l = 0; l < L; ++l) {
-    vt.nu[l] = nu_at(P, l);
-    smooth_weights<T>(P, op, l, vt.w[l]);
-    const Stencil<T> &S = stencil_of<T>(P, op, l);
-    vt.g[l] = P->lv[l].g;
-    vt.diag[l] = S.diag;
-    vt.invdiag[l] = S.invdiag;
-    vt.c[l] = S.c;
-    vt.rg[l] = const_cast<T *>(rl[l]);
-    vt.ag[l] = ea[l];
-    vt.gs[l] = gsl[l];
-  }
-  vt.r0 = rl[l0];
-  vt.dst = dst;
-  vt.gs0 = gsl[l0];
-  const size_t bytes = smem_tail_layout<T>(P, l0, (int)(sizeof(T) * VW), &vt);
-  const bool full = stencil_of<T>(P, op, l0).full;
-  void (*down)(VTailS<T>) = nullptr, (*up)(VTailS<T>) = nullptr;
-  if (P->lv[0].g.dim == 2) {
-    down = full ? k_vtail_smem<T, VW, 2, true, 0> : k_vtail_smem<T, VW, 2, false, 0>;
-    up = full ? k_vtail_smem<T, VW, 2, true, 1> : k_vtail_smem<T, VW, 2, false, 1>;
-  } else {
-    down = full ? k_vtail_smem<T, VW, 3, true, 0> : k_vtail_smem<T, VW, 3, false, 0>;
-    up = full ? k_vtail_smem<T, VW, 3, true, 1> : k_vtail_smem<T, VW, 3, false, 1>;
-  }
-  // every caller sets the same limit (the device's opt-in maximum less the kernel's static
-  // shared memory), so solves launching from several host threads never lower it under
-  // one another's launch; the launch's own size is the fallback
-  auto allow = [&](void (*k)(VTailS<T>)) {
-    cudaFuncAttributes fa{};
-    int cap = smem_optin();
-    const bool clean = cudaPeekAtLastError() == cudaSuccess;  // an earlier error stays for the caller
-    if (cudaFuncGetAttributes(&fa, k) == cudaSuccess) cap -= (int)fa.sharedSizeBytes;
-    if (cap < (int)bytes || cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, cap) != cudaSuccess) {
-      if (clean) (void)cudaGetLastError();  // a refused limit is not an error of the solve
-      cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes);
-    }
-  };
-  allow(down);
-  allow(up);
-  down<<<dim3(1, ng), VS_NT, bytes, P->st>>>(vt);
-  const int lc = L - 1, nc = (int)P->lv[lc].g.n;
-  k_coarse_apply<T, VW><<<dim3((nc + 31) / 32, ng), 256, sizeof(T) * nc * VW, P->st>>>(
-      coarse_inv<T>(P, op), nc, rl[lc], gsl[lc], ea[lc], gsl[lc]);
-  up<<<dim3(1, ng), VS_NT, bytes, P->st>>>(vt);
-  count_launch(3);
-  count_bytes(BY_STENCILC, tail_bytes<T>(P, op, s, l0));
 }
 
 // Preconditioner z = M^{-1} r with the fused <r, z> -> fin.
@@ -2177,16 +1912,10 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
   }
   T *cur[HP_MAXL], *oth[HP_MAXL];
   const Fin nofin{};
-  const int l0 = tail_level(P, (int)(sizeof(T) * VW));  // levels >= l0 run inside one launch
+  const int l0 = tail_level(P, op, (int)sizeof(T), VW);  // levels >= l0 run inside one launch
   for (int l = 0; l + 1 < L; ++l) {
     const int nu = nu_at(P, l);
-    if (l >= l0) {  // buffer bookkeeping only: the fused kernel makes the same choices
-      T *c = nu >= 2 ? ea[l] : eb[l], *o = nu >= 2 ? eb[l] : ea[l];
-      for (int k = 2; k < nu; ++k) std::swap(c, o);
-      cur[l] = c;
-      oth[l] = o;
-      continue;
-    }
+    if (l >= l0) break;
     const GridDesc &g = P->lv[l].g;
     const Stencil<T> &S = stencil_of<T>(P, op, l);
     T w[4];
@@ -2244,13 +1973,15 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
     oth[l] = o;
   }
   if (l0 < L) {
-    cur[L - 1] = ea[L - 1];
-    for (int l = L - 2; l >= l0; --l) {
-      T *c = cur[l], *o = oth[l];
-      for (int k = 0; k < nu_at(P, l); ++k) std::swap(c, o);
-      cur[l] = c;
+    if constexpr (sizeof(T) == 4) {
+      ColArgs a;
+      col_args(P, op, VW, s, l0, &a);
+      a.r = rl[l0];
+      a.x = cur[l0] = ea[l0];
+      a.gs = gsl[l0];
+      launch_vtail(a, P->dim, stencil_of<T>(P, op, l0).full, s, st);
+      count_bytes(BY_STENCILC, tail_bytes<T>(P, op, s, l0));
     }
-    launch_vtail_smem<T, VW>(P, op, s, l0, rl, ea, gsl, cur[l0]);
   } else {
     const int lc = L - 1;
     const int nc = (int)P->lv[lc].g.n;
@@ -2260,7 +1991,7 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
     count_bytes(BY_STENCILC, (double)sizeof(T) * ((double)nc * nc + 2.0 * nc * s));
     cur[lc] = ea[lc];
   }
-  for (int l = std::min(L, l0) - 2 + (l0 < L ? 1 : 0); l >= 0; --l) {
+  for (int l = l0 < L ? l0 - 1 : L - 2; l >= 0; --l) {
     const GridDesc &g = P->lv[l].g, &gc = P->lv[l + 1].g;
     const Stencil<T> &S = stencil_of<T>(P, op, l);
     const int nu = nu_at(P, l);
@@ -2335,6 +2066,23 @@ static void pcg_init(hp_problem *P, OpKind op, int s, cudaGraphConditionalHandle
   count_launch(2);
 }
 
+// The PCG of every column in one launch (column.cu), the iteration count of the slowest in
+// sc.iter.
+template <int VW> static int pcg_columns(hp_problem *P, OpKind op, int s) {
+  BlockWS<float> &W = P->w32;
+  cudaMemsetAsync(P->sc.iter.p, 0, sizeof(int), P->st);
+  ColArgs a;
+  col_args(P, op, VW, s, 0, &a);
+  a.r = W.r.as<float>();
+  a.x = W.x.as<float>();
+  a.gs = W.ldn * VW;
+  a.tol2col = P->sc.tol2col.as<double>();
+  a.open = tl_open;
+  a.iter = P->sc.iter.as<int>();
+  count_bytes(BY_VECTOR, 8.0 * (double)P->n * s);  // r read, x written: the rest stays on chip
+  return launch_colpcg(a, P->dim, stencil_of<float>(P, op, 0).full, (s + VW - 1) / VW * VW, P->st);
+}
+
 template <typename T, int VW>
 static void pcg_body(hp_problem *P, OpKind op, int s, double tol2, cudaGraphConditionalHandle h, int use_handle,
                      int maxit) {
@@ -2398,8 +2146,21 @@ static cudaError_t capture_leaf(cudaStream_t st, cudaGraphNode_t *leaf) {
 template <typename T, int VW>
 static cudaError_t append_pcg(hp_problem *P, OpKind op, int s, double tol, int maxit, cudaGraph_t g,
                               cudaGraphNode_t dep, cudaGraphNode_t *last) {
+  cudaError_t e;
+  if constexpr (sizeof(T) == 4) {
+    if (col_pcg_rule(P, op, 4, VW)) {
+      e = cudaStreamBeginCaptureToGraph(P->cap, g, dep ? &dep : nullptr, nullptr, dep ? 1 : 0,
+                                        cudaStreamCaptureModeRelaxed);
+      if (e != cudaSuccess) return e;
+      const int rc = pcg_columns<VW>(P, op, s);
+      const cudaError_t el = capture_leaf(P->cap, last);
+      cudaGraph_t gg = g;
+      e = cudaStreamEndCapture(P->cap, &gg);
+      return el != cudaSuccess ? el : e != cudaSuccess ? e : rc ? cudaErrorUnknown : cudaSuccess;
+    }
+  }
   cudaGraphConditionalHandle h;
-  cudaError_t e = cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault);
+  e = cudaGraphConditionalHandleCreate(&h, g, 0, cudaGraphCondAssignDefault);
   if (e != cudaSuccess) return e;
   e = cudaStreamBeginCaptureToGraph(P->cap, g, dep ? &dep : nullptr, nullptr, dep ? 1 : 0,
                                     cudaStreamCaptureModeRelaxed);
@@ -2459,19 +2220,26 @@ static int build_graph(hp_problem *P, OpKind op, int s, double tol, int maxit, P
   });
 }
 
-static int kernels_per_iteration(const hp_problem *P, OpKind op, int node_bytes) {
+// launches of one PCG iteration (0 when the whole PCG is one launch per solve)
+static int kernels_per_iteration(const hp_problem *P, OpKind op, int tbytes, int vw) {
+  if (col_pcg_rule(P, op, tbytes, vw)) return 0;
   if (op == OP_M) return 8;
-  // V-cycle: per non-coarsest level pre (1 + nu - 2), resid, restrict, prolong, nu post; coarse 1
-  // (with the shared-memory tail from tail_level on: down leg, coarse solve, up leg = 3
-  // launches); plus p update, matvec, cg update, condition and three dot finalisations
-  const int tl = tail_level(P, node_bytes);
-  const int separate = std::min(P->L, tl) - 1 + (tl < P->L ? 1 : 0);
+  // V-cycle: per level above the one-launch coarse end (or the dense coarse solve) pre
+  // (1 + nu - 2), resid, restrict, prolong, nu post; then 1; plus p update, matvec, cg
+  // update, condition and three dot finalisations
+  const int separate = std::min(P->L - 1, tail_level(P, op, tbytes, vw));
   int vc = 0;
   for (int l = 0; l < separate; ++l) {
     const int nu = nu_at(P, l);
     vc += (nu >= 2 ? nu - 1 : 1) + nu + (fuse_at(P, l) ? (nu >= 2 ? 1 : 2) : 3);
   }
-  return 7 + vc + 1 + 2 * (P->L == 1) + ((P->smem_tail && tl < P->L) ? 2 : 0);
+  return 7 + vc + 1 + 2 * (P->L == 1);
+}
+
+// launches that start a PCG: the first residual's norm with its finalisation and the loop
+// condition, or the whole PCG in one launch
+static int kernels_per_pcg(const hp_problem *P, OpKind op, int tbytes, int vw) {
+  return col_pcg_rule(P, op, tbytes, vw) ? 1 : 3;
 }
 
 // after a PCG: fails the solve if a tile kernel gave up waiting for its copies
@@ -2504,10 +2272,20 @@ static int pcg(hp_problem *P, OpKind op, int s, double rtol, int maxit, int *its
     HP_CUDA(cudaMemcpyAsync(h_it, P->sc.iter.p, sizeof(int), cudaMemcpyDeviceToHost, st));
     HP_CUDA(cudaMemcpyFromSymbolAsync(h_it + 1, g_tile_timeout, sizeof(int), 0, cudaMemcpyDeviceToHost, st));
     HP_CUDA(cudaStreamSynchronize(st));
-    count_launch((unsigned long long)(*h_it) * kernels_per_iteration(P, op, (int)(sizeof(T) * VW)) + 2);
+    count_launch((unsigned long long)(*h_it) * kernels_per_iteration(P, op, (int)sizeof(T), VW) +
+                 kernels_per_pcg(P, op, (int)sizeof(T), VW));
     *its = *h_it;
     HP_TRY(tile_timeout_check(P, h_it));
     return *h_it >= maxit ? HP_ERR_NOT_CONVERGED : 0;
+  }
+  if constexpr (sizeof(T) == 4) {
+    if (col_pcg_rule(P, op, 4, VW)) {
+      HP_TRY((pcg_columns<VW>(P, op, s)));
+      HP_CUDA(cudaMemcpyAsync(h_it, P->sc.iter.p, sizeof(int), cudaMemcpyDeviceToHost, st));
+      HP_CUDA(cudaStreamSynchronize(st));
+      *its = *h_it;
+      return *h_it >= maxit ? HP_ERR_NOT_CONVERGED : 0;
+    }
   }
   const double tol2 = rtol * rtol;
   pcg_init<T, VW>(P, op, s, 0, 0, maxit);
@@ -2677,10 +2455,10 @@ static int ir_solve_graph(hp_problem *P, OpKind op, const double *B, long ldb, d
   HP_CUDA(cudaStreamSynchronize(st));
   const RefineCtl c = *P->h_rctl;
   HP_TRY(tile_timeout_check(P, h_it));
-  // kernels run: the first check, and per step the scaling, the PCG init (3) and
+  // kernels run: the first check, and per step the scaling, the PCG's start and
   // iterations, the accumulation, the residual with its finalisation and the check
-  count_launch(1ull + 8ull * (unsigned long long)c.outer +
-               (unsigned long long)c.total_its * (unsigned long long)kernels_per_iteration(P, op, (int)(sizeof(T) * VW)));
+  count_launch(1ull + (5ull + kernels_per_pcg(P, op, (int)sizeof(T), VW)) * (unsigned long long)c.outer +
+               (unsigned long long)c.total_its * (unsigned long long)kernels_per_iteration(P, op, (int)sizeof(T), VW));
   if (c.flags & 2) return set_error(HP_ERR_NONFINITE, "non-finite residual in a PDE solve");
   if (stats) {
     stats->iterations += c.total_its;
@@ -2872,10 +2650,10 @@ static int ir_solve_dfp(hp_problem *P, OpKind op, const double *B, long ldb, dou
       HP_CUDA(cudaStreamSynchronize(st));
       const RefineCtl c = *P->h_rctl;
       HP_TRY(tile_timeout_check(P, h_it));
-      // kernels run: the first check and right-hand side, per step the PCG init (3) and
+      // kernels run: the first check and right-hand side, per step the PCG's start and
       // iterations, the update, the residual with its finalisation and the check
-      count_launch(2ull + 7ull * (unsigned long long)c.outer +
-                   (unsigned long long)c.total_its * (unsigned long long)kernels_per_iteration(P, op, (int)(sizeof(T) * VW)));
+      count_launch(2ull + (4ull + kernels_per_pcg(P, op, (int)sizeof(T), VW)) * (unsigned long long)c.outer +
+                   (unsigned long long)c.total_its * (unsigned long long)kernels_per_iteration(P, op, (int)sizeof(T), VW));
       if (c.flags & 2) return set_error(HP_ERR_NONFINITE, "non-finite residual in a PDE solve");
       total_its = c.total_its;
       outer = c.outer;

@@ -151,12 +151,6 @@ static int autotune_on(hp_problem *P, const double *X, int ldx, int nrhs, int re
       t.fuse_transfer = ft;
       if ((rc = consider(t))) return cleanup(rc);
     }
-    for (int st : {0, 1}) {
-      if (st == cur.smem_tail) continue;
-      hp_tuning t = cur;
-      t.smem_tail = st;
-      if ((rc = consider(t))) return cleanup(rc);
-    }
     for (int tt : {0, 1, 2}) {
       if (tt == cur.tma_tiles) continue;
       hp_tuning t = cur;
