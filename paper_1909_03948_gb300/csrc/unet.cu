@@ -23,6 +23,7 @@
 #include <random>
 #include <vector>
 
+#include "dfloat.cuh"
 #include "internal.h"
 #include "tc.cuh"
 
@@ -54,6 +55,7 @@ struct hp_unet {
   float *a[hp::kUL] = {};         // layer outputs (post-ReLU; out: linear)
   float *pl[3] = {};              // pooled inputs of enc2a, enc3a, bota
   float *da = nullptr, *db = nullptr, *dc = nullptr;  // gradient scratch (largest activation)
+  double *gpart = nullptr;        // bias sums [image][channel], then the weight gradients' chunks
   double *lossbuf = nullptr;      // [0, 64): per-sample loss weights; then block partials
   cudaStream_t st = nullptr;
   // 3x3 convolutions on the tensor cores (default) or on the FP32 pipes
@@ -392,12 +394,6 @@ __global__ void k_pack_tc(const __nv_bfloat16 *__restrict__ w16, TcPack P, __nv_
   }
 }
 
-// dz = da * [a > 0] (relu) or da (linear), in place on da
-__global__ void k_relu_back(float *da, const float *__restrict__ a, long cnt) {
-  for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < cnt; i += (long)gridDim.x * blockDim.x)
-    if (a[i] <= 0.f) da[i] = 0.f;
-}
-
 // d_in[n, ci, y, x] = sum_{co, dy, dx} w[co, ci, dy, dx] dz[n, co, y-dy+1, x-dx+1]  (full-resolution input grad)
 __global__ void __launch_bounds__(256) k_conv_bwd_data(const float *__restrict__ dz, const __nv_bfloat16 *__restrict__ w,
                                                        float *__restrict__ din, int ci_n, int co_n, int H, int W,
@@ -450,38 +446,226 @@ __global__ void __launch_bounds__(256) k_conv_bwd_data(const float *__restrict__
   }
 }
 
-// gw[co, ci, dy, dx] = sum_{n, y, x} dz[n, co, y, x] in[n, ci, y+dy-1, x+dx-1];  one block per (co, ci)
-__global__ void __launch_bounds__(256) k_conv_bwd_weight(ConvIn I, const float *__restrict__ dz, float *__restrict__ gw,
-                                                         int co_n, int N, int H, int W, int K) {
-  const int ci_n = I.c1 + I.c2;
-  const int co = blockIdx.x / ci_n, ci = blockIdx.x % ci_n;
-  const int hal = K == 3 ? 1 : 0;
-  float acc[9] = {0, 0, 0, 0, 0, 0, 0, 0, 0};
-  const long HW = (long)H * W;
-  for (long t = threadIdx.x; t < (long)N * HW; t += blockDim.x) {
-    const int n = (int)(t / HW);
-    const int y = (int)((t % HW) / W), x = (int)(t % W);
-    const float g = dz[((long)n * co_n + co) * HW + (long)y * W + x];
-    if (g == 0.f) continue;
-    for (int dy = 0; dy < K; ++dy)
-      for (int dx = 0; dx < K; ++dx) acc[dy * K + dx] += g * read_in(I, n, ci, y + dy - hal, x + dx - hal, H, W);
+// Weight gradient gw[co, ci, dy, dx] = sum_{n, y, x} dz[n, co, y, x] in[n, ci, y + dy - h, x + dx - h]
+// (h = 1 for K = 3, 0 for the 1x1 layer), in two kernels.
+//
+// k_conv_bwd_weight: a block takes GW_C output channels and eight input channels (one per
+// warp) over a chunk of the pixels.  A unit is a strip of sw image columns over GW_ROWS rows;
+// a warp's lanes hold `per` units side by side (so that images narrower than a warp still fill
+// it).  For each set of units the block stages the gradients of its output channels in shared
+// memory, each warp its input channel's pixels with their halo -- every load of a warp in
+// flight at once, the two resident blocks covering each other's loads -- and a lane then
+// marches down its column keeping the K x K input window and the GW_C K^2 sums in registers:
+// K + GW_C shared-memory loads per GW_C K^2 multiply-adds.  A lane sums up to GW_HELD sets in
+// FP32 (288 terms; the previous form up to 324 for the same batch), the lanes are added in
+// FP32 and everything above in FP64.
+// k_conv_bwd_weight_final: adds the chunks (FP64), and the bias gradient's per-image sums.
+//
+// Bound: the FP32 pipes and the issue slots (16 images of 72^2 pixels: 3.4 G multiply-adds).
+// One block per (co, ci), reading nine inputs per pixel with their index divisions, took 7.7
+// ms for that batch's 15 layers and the bias sums 1.3 ms; the marching lanes with plain loads
+// 2.6 ms (each row waited for its loads from L2).
+constexpr int GW_C = 8, GW_ROWS = 18, GW_WARPS = 8;
+constexpr int GW_HELD = 16;  // sets whose FP32 sums a lane carries on
+constexpr int GW_INW = 48;   // floats per staged input row: 32 lanes and the units' halos
+
+struct GwArgs {
+  ConvIn I;
+  const float *dz;
+  int co, N, H, W;
+  int per, sw;           // units per warp, columns per unit
+  int strips, segs;      // units per image row and column
+  int units, sets;       // units in all, sets of `per` units
+  double *part;          // [chunk][co][ci][K^2]
+};
+
+// Sums of NV values over the warp's lanes (NV a power of two up to 32): the value with index
+// lane % NV, by halving the values at each exchange (31 shuffles for 32 values).
+template <int NV> __device__ __forceinline__ float gw_lane_sums(float (&v)[32], int lane) {
+#pragma unroll
+  for (int o = NV / 2; o > 0; o >>= 1) {
+    const bool up = lane & o;
+#pragma unroll
+    for (int i = 0; i < o; ++i) {
+      const float keep = up ? v[i + o] : v[i], send = up ? v[i] : v[i + o];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+    }
   }
-  for (int kk = 0; kk < K * K; ++kk) {
-    const double s = block_sum<256>((double)acc[kk]);
-    if (threadIdx.x == 0) gw[((long)co * ci_n + ci) * K * K + kk] = (float)s;
+  float r = v[0];
+#pragma unroll
+  for (int o = NV; o < 32; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
+  return r;
+}
+
+template <int K, int C>
+__global__ void __launch_bounds__(32 * GW_WARPS, 2) k_conv_bwd_weight(GwArgs a) {
+  constexpr int KK = K * K, h = K / 2, NV = C * KK, NT32 = (NV + 31) / 32, RI = GW_ROWS + 2 * h;
+  __shared__ float gs[C][GW_ROWS][32];
+  extern __shared__ float gw_in[];  // [warp][RI][GW_INW]
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  const int ci_n = a.I.c1 + a.I.c2, cig = (ci_n + GW_WARPS - 1) / GW_WARPS;
+  const int ci = blockIdx.x % cig * GW_WARPS + w, co0 = blockIdx.x / cig * C;
+  const int H = a.H, W = a.W;
+  const long HW = (long)H * W;
+  const bool mine = ci < ci_n, first = ci < a.I.c1;
+  const int sh = first && a.I.up1 ? 1 : 0;  // the input is at half resolution
+  const int Wi = W >> sh, cn = first ? a.I.c1 : a.I.c2, cc = !mine ? 0 : first ? ci : ci - a.I.c1;
+  const long HWi = (long)(H >> sh) * Wi;
+  const float *__restrict__ in = first ? a.I.in1 : (mine ? a.I.in2 : a.I.in1);
+  float *my = gw_in + w * RI * GW_INW;
+  const int sub = lane / a.sw, col = lane - sub * a.sw;
+  double tot[NT32];  // lane t keeps the warp's sums t, t + 32, ...
+#pragma unroll
+  for (int t = 0; t < NT32; ++t) tot[t] = 0.0;
+  float acc[C][KK];
+  auto clear = [&]() {
+#pragma unroll
+    for (int c = 0; c < C; ++c)
+#pragma unroll
+      for (int q = 0; q < KK; ++q) acc[c][q] = 0.f;
+  };
+  auto flush = [&]() {  // the lanes' FP32 sums into tot
+#pragma unroll
+    for (int t = 0; t < NT32; ++t) {
+      constexpr int LAST = NV % 32 ? NV % 32 : 32;
+      float v[32];
+#pragma unroll
+      for (int i = 0; i < 32; ++i) {
+        const int j = t * 32 + i < NV ? t * 32 + i : 0;
+        v[i] = acc[j / KK][j % KK];
+      }
+      tot[t] += (double)(t + 1 < NT32 ? gw_lane_sums<32>(v, lane) : gw_lane_sums<LAST>(v, lane));
+    }
+    clear();
+  };
+  // unit u's image, first column and first row
+  auto where = [&](int u, int &n, int &x0, int &y0) {
+    const int seg = u % a.segs, r = u / a.segs;
+    n = r / a.strips;
+    x0 = (r - n * a.strips) * a.sw;
+    y0 = seg * GW_ROWS;
+  };
+  clear();
+  int held = 0;
+  for (int set = blockIdx.y; set < a.sets; set += gridDim.y) {
+    int n, x0, y0;
+    const int u = min(set * a.per + min(sub, a.per - 1), a.units - 1);
+    where(u, n, x0, y0);
+    const int x = x0 + col;
+    const bool ok = sub < a.per && set * a.per + sub < a.units && x < W;
+    {  // gradients: warp c stages output channel co0 + c (all loads at clamped places)
+      float v[GW_ROWS];
+      if (w < C) {
+        const float *g = a.dz + ((long)n * a.co + co0 + w) * HW + min(x, W - 1);
+#pragma unroll
+        for (int r = 0; r < GW_ROWS; ++r) v[r] = __ldg(g + (long)min(y0 + r, H - 1) * W);
+#pragma unroll
+        for (int r = 0; r < GW_ROWS; ++r) gs[w][r][lane] = ok && y0 + r < H ? v[r] : 0.f;
+      }
+    }
+    if (mine) {  // the warp's input channel: rows y0 - h .., columns x0 - h .. of each unit
+      const float *src = in + ((long)n * cn + cc) * HWi + (min(x, W - 1) >> sh);
+      float v[RI];
+#pragma unroll
+      for (int r = 0; r < RI; ++r) v[r] = __ldg(src + (long)(min(max(y0 + r - h, 0), H - 1) >> sh) * Wi);
+      if (sub < a.per) {
+#pragma unroll
+        for (int r = 0; r < RI; ++r) {
+          const int y = y0 + r - h;
+          my[r * GW_INW + sub * (a.sw + 2 * h) + h + col] = ok && y >= 0 && y < H ? v[r] : 0.f;
+        }
+      }
+      if (h) {  // the halo columns: element t is row t % RI of halo column t / RI
+        for (int t = lane; t < 2 * a.per * RI; t += 32) {
+          const int hc = t / RI, r = t - hc * RI, us = set * a.per + (hc >> 1);
+          int n2, xx, yy;
+          where(min(us, a.units - 1), n2, xx, yy);
+          const int xh = (hc & 1) ? xx + a.sw : xx - 1, y = yy + r - h;
+          const bool in_im = us < a.units && xh >= 0 && xh < W && y >= 0 && y < H;
+          const float t2 = __ldg(in + ((long)n2 * cn + cc) * HWi + (long)(min(max(y, 0), H - 1) >> sh) * Wi +
+                                 (min(max(xh, 0), W - 1) >> sh));
+          my[r * GW_INW + (hc >> 1) * (a.sw + 2) + ((hc & 1) ? a.sw + 1 : 0)] = in_im ? t2 : 0.f;
+        }
+      }
+    }
+    __syncthreads();
+    if (mine) {
+      const float *p = my + min(sub, a.per - 1) * (a.sw + 2 * h) + min(col, a.sw - 1);
+      float win[K][K];
+#pragma unroll
+      for (int d = 0; d + 1 < K; ++d)
+#pragma unroll
+        for (int q = 0; q < K; ++q) win[d][q] = p[d * GW_INW + q];
+#pragma unroll 3
+      for (int r = 0; r < GW_ROWS; ++r) {
+        float gv[C];
+#pragma unroll
+        for (int c = 0; c < C; ++c) gv[c] = gs[c][r][lane];
+#pragma unroll
+        for (int q = 0; q < K; ++q) win[K - 1][q] = p[(r + K - 1) * GW_INW + q];
+#pragma unroll
+        for (int c = 0; c < C; ++c)
+#pragma unroll
+          for (int q = 0; q < KK; ++q) acc[c][q] = fmaf(gv[c], win[q / K][q % K], acc[c][q]);
+#pragma unroll
+        for (int d = 0; d + 1 < K; ++d)
+#pragma unroll
+          for (int q = 0; q < K; ++q) win[d][q] = win[d + 1][q];
+      }
+    }
+    __syncthreads();
+    if (++held == GW_HELD) {
+      flush();
+      held = 0;
+    }
+  }
+  if (held) flush();
+  if (!mine) return;
+#pragma unroll
+  for (int t = 0; t < NT32; ++t) {
+    const int i = t * 32 + lane;
+    if (i < NV) a.part[(((long)blockIdx.y * a.co + co0 + i / KK) * ci_n + ci) * KK + i % KK] = tot[t];
   }
 }
 
-__global__ void __launch_bounds__(256) k_bias_grad(const float *__restrict__ dz, float *__restrict__ gb, int co_n, int N,
-                                                   long HW) {
-  const int co = blockIdx.x;
-  double acc = 0.0;
-  for (long t = threadIdx.x; t < (long)N * HW; t += blockDim.x) {
-    const int n = (int)(t / HW);
-    acc += dz[((long)n * co_n + co) * HW + t % HW];
+// gw[i] = sum over the chunks of part[chunk][i]; gb[c] = sum over the images of bpart[n][c]
+__global__ void __launch_bounds__(256) k_conv_bwd_weight_final(const double *__restrict__ part, int chunks, long cnt,
+                                                               float *__restrict__ gw, const double *__restrict__ bpart,
+                                                               int N, int co, float *__restrict__ gb) {
+  const long i = blockIdx.x * 256L + threadIdx.x;
+  if (i < cnt) {
+    double s = 0.0;
+#pragma unroll 8
+    for (int c = 0; c < chunks; ++c) s += __ldg(part + c * cnt + i);
+    gw[i] = (float)s;
+  } else if (i < cnt + co) {
+    const int c = (int)(i - cnt);
+    double s = 0.0;
+    for (int n = 0; n < N; ++n) s += bpart[(long)n * co + c];
+    gb[c] = (float)s;
   }
-  acc = block_sum<256>(acc);
-  if (threadIdx.x == 0) gb[co] = (float)acc;
+}
+
+// dz = da [a > 0] in place (relu; linear layers keep da) and the sum of each plane (n, c) of
+// dz into bpart[n][c]: one block per plane, the sums in pairs of floats per thread (two_sum)
+// and FP64 across them
+__global__ void __launch_bounds__(256) k_relu_back_bias(float *__restrict__ da, const float *__restrict__ a, int HW,
+                                                        double *__restrict__ bpart) {
+  float *d = da + (long)blockIdx.x * HW;
+  const float *av = a ? a + (long)blockIdx.x * HW : nullptr;
+  float s = 0.f, c = 0.f;
+  for (int i = threadIdx.x; i < HW; i += 256) {
+    float v = d[i];
+    if (av && av[i] <= 0.f) {
+      v = 0.f;
+      d[i] = 0.f;
+    }
+    const dfl t = two_sum(s, v);
+    s = t.hi;
+    c += t.lo;
+  }
+  const double sum = block_sum<256>((double)s + (double)c);
+  if (threadIdx.x == 0) bpart[blockIdx.x] = sum;
 }
 
 __global__ void k_pool(const float *__restrict__ in, float *__restrict__ out, long NC, int H, int W) {
@@ -712,18 +896,60 @@ static void unet_forward(hp_unet *U, int N) {
   count_launch(3);
 }
 
+// columns per unit and units per warp for images of W columns: the split that leaves the
+// fewest lanes idle (72 columns: 3 x 24 of 32 lanes or 9 x 8 of 4 x 8; the halos must fit a
+// staged row), wider units first
+static void gw_units(int W, int *per, int *sw) {
+  double best = 0.0;
+  for (int s = std::min(W, 32); s >= 6 || s == std::min(W, 32); --s) {
+    const int p = std::min(32 / s, GW_INW / (s + 2)), strips = (W + s - 1) / s;
+    const double use = (double)W / (strips * s) * (p * s) / 32.0;
+    if (use > best + 0.02) {
+      best = use;
+      *per = p;
+      *sw = s;
+    }
+  }
+}
+
+// blocks per pixel chunk of a layer's weight gradient
+static int gw_blocks(const ULayer &L) {
+  return (L.ci + GW_WARPS - 1) / GW_WARPS * (L.k == 1 ? L.co : L.co / GW_C);
+}
+
+// pixel chunks: as many as leave the blocks within two rounds of the two per SM, at least one
+// set each
+static int gw_chunks(int blocks, int sets) { return std::max(1, std::min(4 * NSM / blocks, sets)); }
+
 // backward of conv layer li: dz (in place in `d`, N x co x H x W) -> weight / bias grads and input grad d_in
 static void conv_bwd(hp_unet *U, int li, ConvIn I, float *d, const float *a_out, bool relu, float *d_in, int N, int H,
                      int W) {
   const ULayer &L = U->L[li];
-  const long cnt = (long)N * L.co * H * W;
-  if (relu) {
-    k_relu_back<<<gblocks(cnt), 256, 0, U->st>>>(d, a_out, cnt);
-    count_launch();
-  }
-  k_conv_bwd_weight<<<L.co * L.ci, 256, 0, U->st>>>(I, d, U->g + L.woff, L.co, N, H, W, L.k);
-  k_bias_grad<<<L.co, 256, 0, U->st>>>(d, U->g + L.boff, L.co, N, (long)H * W);
-  count_launch(2);
+  double *bpart = U->gpart, *part = U->gpart + (long)U->cap * 128;
+  k_relu_back_bias<<<N * L.co, 256, 0, U->st>>>(d, relu ? a_out : nullptr, H * W, bpart);
+  GwArgs g;
+  g.I = I;
+  g.dz = d;
+  g.co = L.co;
+  g.N = N;
+  g.H = H;
+  g.W = W;
+  gw_units(W, &g.per, &g.sw);
+  g.strips = (W + g.sw - 1) / g.sw;
+  g.segs = (H + GW_ROWS - 1) / GW_ROWS;
+  g.units = N * g.strips * g.segs;
+  g.sets = (g.units + g.per - 1) / g.per;
+  g.part = part;
+  const int blocks = gw_blocks(L);
+  const long cnt = (long)L.co * L.ci * L.k * L.k;
+  const int chunks = gw_chunks(blocks, g.sets);
+  const dim3 gr(blocks, chunks);
+  const size_t shm = sizeof(float) * GW_WARPS * (GW_ROWS + L.k - 1) * GW_INW;
+  if (L.k == 1) k_conv_bwd_weight<1, 1><<<gr, 32 * GW_WARPS, shm, U->st>>>(g);
+  else k_conv_bwd_weight<3, GW_C><<<gr, 32 * GW_WARPS, shm, U->st>>>(g);
+  k_conv_bwd_weight_final<<<(unsigned)((cnt + L.co + 255) / 256), 256, 0, U->st>>>(part, chunks, cnt, U->g + L.woff,
+                                                                                   bpart, N, L.co, U->g + L.boff);
+  count_launch(3);
   if (d_in && use_tc(U, li) && U->tc_bo[li] >= 0) {
     conv_tc(U, ConvIn{d, L.co, 0, nullptr, 0}, L.co, U->wtc + U->tc_bo[li], nullptr, d_in, L.ci, N, H, W, 0);
   } else if (d_in) {
@@ -857,6 +1083,14 @@ int hp_unet_create(int H, int W, int batch_cap, hp_unet **out) {
       cudaMalloc(&U->db, sizeof(float) * big) || cudaMalloc(&U->dc, sizeof(float) * std::max(big, skips)) ||
       cudaMalloc(&U->lossbuf, sizeof(double) * (64 + 4096)))
     return fail("hp_unet_create: buffers");
+  // a layer's chunks never exceed 4 SMs' worth of blocks per pair, so chunks x weights is
+  // bounded for any batch
+  long most = 0;
+  for (int l = 0; l < kUL; ++l) {
+    const ULayer &L = U->L[l];
+    most = std::max(most, (long)gw_chunks(gw_blocks(L), 1 << 28) * L.co * L.ci * L.k * L.k);
+  }
+  if (cudaMalloc(&U->gpart, sizeof(double) * (N * 128 + most))) return fail("hp_unet_create: gradient sums");
   *out = U;
   return HP_OK;
 }
@@ -865,7 +1099,7 @@ void hp_unet_destroy(hp_unet *U) {
   if (!U) return;
   cudaDeviceSynchronize();
   for (void *p : {(void *)U->p32, (void *)U->w16, (void *)U->wtc, (void *)U->g, (void *)U->am, (void *)U->av, (void *)U->x,
-                  (void *)U->aux, (void *)U->da, (void *)U->db, (void *)U->dc, (void *)U->lossbuf})
+                  (void *)U->aux, (void *)U->da, (void *)U->db, (void *)U->dc, (void *)U->lossbuf, (void *)U->gpart})
     if (p) cudaFree(p);
   for (int l = 0; l < kUL; ++l)
     if (U->a[l]) cudaFree(U->a[l]);
