@@ -437,78 +437,167 @@ __global__ void k_dense_inverse(const double *L, int nc, double *inv, float *inv
 
 // FP32 coarse factorisation for the FP32 inner solves (the only consumer of inv32 when the
 // refinement runs in FP32): one CTA, the lower triangle packed in shared memory (row i at
-// offset i (i + 1) / 2), right-looking Cholesky; FP32 runs at 64x the FP64 rate of an SM.
-// L (row-major, lower) goes to Lg for the triangular solves.
-__device__ __forceinline__ int tri_at(int i, int j) { return i * (i + 1) / 2 + j; }
-
-__global__ void __launch_bounds__(1024) k_dense_cholesky32(const double *__restrict__ A, int nc, float *Lg,
-                                                           int *status) {
-  extern __shared__ float tri[];
-  __shared__ int bad;
-  if (threadIdx.x == 0) bad = 0;
-  for (int t = threadIdx.x; t < nc * (nc + 1) / 2; t += blockDim.x) {
-    int i = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
-    while (tri_at(i, 0) > t) --i;
-    while (tri_at(i + 1, 0) <= t) ++i;
-    tri[t] = (float)A[(long)i * nc + (t - tri_at(i, 0))];
-  }
-  __syncthreads();
-  for (int k = 0; k < nc; ++k) {
-    if (threadIdx.x == 0) {
-      const float d = tri[tri_at(k, k)];
-      if (!(d > 0.f) || !isfinite(d)) bad = 1;
-      tri[tri_at(k, k)] = d > 0.f ? sqrtf(d) : 1.f;
-    }
-    __syncthreads();
-    const float dk = tri[tri_at(k, k)];
-    for (int i = k + 1 + threadIdx.x; i < nc; i += blockDim.x) tri[tri_at(i, k)] /= dk;
-    __syncthreads();
-    const int m = nc - k - 1;
-    for (int t = threadIdx.x; t < m * (m + 1) / 2; t += blockDim.x) {  // i >= j > k
-      int a = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
-      while (a * (a + 1) / 2 > t) --a;
-      while ((a + 1) * (a + 2) / 2 <= t) ++a;
-      const int i = k + 1 + a, j = k + 1 + (t - a * (a + 1) / 2);
-      tri[tri_at(i, j)] -= tri[tri_at(i, k)] * tri[tri_at(j, k)];
-    }
-    __syncthreads();
-  }
-  for (int t = threadIdx.x; t < nc * nc; t += blockDim.x) {
-    const int i = t / nc, j = t % nc;
-    Lg[t] = j <= i ? tri[tri_at(i, j)] : 0.f;
-  }
-  if (threadIdx.x == 0) *status = bad;
+// offset i (i + 1) / 2), filled from the stencil.  Cholesky in panels of CH_B columns:
+//   diagonal block: thread (lane i, warp j) holds entry (i, j); one barrier per column;
+//   rows below: a thread per row solves its CH_B entries in registers;
+//   trailing triangle: 4 x 4 tiles per thread against the panel, kept transposed so that a
+//     tile's two operands are one 16-byte load each per column.
+// Every entry takes its updates in ascending column order, then the division or the root, as
+// the unblocked right-looking form does, so the factor has the same bits.  That form was bound
+// by its three barriers and its index arithmetic per column: 1,200 us for 17^2 nodes.
+constexpr int CH_B = 32;
+__host__ __device__ __forceinline__ constexpr int tri_at(int i, int j) { return i * (i + 1) / 2 + j; }
+static size_t chol32_smem(long nc) {  // the triangle and the transposed panel
+  return sizeof(float) * ((size_t)(nc * (nc + 1) / 2 + 3) / 4 * 4 + (size_t)CH_B * ((nc + 3) / 4 * 4));
 }
 
-// Column j of the inverse from L, one warp per column: the forward substitution L y = e_j
-// from row j on (rows above are zero), then L^T x = y, each row's sum split over the 32
-// lanes and reduced; the column is kept in shared memory and written as row j of inv32
-// (the inverse is symmetric).
-__global__ void __launch_bounds__(128) k_dense_inverse32(const float *__restrict__ L, int nc, float *inv32) {
-  extern __shared__ float colbuf[];  // [4 warps][nc]
-  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5;
-  const int j = blockIdx.x * 4 + w;
+template <int D>
+__global__ void __launch_bounds__(1024) k_dense_cholesky32(GridDesc g, const float *__restrict__ diag,
+                                                           const float *__restrict__ c, int nf, bool full,
+                                                           float *__restrict__ Lg, int *status) {
+  extern __shared__ __align__(16) float tri[];
+  __shared__ float colb[2][CH_B];
+  __shared__ int bad;
+  const int nc = (int)g.n, nt = nc * (nc + 1) / 2, tid = threadIdx.x, lane = tid & 31, w = tid >> 5;
+  const int ldp = (nc + 3) / 4 * 4;
+  float *PT = tri + (nt + 3) / 4 * 4;  // PT[k][r]: column k of the panel, rows past the panel
+  if (tid == 0) bad = 0;
+  for (int t = tid; t < nt; t += 1024) tri[t] = 0.f;
+  __syncthreads();
+  for (int i = tid; i < nc; i += 1024) {
+    int v[3];
+    node_coords<D>(g, i, v);
+    tri[tri_at(i, i)] = diag[i];
+    for (int f = 0; f < nf; ++f) {
+      const int b = full ? f + 1 : (1 << f);
+      bool fwd = true;
+      for (int a = 0; a < D; ++a)
+        if ((b >> a) & 1) fwd = fwd && (v[a] < g.N);
+      if (fwd) tri[tri_at(i + (int)mask_offset(g, b), i)] = c[(long)f * nc + i];
+    }
+  }
+  __syncthreads();
+  for (int k0 = 0; k0 < nc; k0 += CH_B) {
+    const int kb = min(CH_B, nc - k0), r0 = k0 + kb, R = nc - r0;
+    // diagonal block
+    const bool held = lane >= w && lane < kb;
+    float a = held ? tri[tri_at(k0 + lane, k0 + w)] : 0.f;
+    for (int k = 0; k < kb; ++k) {
+      if (w == k) {
+        const float d = __shfl_sync(0xffffffffu, a, k);
+        const float dk = d > 0.f ? sqrtf(d) : 1.f;
+        if (lane == k && (!(d > 0.f) || !isfinite(d))) bad = 1;
+        a = lane == k ? dk : a / dk;
+        colb[k & 1][lane] = a;
+      }
+      __syncthreads();
+      if (w > k && lane >= w) a = fmaf(-colb[k & 1][lane], colb[k & 1][w], a);
+    }
+    if (held) tri[tri_at(k0 + lane, k0 + w)] = a;
+    __syncthreads();
+    // rows below
+    if (tid < R) {
+      float v[CH_B];
+      float *row = tri + tri_at(r0 + tid, k0);
+#pragma unroll
+      for (int k = 0; k < CH_B; ++k) v[k] = row[k];  // R > 0: the panel is full
+#pragma unroll
+      for (int k = 0; k < CH_B; ++k) {
+        v[k] = v[k] / tri[tri_at(k0 + k, k0 + k)];
+#pragma unroll
+        for (int m = k + 1; m < CH_B; ++m) v[m] = fmaf(-v[k], tri[tri_at(k0 + m, k0 + k)], v[m]);
+      }
+#pragma unroll
+      for (int k = 0; k < CH_B; ++k) {
+        row[k] = v[k];
+        PT[k * ldp + tid] = v[k];
+      }
+    }
+    __syncthreads();
+    // trailing triangle (rows past R of the panel hold stale values that are never stored)
+    const int nb = (R + 3) / 4;
+    for (int t = tid; t < nb * (nb + 1) / 2; t += 1024) {
+      int ti = (int)((sqrtf(8.f * t + 1.f) - 1.f) * 0.5f);
+      while (ti * (ti + 1) / 2 > t) --ti;
+      while ((ti + 1) * (ti + 2) / 2 <= t) ++ti;
+      const int tj = t - ti * (ti + 1) / 2;
+      float acc[4][4];
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int i = 4 * ti + p, j = 4 * tj + q;
+          acc[p][q] = i < R && j <= i ? tri[tri_at(r0 + i, r0 + j)] : 0.f;
+        }
+#pragma unroll 8
+      for (int k = 0; k < CH_B; ++k) {
+        const float4 x = *reinterpret_cast<const float4 *>(PT + k * ldp + 4 * ti);
+        const float4 y = *reinterpret_cast<const float4 *>(PT + k * ldp + 4 * tj);
+        const float xv[4] = {x.x, x.y, x.z, x.w}, yv[4] = {y.x, y.y, y.z, y.w};
+#pragma unroll
+        for (int p = 0; p < 4; ++p)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) acc[p][q] = fmaf(-xv[p], yv[q], acc[p][q]);
+      }
+#pragma unroll
+      for (int p = 0; p < 4; ++p)
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+          const int i = 4 * ti + p, j = 4 * tj + q;
+          if (i < R && j <= i) tri[tri_at(r0 + i, r0 + j)] = acc[p][q];
+        }
+    }
+    __syncthreads();
+  }
+  for (int t = tid; t < nt; t += 1024) Lg[t] = tri[t];
+  if (tid == 0) *status = bad;
+}
+
+// Column j of the inverse from the packed L, one warp per column: the forward substitution
+// L y = e_j from row j on (rows above are zero), then L^T x = y, each row's sum split over
+// the 32 lanes and reduced.  L is held in shared memory: a row is a chain of loads, lane sums,
+// five shuffles and a division, and with L read from L2 the chains took 500 us.  x goes out
+// as row j of inv32 (the inverse is symmetric) and its entries from j on as column j of tri32.
+constexpr int CI_W = 16;  // columns per CTA
+static size_t inv32_smem(long nc) {
+  return sizeof(float) * ((size_t)(nc * (nc + 1) / 2 + 3) / 4 * 4 + (size_t)CI_W * nc);
+}
+
+__global__ void __launch_bounds__(32 * CI_W) k_dense_inverse32(const float *__restrict__ Lg, int nc,
+                                                               float *__restrict__ inv32, float *__restrict__ tri32) {
+  extern __shared__ __align__(16) float L[];
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nt4 = (nc * (nc + 1) / 2 + 3) / 4;
+  for (int t = threadIdx.x; t < nt4; t += 32 * CI_W)
+    reinterpret_cast<float4 *>(L)[t] = reinterpret_cast<const float4 *>(Lg)[t];
+  __syncthreads();
+  const int j = blockIdx.x * CI_W + w;
   if (j >= nc) return;
-  float *x = colbuf + (long)w * nc;
+  float *x = L + 4 * nt4 + w * nc;
   for (int i = lane; i < nc; i += 32) x[i] = 0.f;
   __syncwarp();
   for (int i = j; i < nc; ++i) {
+    const float *row = L + tri_at(i, 0);
     float sum = 0.f;
-    for (int k = j + lane; k < i; k += 32) sum += L[(long)i * nc + k] * x[k];
+#pragma unroll 3
+    for (int k = j + lane; k < i; k += 32) sum = fmaf(row[k], x[k], sum);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane == 0) x[i] = ((i == j ? 1.f : 0.f) - sum) / L[(long)i * nc + i];
+    if (lane == 0) x[i] = ((i == j ? 1.f : 0.f) - sum) / row[i];
     __syncwarp();
   }
   for (int i = nc - 1; i >= 0; --i) {
     float sum = 0.f;
-    for (int k = i + 1 + lane; k < nc; k += 32) sum += L[(long)k * nc + i] * x[k];
+#pragma unroll 3
+    for (int k = i + 1 + lane; k < nc; k += 32) sum = fmaf(L[tri_at(k, i)], x[k], sum);
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
-    if (lane == 0) x[i] = (x[i] - sum) / L[(long)i * nc + i];
+    if (lane == 0) x[i] = (x[i] - sum) / L[tri_at(i, i)];
     __syncwarp();
   }
-  for (int i = lane; i < nc; i += 32) inv32[(long)j * nc + i] = x[i];
+  for (int i = lane; i < nc; i += 32) {
+    inv32[(long)j * nc + i] = x[i];
+    if (i >= j) tri32[tri_at(i, j)] = x[i];
+  }
 }
 
 // lower triangle of the symmetric FP32 inverse, row i at i (i + 1) / 2 (the one-CTA coarse
@@ -523,36 +612,43 @@ int coarse_setup(hp_problem *P, OpKind op) {
   CoarseInv &C = op == OP_K ? P->cK : P->cA;
   const Stencil<double> &S = op == OP_K ? lc.K64 : lc.A64;
   const long nc = lc.g.n;
-  HP_CUDA(cudaMemsetAsync(C.dense, 0, sizeof(double) * nc * nc, P->st));
-  const int nb = (int)std::min<long>((nc + 255) / 256, 1024);
-  if (P->dim == 2)
-    k_dense_from_stencil<2><<<nb, 256, 0, P->st>>>(lc.g, S.diag, S.c, S.nf, S.full, C.dense);
-  else
-    k_dense_from_stencil<3><<<nb, 256, 0, P->st>>>(lc.g, S.diag, S.c, S.nf, S.full, C.dense);
   int *dstat = P->sc.active.as<int>();
-  const size_t tri_bytes = sizeof(float) * (size_t)nc * (nc + 1) / 2;
-  if (P->precision == HP_FP32_IR && tri_bytes <= 200u * 1024u) {
+  constexpr size_t SMEM32 = 222 * 1024;
+  if (P->precision == HP_FP32_IR && std::max(chol32_smem(nc), inv32_smem(nc)) <= SMEM32) {
     // only inv32 is used by FP32 inner solves: factor and invert in FP32 (inv64 is
     // rebuilt by hp_set_precision if the plain FP64 path is selected later)
     static std::atomic<unsigned long long> attr_set{0};
     int dev = 0;
     HP_CUDA(cudaGetDevice(&dev));
-    if (dev < 64 && !(attr_set.load(std::memory_order_acquire) & (1ull << dev))) {
-      HP_CUDA(cudaFuncSetAttribute(k_dense_cholesky32, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                   200 * 1024));
-      attr_set.fetch_or(1ull << dev, std::memory_order_release);
+    if (dev >= 64 || !(attr_set.load(std::memory_order_acquire) & (1ull << dev))) {
+      for (const void *k : {(const void *)k_dense_cholesky32<2>, (const void *)k_dense_cholesky32<3>,
+                            (const void *)k_dense_inverse32})
+        HP_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)SMEM32));
+      if (dev < 64) attr_set.fetch_or(1ull << dev, std::memory_order_release);
     }
     float *L32 = reinterpret_cast<float *>(C.inv64);  // scratch: the FP64 inverse is not kept in this mode
-    k_dense_cholesky32<<<1, 1024, tri_bytes, P->st>>>(C.dense, (int)nc, L32, dstat);
-    k_dense_inverse32<<<(int)((nc + 3) / 4), 128, sizeof(float) * 4 * nc, P->st>>>(L32, (int)nc, C.inv32);
+    const Stencil<float> &S32 = op == OP_K ? lc.K32 : lc.A32;
+    if (P->dim == 2)
+      k_dense_cholesky32<2><<<1, 1024, chol32_smem(nc), P->st>>>(lc.g, S32.diag, S32.c, S32.nf, S32.full, L32, dstat);
+    else
+      k_dense_cholesky32<3><<<1, 1024, chol32_smem(nc), P->st>>>(lc.g, S32.diag, S32.c, S32.nf, S32.full, L32, dstat);
+    k_dense_inverse32<<<(int)((nc + CI_W - 1) / CI_W), 32 * CI_W, inv32_smem(nc), P->st>>>(L32, (int)nc, C.inv32,
+                                                                                           C.tri32);
     C.fp64_valid = false;
+    count_launch(2);
   } else {
+    HP_CUDA(cudaMemsetAsync(C.dense, 0, sizeof(double) * nc * nc, P->st));
+    const int nb = (int)std::min<long>((nc + 255) / 256, 1024);
+    if (P->dim == 2)
+      k_dense_from_stencil<2><<<nb, 256, 0, P->st>>>(lc.g, S.diag, S.c, S.nf, S.full, C.dense);
+    else
+      k_dense_from_stencil<3><<<nb, 256, 0, P->st>>>(lc.g, S.diag, S.c, S.nf, S.full, C.dense);
     k_dense_cholesky<<<1, 1024, 0, P->st>>>(C.dense, (int)nc, dstat);
     k_dense_inverse<<<(int)((nc + 31) / 32), 32, 0, P->st>>>(C.dense, (int)nc, C.inv64, C.inv32);
+    k_pack_tri<<<(int)nc, 128, 0, P->st>>>(C.inv32, (int)nc, C.tri32);
     C.fp64_valid = true;
+    count_launch(4);
   }
-  k_pack_tri<<<(int)nc, 128, 0, P->st>>>(C.inv32, (int)nc, C.tri32);
-  count_launch(4);
   int h = 0;
   HP_CUDA(cudaMemcpyAsync(&h, dstat, sizeof(int), cudaMemcpyDeviceToHost, P->st));
   HP_CUDA(cudaStreamSynchronize(P->st));
