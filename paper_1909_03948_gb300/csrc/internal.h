@@ -345,6 +345,25 @@ bool col_fits(const ColArgs &a, bool pcg);
 int launch_vtail(ColArgs a, int dim, bool full, int cols, cudaStream_t st);
 int launch_colpcg(ColArgs a, int dim, bool full, int cols, cudaStream_t st);
 
+// ---- legs.cu --------------------------------------------------------------------
+// One leg of a 2D level's part of the V-cycle in one launch (FP32; see legs.cu).
+struct LegArgs {
+  const float *diag, *invdiag, *c;  // the level's stencil
+  float w[4];                        // smoothing weights
+  int nu, zero_dirichlet;
+  const float *r;                    // right-hand side, [group][node][vw], group stride gs
+  const float *xin;                  // up: the smoothed iterate
+  float *x;                          // down: the smoothed iterate; up: the correction
+  float *rc;                         // down: coarse right-hand side (group stride gsc)
+  const float *ec;                   // up: coarse correction
+  long gs, gsc;
+  double *part;                      // up: <r, x> partials [column][tile], or null
+  int np, npc, s, ntx, nty, W, strips, pad, vec;  // set by launch_leg
+};
+constexpr int LEG_MAXNU = 3;       // most sweeps of a leg
+int leg_tiles(const GridDesc &g);  // CTAs per column group (partials per column)
+int launch_leg(LegArgs a, const GridDesc &g, bool full, bool up, int vw, int s, cudaStream_t st);
+
 // ---- dense.cu ---------------------------------------------------------------
 // G (s1 x s2, column-major, ldg) = X^T Y ; X: n x s1, Y: n x s2 (FP64)
 int gram(hp_problem *P, const double *X, long ldx, int s1, const double *Y, long ldy, int s2, double *G,

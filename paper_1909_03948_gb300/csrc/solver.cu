@@ -971,6 +971,25 @@ __global__ void __launch_bounds__(NB) k_dot(long n, long gs, const T *__restrict
   dot_partial<T, VW>(acc, fin.part, grp, s, blockIdx.x, gridDim.x);
 }
 
+// <a, b> per column with the row kernels' grid and sums (k_st's dots): lanes along a row, a
+// thread's FP32 sum over its rows
+template <typename T, int VW>
+__global__ void __launch_bounds__(NB) k_row_dot(GridDesc g, const T *__restrict__ a, const T *__restrict__ b, long gs,
+                                                int s, Fin fin) {
+  using PK = Pack<T, VW>;
+  const int i0 = blockIdx.x * 32 + (threadIdx.x & 31), grp = blockIdx.z;
+  const int nrows = g.dim == 2 ? g.np : g.np * g.np;
+  PK acc = PK::zero();
+  if (i0 < g.np)
+    for (int row = blockIdx.y * (NB / 32) + (threadIdx.x >> 5); row < nrows; row += gridDim.y * (NB / 32)) {
+      const long o = grp * gs + (i0 + (long)g.np * row) * VW;
+      const PK x = PK::ld(a + o), y = PK::ld(b + o);
+#pragma unroll
+      for (int c = 0; c < VW; ++c) acc.v[c] = fmadd(x.v[c], y.v[c], acc.v[c]);
+    }
+  dot_partial<T, VW>(acc, fin.part, grp, s, blockIdx.x + gridDim.x * blockIdx.y, gridDim.x * gridDim.y);
+}
+
 // r_T (grouped) = scale * r64 (column-major); columns >= s and converged ones are 0
 template <typename T, int VW>
 __global__ void __launch_bounds__(NB) k_to_inner(long n, const double *__restrict__ R, long ldr,
@@ -1851,6 +1870,12 @@ static int tail_level(const hp_problem *P, OpKind op, int tbytes, int vw) {
   return l + 1 < P->L ? l : P->L;
 }
 
+// Whether a level's legs run as one launch each (legs.cu): FP32, 2D, up to LEG_MAXNU sweeps
+// (the halo), neither asked to run as TMA tiles nor with the transfers fused the other way.
+static bool leg_level(const hp_problem *P, OpKind op, int l, int tbytes, int vw) {
+  return tbytes == 4 && P->dim == 2 && nu_at(P, l) <= LEG_MAXNU && !fuse_at(P, l) && !tiled_level(P, op, l, vw);
+}
+
 // Algorithmic bytes of the V-cycle's levels l0 .. L-1 as the per-level kernels would move
 // them (smoothing sweeps, residual, restriction, prolongation, the dense coarse solve): the
 // fused tails do the same work in fewer launches, and are counted with these bytes.
@@ -1869,6 +1894,23 @@ static double tail_bytes(const hp_problem *P, OpKind op, int s, int l0) {
   }
   const double nc = (double)P->lv[P->L - 1].g.n;
   return b + (nc * nc + 2.0 * nc * s) * w;
+}
+
+// Whether the finest level's up leg forms the <r, z> partials itself: the FP32 sums of the row
+// kernels run over one row's 32 nodes per thread block while their grid is not capped; where
+// it is, a thread carries its FP32 sum over several rows far apart, and k_row_dot forms the
+// same sums in a pass of its own (a tile does not hold those rows).
+static bool leg_dot(const GridDesc &g, int ng) { return rowgrid_capped(g, ng).y == rowgrid(g, ng).y; }
+
+static LegArgs leg_args(const Stencil<float> &S, const float w[4], int nu, OpKind op) {
+  LegArgs a{};
+  a.diag = S.diag;
+  a.invdiag = S.invdiag;
+  a.c = S.c;
+  for (int k = 0; k < 4; ++k) a.w[k] = w[k];
+  a.nu = nu;
+  a.zero_dirichlet = op == OP_K;
+  return a;
 }
 
 // Preconditioner z = M^{-1} r with the fused <r, z> -> fin.
@@ -1920,6 +1962,20 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
     const Stencil<T> &S = stencil_of<T>(P, op, l);
     T w[4];
     smooth_weights<T>(P, op, l, w);
+    if constexpr (sizeof(T) == 4) {
+      if (leg_level(P, op, l, 4, VW)) {
+        LegArgs a = leg_args(S, w, nu, op);
+        a.r = rl[l];
+        a.gs = gsl[l];
+        a.x = cur[l] = eb[l];
+        oth[l] = ea[l];
+        a.rc = const_cast<T *>(rl[l + 1]);
+        a.gsc = gsl[l + 1];
+        launch_leg(a, g, S.full, false, VW, s, st);
+        count_bytes(level_family(g.n), 4.0 * ((2.0 * s + 2.0 + S.nf) * (double)g.n + (double)s * P->lv[l + 1].g.n));
+        continue;
+      }
+    }
     // Pre-smoothing from zero.  Each later sweep flips buffers (nu - 2 more pre, nu post), so the
     // fused two-sweep kernel writes ea[l] and the single sweep (nu = 1) writes eb[l]: either way the
     // level's final correction lands in ea[l] (z0 at level 0).
@@ -1998,6 +2054,31 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
     T *c = cur[l], *o = oth[l];
     T w[4];
     smooth_weights<T>(P, op, l, w);
+    if constexpr (sizeof(T) == 4) {
+      if (leg_level(P, op, l, 4, VW)) {
+        LegArgs a = leg_args(S, w, nu, op);
+        a.r = rl[l];
+        a.gs = gsl[l];
+        a.xin = c;
+        a.x = cur[l] = o;
+        a.ec = cur[l + 1];
+        a.gsc = gsl[l + 1];
+        const bool own_dot = l == 0 && leg_dot(g, ng);
+        a.part = own_dot ? fin.part : nullptr;
+        launch_leg(a, g, S.full, true, VW, s, st);
+        count_bytes(level_family(g.n), 4.0 * ((3.0 * s + 2.0 + S.nf) * (double)g.n + (double)s * gc.n));
+        if (own_dot) {
+          dot_finalize(fin, leg_tiles(g), s, st);
+        } else if (l == 0) {
+          const dim3 gr = rowgrid_capped(g, ng);
+          k_row_dot<T, VW><<<gr, NB, 0, st>>>(g, rl[0], cur[0], gsl[0], s, fin);
+          count_launch();
+          count_bytes(BY_VECTOR, 8.0 * s * (double)g.n);
+          dot_finalize(fin, gr.x * gr.y, s, st);
+        }
+        continue;
+      }
+    }
     int k0 = 0;
     if (fuse_at(P, l) && nu >= 2) {
       // prolongation and the first post-smoothing sweep in one pass (x + P e_c is not stored)
@@ -2221,7 +2302,7 @@ static int build_graph(hp_problem *P, OpKind op, int s, double tol, int maxit, P
 }
 
 // launches of one PCG iteration (0 when the whole PCG is one launch per solve)
-static int kernels_per_iteration(const hp_problem *P, OpKind op, int tbytes, int vw) {
+static int kernels_per_iteration(const hp_problem *P, OpKind op, int tbytes, int vw, int s) {
   if (col_pcg_rule(P, op, tbytes, vw)) return 0;
   if (op == OP_M) return 8;
   // V-cycle: per level above the one-launch coarse end (or the dense coarse solve) pre
@@ -2231,8 +2312,10 @@ static int kernels_per_iteration(const hp_problem *P, OpKind op, int tbytes, int
   int vc = 0;
   for (int l = 0; l < separate; ++l) {
     const int nu = nu_at(P, l);
-    vc += (nu >= 2 ? nu - 1 : 1) + nu + (fuse_at(P, l) ? (nu >= 2 ? 1 : 2) : 3);
+    if (leg_level(P, op, l, tbytes, vw)) vc += 2;
+    else vc += (nu >= 2 ? nu - 1 : 1) + nu + (fuse_at(P, l) ? (nu >= 2 ? 1 : 2) : 3);
   }
+  if (separate > 0 && leg_level(P, op, 0, tbytes, vw) && !leg_dot(P->lv[0].g, (s + vw - 1) / vw)) vc += 1;
   return 7 + vc + 1 + 2 * (P->L == 1);
 }
 
@@ -2272,7 +2355,7 @@ static int pcg(hp_problem *P, OpKind op, int s, double rtol, int maxit, int *its
     HP_CUDA(cudaMemcpyAsync(h_it, P->sc.iter.p, sizeof(int), cudaMemcpyDeviceToHost, st));
     HP_CUDA(cudaMemcpyFromSymbolAsync(h_it + 1, g_tile_timeout, sizeof(int), 0, cudaMemcpyDeviceToHost, st));
     HP_CUDA(cudaStreamSynchronize(st));
-    count_launch((unsigned long long)(*h_it) * kernels_per_iteration(P, op, (int)sizeof(T), VW) +
+    count_launch((unsigned long long)(*h_it) * kernels_per_iteration(P, op, (int)sizeof(T), VW, s) +
                  kernels_per_pcg(P, op, (int)sizeof(T), VW));
     *its = *h_it;
     HP_TRY(tile_timeout_check(P, h_it));
@@ -2458,7 +2541,7 @@ static int ir_solve_graph(hp_problem *P, OpKind op, const double *B, long ldb, d
   // kernels run: the first check, and per step the scaling, the PCG's start and
   // iterations, the accumulation, the residual with its finalisation and the check
   count_launch(1ull + (5ull + kernels_per_pcg(P, op, (int)sizeof(T), VW)) * (unsigned long long)c.outer +
-               (unsigned long long)c.total_its * (unsigned long long)kernels_per_iteration(P, op, (int)sizeof(T), VW));
+               (unsigned long long)c.total_its * (unsigned long long)kernels_per_iteration(P, op, (int)sizeof(T), VW, s));
   if (c.flags & 2) return set_error(HP_ERR_NONFINITE, "non-finite residual in a PDE solve");
   if (stats) {
     stats->iterations += c.total_its;
@@ -2653,7 +2736,7 @@ static int ir_solve_dfp(hp_problem *P, OpKind op, const double *B, long ldb, dou
       // kernels run: the first check and right-hand side, per step the PCG's start and
       // iterations, the update, the residual with its finalisation and the check
       count_launch(2ull + (4ull + kernels_per_pcg(P, op, (int)sizeof(T), VW)) * (unsigned long long)c.outer +
-                   (unsigned long long)c.total_its * (unsigned long long)kernels_per_iteration(P, op, (int)sizeof(T), VW));
+                   (unsigned long long)c.total_its * (unsigned long long)kernels_per_iteration(P, op, (int)sizeof(T), VW, s));
       if (c.flags & 2) return set_error(HP_ERR_NONFINITE, "non-finite residual in a PDE solve");
       total_its = c.total_its;
       outer = c.outer;
