@@ -1193,7 +1193,7 @@ int hp_laplace_sample(hp_problem *P, const double *m_map, const double *lambda, 
   if (chunk == 0) return HP_OK;
   const long nper = P->nelems * (P->dim + 1);
   double *etag = nullptr;
-  if (!eta) {
+  if (!eta && P->dim == 2) {
     HP_TRY(P->etabuf.ensure(sizeof(double) * (size_t)nper * chunk));
     etag = P->etabuf.as<double>();
   }
@@ -1211,6 +1211,8 @@ int hp_laplace_sample(hp_problem *P, const double *m_map, const double *lambda, 
     const int cs = std::min(chunk, nsamples - c0);
     if (eta) {
       launch_mass_factor(P, eta + (long)ldeta * c0, ldeta, W, ld, cs);
+    } else if (P->dim == 3) {
+      launch_mass_factor_philox3(P, seed, c0, W, ld, cs);
     } else {
       launch_philox_normals(seed, c0, cs, (int)nper, etag, nper, 0, P->st);
       launch_mass_factor(P, etag, nper, W, ld, cs);

@@ -32,6 +32,7 @@
 
 #include "dfloat.cuh"
 #include "internal.h"
+#include "philox.cuh"
 
 namespace hp {
 
@@ -1234,6 +1235,105 @@ void launch_mass_factor(hp_problem *P, const double *eta, long ldeta, double *W,
     k_mass_factor<2><<<grid, NT, 0, P->st>>>(P->lv[0].g, eta, ldeta, W, ldw);
   else
     k_mass_factor<3><<<grid, NT, 0, P->st>>>(P->lv[0].g, eta, ldeta, W, ldw);
+  count_launch();
+}
+
+// W = C_M eta in 3D with eta drawn on the way: column j holds the normals of sample first + j
+// (element e takes the four of call e, as launch_philox_normals lays them out), which never
+// reach memory.  A CTA marches up through a segment of cell layers over a tile of cells, one
+// cell per thread and layer; the nodes of the tile but its first row and column are summed.
+// With w_qk = qa for q = k and qb otherwise, a node's value is
+//   sw (qb sum_e S_e + (qa - qb) sum_e eta_{e,k(e)}),  S_e the sum of the element's four.
+// The normals are floats, so both sums are taken in 64-bit integers of 2^-52 each (|eta| < 6,
+// 96 terms: no overflow): a term is within 2^-53, the additions are exact, no less precise than
+// FP64 sums of such values (half an ulp of a partial sum is 2^-53 to 2^-50), and the FP64 pipe,
+// which bounded the gathering form (96 multiply-adds per node), is left with five operations
+// per node.  64 samples on 64^3 cells: 6.1 ms and 1.6 ms for the normals before; now bound by
+// the generator's own arithmetic.
+constexpr int MF_NT = 256;
+
+__device__ __forceinline__ long long fixed52(float z) {  // z 2^52 rounded, |z| < 8
+  const float a = z * 0x1p27f;
+  const int hi = __float2int_rz(a);
+  const int lo = __float2int_rn((a - (float)hi) * 0x1p25f);
+  return ((long long)hi << 25) + lo;
+}
+
+__global__ void __launch_bounds__(MF_NT) k_mass_factor_philox3(GridDesc g, unsigned long long seed, long long first,
+                                                               double *__restrict__ W, long ldw, int tx, int ty,
+                                                               int nzs) {
+  __shared__ long long sa[8][MF_NT], st[8][MF_NT];  // per corner: sums of S_e and of the corner's own normals
+  const int np = g.np, N = g.N, bw = tx + 1, t = threadIdx.x;
+  const int ntx = (np + tx - 1) / tx;
+  const int bx = blockIdx.x % ntx, by = blockIdx.x / ntx;
+  const int ly = t / bw, lx = t - ly * bw;
+  // this thread's cell column, and the node at the same place
+  const int cx = bx * tx - 1 + lx, cy = by * ty - 1 + ly;
+  const bool cell = ly <= ty && cx >= 0 && cx < N && cy >= 0 && cy < N;
+  const bool node = ly >= 1 && ly <= ty && lx >= 1 && cx < np && cy < np;
+  const int zb = (int)((long)blockIdx.y * np / nzs), ze = (int)((long)(blockIdx.y + 1) * np / nzs);
+  const unsigned long long smp = (unsigned long long)(first + blockIdx.z);
+  const uint2 key = make_uint2((unsigned)seed, (unsigned)(seed >> 32));
+  const double h3 = g.h * g.h * g.h / 6.0;
+  const double sw = sqrt(h3 / 4.0) * 0x1p-52;
+  const double qa = (5.0 + 3.0 * sqrt(5.0)) / 20.0, qb = (5.0 - sqrt(5.0)) / 20.0;
+  const double wa = sw * qb, wt = sw * (qa - qb);
+  double *out = W + ldw * blockIdx.z;
+  long long ua = 0, ut = 0;  // what the layer below contributes to the node
+  for (int cz = zb - 1; cz < ze; ++cz) {
+    long long A[8] = {0, 0, 0, 0, 0, 0, 0, 0}, T[8] = {0, 0, 0, 0, 0, 0, 0, 0};
+    if (cell && cz >= 0 && cz < N) {
+      const unsigned long long e0 = 6ull * (unsigned long long)(cx + (long)N * (cy + (long)N * cz));
+#pragma unroll
+      for (int p = 0; p < 6; ++p) {
+        const unsigned long long e = e0 + p;
+        const uint4 w = philox4x32_10(make_uint4((unsigned)e, (unsigned)(e >> 32), (unsigned)smp, (unsigned)(smp >> 32)),
+                                      key);
+        float z[4];
+        box_muller(w.x, w.y, &z[0], &z[1]);
+        box_muller(w.z, w.w, &z[2], &z[3]);
+        long long f[4], S = 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) S += f[k] = fixed52(z[k]);
+        constexpr int chain[6][4] = {{0, 1, 3, 7}, {0, 1, 5, 7}, {0, 2, 3, 7}, {0, 2, 6, 7}, {0, 4, 5, 7}, {0, 4, 6, 7}};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+          A[chain[p][k]] += S;
+          T[chain[p][k]] += f[k];
+        }
+      }
+    }
+#pragma unroll
+    for (int b = 0; b < 8; ++b) {
+      sa[b][t] = A[b];
+      st[b][t] = T[b];
+    }
+    __syncthreads();
+    if (node) {
+      // the node is corner s of the cell at its place less s
+      long long da = ua, dt = ut;
+      ua = ut = 0;
+#pragma unroll
+      for (int s = 0; s < 4; ++s) {
+        const int q = t - (s & 1) - (s >> 1) * bw;
+        da += sa[s][q];
+        dt += st[s][q];
+        ua += sa[s + 4][q];
+        ut += st[s + 4][q];
+      }
+      if (cz >= zb) out[cx + (long)np * (cy + (long)np * cz)] = fma(wt, (double)dt, wa * (double)da);
+    }
+    __syncthreads();
+  }
+}
+
+void launch_mass_factor_philox3(hp_problem *P, unsigned long long seed, long long first, double *W, long ldw, int s) {
+  const GridDesc &g = P->lv[0].g;
+  // tiles of equal width, as large as 256 cells with their extra row and column allow
+  const int ntx = (g.np + 30) / 31, tx = (g.np + ntx - 1) / ntx;
+  const int tm = MF_NT / (tx + 1) - 1, nty = (g.np + tm - 1) / tm, ty = (g.np + nty - 1) / nty;
+  const int nzs = std::max(1, g.np / 16);
+  k_mass_factor_philox3<<<dim3(ntx * nty, nzs, s), MF_NT, 0, P->st>>>(g, seed, first, W, ldw, tx, ty, nzs);
   count_launch();
 }
 

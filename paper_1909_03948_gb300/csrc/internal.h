@@ -262,6 +262,8 @@ void launch_Ct_apply(hp_problem *P, const double *W, long ldw, double *Y, long l
 void launch_obs_gather(hp_problem *P, const double *X, long ldx, double *Yq, int s);
 void launch_obs_scatter(hp_problem *P, const double *Yq, double *X, long ldx, int s, double scale);
 void launch_mass_factor(hp_problem *P, const double *eta, long ldeta, double *W, long ldw, int s);
+// 3D: C_M eta for the Philox normals of samples first .. first + s - 1 (nothing stored)
+void launch_mass_factor_philox3(hp_problem *P, unsigned long long seed, long long first, double *W, long ldw, int s);
 void launch_zero_dirichlet(hp_problem *P, double *X, long ldx, int s);
 
 // ---- rng.cu ----------------------------------------------------------------
