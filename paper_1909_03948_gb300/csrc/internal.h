@@ -366,6 +366,20 @@ constexpr int LEG_MAXNU = 3;       // most sweeps of a leg
 int leg_tiles(const GridDesc &g);  // CTAs per column group (partials per column)
 int launch_leg(LegArgs a, const GridDesc &g, bool full, bool up, int vw, int s, cudaStream_t st);
 
+// ---- march.cu -------------------------------------------------------------------
+// 3D stencils over all Kuhn edges with constant coefficients (A, M) on grouped FP32 blocks of
+// four columns per group, in one launch; returns the CTAs per group (partials per column).
+enum { MA_APPLY_DOT = 0, MA_RESID = 1, MA_JACOBI = 2, MA_JACOBI_DOT = 3, MA_JAC2 = 4 };
+struct MarchArgs {
+  const float *diag, *invdiag, *c, *X, *B;
+  float *Y;
+  long gx, gb, gy;  // group strides
+  float omega, omega2;
+  double *part;     // dot partials [column][CTA]
+  int np, s, ntx, nty, nzs;  // set by launch_march
+};
+int launch_march(MarchArgs a, const GridDesc &g, int mode, int s, cudaStream_t st);
+
 // ---- dense.cu ---------------------------------------------------------------
 // G (s1 x s2, column-major, ldg) = X^T Y ; X: n x s1, Y: n x s2 (FP64)
 int gram(hp_problem *P, const double *X, long ldx, int s1, const double *Y, long ldy, int s2, double *G,

@@ -37,7 +37,7 @@ void drop_graphs(hp_problem *P);
 
 constexpr int NB = 128;  // threads per block of the node kernels (4 warps)
 
-enum { FIN_STORE = 0, FIN_ALPHA = 1, FIN_RR = 2, FIN_BETA = 3, FIN_INIT = 4 };
+enum { FIN_STORE = 0, FIN_ALPHA = 1, FIN_RR = 2, FIN_BETA = 3, FIN_INIT = 4, FIN_BETA_NEXT = 5 };
 
 struct Fin {
   double *part = nullptr;
@@ -61,6 +61,11 @@ __device__ __forceinline__ void fin_apply(const Fin &f, int j, double s) {
       break;
     case FIN_BETA: {
       const double b = (*f.iter > 0 && f.active[j] && f.rz[j] != 0.0) ? s / f.rz[j] : 0.0;
+      f.beta[j] = b;
+      f.rz[j] = s;
+    } break;
+    case FIN_BETA_NEXT: {  // beta of the iteration that follows (never the first)
+      const double b = (f.active[j] && f.rz[j] != 0.0) ? s / f.rz[j] : 0.0;
       f.beta[j] = b;
       f.rz[j] = s;
     } break;
@@ -150,6 +155,23 @@ __global__ void k_dot_finalize(const double *__restrict__ part, unsigned nblk, F
   for (unsigned b = threadIdx.x; b < nblk; b += NB) sum += part[(long)col * nblk + b];
   sum = block_sum<NB>(sum);
   if (threadIdx.x == 0) fin_apply(fin, col, sum);
+}
+
+// two products at once: fin's partials, then fin2's
+__global__ void k_dot_finalize2(const double *__restrict__ part, const double *__restrict__ part2, unsigned nblk,
+                                Fin fin, Fin fin2) {
+  const int col = blockIdx.x;
+  double sum = 0.0, sum2 = 0.0;
+  for (unsigned b = threadIdx.x; b < nblk; b += NB) {
+    sum += part[(long)col * nblk + b];
+    sum2 += part2[(long)col * nblk + b];
+  }
+  sum = block_sum<NB>(sum);
+  sum2 = block_sum<NB>(sum2);
+  if (threadIdx.x == 0) {
+    fin_apply(fin, col, sum);
+    fin_apply(fin2, col, sum2);
+  }
 }
 
 static void dot_finalize(const Fin &fin, unsigned nblk, int s, cudaStream_t st) {
@@ -894,22 +916,17 @@ __global__ void __launch_bounds__(256) k_coarse_apply(const T *__restrict__ inv,
 // 1-D node kernels: blockIdx.x over nodes (NB each), blockIdx.y = group
 template <typename T, int VW>
 __global__ void __launch_bounds__(NB) k_jacobi0(long n, const T *__restrict__ invdiag, const T *__restrict__ B, long gs,
-                                                T *__restrict__ Y, T omega, int s, Fin fin, int with_dot) {
+                                                T *__restrict__ Y, T omega) {
   using PK = Pack<T, VW>;
   const int grp = blockIdx.y;
-  PK acc = PK::zero();
   for (long i = blockIdx.x * (long)NB + threadIdx.x; i < n; i += (long)gridDim.x * NB) {
     const PK b = PK::ld(B + grp * gs + i * VW);
     const T w = omega * invdiag[i];
     PK z;
 #pragma unroll
-    for (int q = 0; q < VW; ++q) {
-      z.v[q] = w * b.v[q];
-      acc.v[q] = fmadd(b.v[q], z.v[q], acc.v[q]);
-    }
+    for (int q = 0; q < VW; ++q) z.v[q] = w * b.v[q];
     z.st(Y + grp * gs + i * VW);
   }
-  if (with_dot) dot_partial<T, VW>(acc, fin.part, grp, s, blockIdx.x, gridDim.x);
 }
 
 template <typename T, int VW>
@@ -936,6 +953,78 @@ __global__ void __launch_bounds__(NB) k_cg_update(long n, long gs, const T *__re
     rr.st(r + o);
   }
   dot_partial<T, VW>(acc, fin.part, grp, s, blockIdx.x, gridDim.x);
+}
+
+// The diagonally preconditioned PCG (the mass matrix) does not store z = D^-1 r: the update of
+// r forms <r, z> with the next residual beside <r, r>, the update of p forms z again.  A third
+// pass per iteration (38 us of 370 for 65^3 nodes and 120 columns) and two launches less; the
+// products and sums are those of k_jacobi0.
+template <typename T, int VW>
+__global__ void __launch_bounds__(NB) k_cg_update_diag(long n, long gs, const T *__restrict__ p,
+                                                       const T *__restrict__ q, T *__restrict__ x, T *__restrict__ r,
+                                                       const T *__restrict__ invdiag,
+                                                       const double *__restrict__ alpha, int s, double *part,
+                                                       double *part2) {
+  using PK = Pack<T, VW>;
+  const int grp = blockIdx.y;
+  PK acc = PK::zero(), acc2 = PK::zero();
+  T a[VW];
+#pragma unroll
+  for (int c = 0; c < VW; ++c) a[c] = (T)alpha[grp * VW + c];
+  for (long i = blockIdx.x * (long)NB + threadIdx.x; i < n; i += (long)gridDim.x * NB) {
+    const long o = grp * gs + i * VW;
+    const PK pp = PK::ld(p + o), qq = PK::ld(q + o);
+    PK xx = PK::ld(x + o), rr = PK::ld(r + o);
+    const T w = invdiag[i];
+#pragma unroll
+    for (int c = 0; c < VW; ++c) {
+      xx.v[c] += a[c] * pp.v[c];
+      rr.v[c] -= a[c] * qq.v[c];
+      acc.v[c] += rr.v[c] * rr.v[c];
+      acc2.v[c] = fmadd(rr.v[c], mulr(w, rr.v[c]), acc2.v[c]);
+    }
+    xx.st(x + o);
+    rr.st(r + o);
+  }
+  dot_partial<T, VW>(acc, part, grp, s, blockIdx.x, gridDim.x);
+  __syncthreads();
+  dot_partial<T, VW>(acc2, part2, grp, s, blockIdx.x, gridDim.x);
+}
+
+template <typename T, int VW>
+__global__ void __launch_bounds__(NB) k_p_update_diag(long n, long gs, const T *__restrict__ r,
+                                                      const T *__restrict__ invdiag, T *__restrict__ p,
+                                                      const double *__restrict__ beta) {
+  using PK = Pack<T, VW>;
+  const int grp = blockIdx.y;
+  T b[VW];
+#pragma unroll
+  for (int c = 0; c < VW; ++c) b[c] = (T)beta[grp * VW + c];
+  for (long i = blockIdx.x * (long)NB + threadIdx.x; i < n; i += (long)gridDim.x * NB) {
+    const long o = grp * gs + i * VW;
+    const PK rr = PK::ld(r + o);
+    const T w = invdiag[i];
+    PK pp = PK::ld(p + o);
+#pragma unroll
+    for (int c = 0; c < VW; ++c) pp.v[c] = fmadd(b[c], pp.v[c], mulr(w, rr.v[c]));
+    pp.st(p + o);
+  }
+}
+
+// <r, D^-1 r> partials (the first product of that PCG)
+template <typename T, int VW>
+__global__ void __launch_bounds__(NB) k_dot_diag(long n, const T *__restrict__ invdiag, const T *__restrict__ R,
+                                                 long gs, int s, double *part) {
+  using PK = Pack<T, VW>;
+  const int grp = blockIdx.y;
+  PK acc = PK::zero();
+  for (long i = blockIdx.x * (long)NB + threadIdx.x; i < n; i += (long)gridDim.x * NB) {
+    const PK b = PK::ld(R + grp * gs + i * VW);
+    const T w = invdiag[i];
+#pragma unroll
+    for (int q = 0; q < VW; ++q) acc.v[q] = fmadd(b.v[q], mulr(w, b.v[q]), acc.v[q]);
+  }
+  dot_partial<T, VW>(acc, part, grp, s, blockIdx.x, gridDim.x);
 }
 
 template <typename T, int VW>
@@ -1620,6 +1709,13 @@ template <typename T, int MODE> static double st_bytes(const GridDesc &g, const 
   return (double)sizeof(T) * (double)g.n * ((two ? 2.0 : 3.0) * s + (sweep ? 2.0 : 1.0) + S.nf);
 }
 
+// Whether a 3D stencil over all Kuhn edges (only the prior and the mass have them) runs as the
+// z-marching kernel: on levels with at least MARCH_MIN nodes times column groups, where its
+// CTAs fill the GPU.  65^3 nodes, 120 columns: matvec 170 -> 99 us; 64 columns: sweep 97 -> 73,
+// matvec 89 -> 57 us; 33^3 nodes, 64 columns (575,000): sweep 15.7 -> 14.2 us.
+constexpr long MARCH_MIN = 500000;
+static bool march_rule(const GridDesc &g, int ng) { return g.dim == 3 && g.n * ng >= MARCH_MIN; }
+
 template <typename T, int VW, int MODE>
 static void st_launch(const GridDesc &g, const Stencil<T> &S, const T *X, long gx, const T *B, long gb, T *Y, long gy,
                       int s, T omega, const Fin &fin, cudaStream_t st, T omega2 = T(0)) {
@@ -1635,6 +1731,28 @@ static void st_launch(const GridDesc &g, const Stencil<T> &S, const T *X, long g
       return;
   }
   const int ng = (s + VW - 1) / VW;
+  if constexpr (sizeof(T) == 4 && VW == 4 && MODE != M_RESID_DOT && MODE != M_APPLY) {
+    if (S.full && march_rule(g, ng)) {
+      MarchArgs a{};
+      a.diag = S.diag;
+      a.invdiag = S.invdiag;
+      a.c = S.c;
+      a.X = X;
+      a.gx = gx;
+      a.B = B;
+      a.gb = gb;
+      a.Y = Y;
+      a.gy = gy;
+      a.omega = omega;
+      a.omega2 = omega2;
+      a.part = fin.part;
+      constexpr int mode = MODE == M_APPLY_DOT ? MA_APPLY_DOT : MODE == M_RESID ? MA_RESID
+                           : MODE == M_JACOBI ? MA_JACOBI : MODE == M_JACOBI_DOT ? MA_JACOBI_DOT : MA_JAC2;
+      const int nblk = launch_march(a, g, mode, s, st);
+      if (MODE == M_APPLY_DOT || MODE == M_JACOBI_DOT) dot_finalize(fin, nblk, s, st);
+      return;
+    }
+  }
   const dim3 grid = rowgrid_capped(g, ng);
   if (g.dim == 2) {
     if (S.full)
@@ -1711,7 +1829,7 @@ int ensure_scalars(hp_problem *P, int s) {
   long nbmax = blocks_for(P->n, 1);
   for (int l = 0; l < std::max(P->L, 1); ++l) nbmax = std::max(nbmax, rowgrid_blocks(P->lv[l].g));
   nbmax = std::max(nbmax, (P->n + NB - 1) / NB);
-  if (S.scap >= sc && S.partial.bytes >= sizeof(double) * (size_t)nbmax * sc) return 0;
+  if (S.scap >= sc && S.partial.bytes >= sizeof(double) * 2 * (size_t)nbmax * sc) return 0;
   const size_t b = sizeof(double) * sc;
   HP_TRY(S.rz.ensure(b));
   HP_TRY(S.pq.ensure(b));
@@ -1724,7 +1842,7 @@ int ensure_scalars(hp_problem *P, int s) {
   HP_TRY(S.tol2col.ensure(b));
   HP_TRY(S.bbr.ensure(b));
   HP_TRY(S.active.ensure(sizeof(int) * sc));
-  HP_TRY(S.partial.ensure(sizeof(double) * (size_t)nbmax * sc));
+  HP_TRY(S.partial.ensure(sizeof(double) * 2 * (size_t)nbmax * sc));  // two products' partials
   HP_TRY(S.counter.ensure(sizeof(unsigned) * sc));
   HP_TRY(S.iter.ensure(sizeof(int) * 4));
   for (DBuf *d : {&S.rz, &S.pq, &S.rr, &S.bb, &S.alpha, &S.beta, &S.scale, &S.iscale, &S.tol2col, &S.bbr})
@@ -1921,15 +2039,6 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
   const T om = (T)P->omega;
   const int ng = (s + VW - 1) / VW;
   const long gs0 = W.ldn * VW;
-  if (op == OP_M) {  // Jacobi
-    const Stencil<T> &S = stencil_of<T>(P, op, 0);
-    const dim3 gr = nodegrid(P->n, ng);
-    k_jacobi0<T, VW><<<gr, NB, 0, st>>>(P->n, S.invdiag, r0, gs0, z0, T(1), s, fin, 1);
-    count_launch();
-    count_bytes(BY_STENCIL0, (double)sizeof(T) * (double)P->n * (2.0 * s + 1.0));
-    dot_finalize(fin, gr.x, s, st);
-    return;
-  }
   const int L = P->L;
   if (L == 1) {  // the coarse solve is the whole preconditioner; the caller forms <r, z>
     const int nc = (int)P->lv[0].g.n;
@@ -1984,7 +2093,7 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
     if (nu >= 2) {
       st_launch<T, VW, M_JAC2>(g, S, rl[l], gsl[l], nullptr, 0, c, gsl[l], s, w[0], nofin, st, w[1]);
     } else {
-      k_jacobi0<T, VW><<<nodegrid(g.n, ng), NB, 0, st>>>(g.n, S.invdiag, rl[l], gsl[l], c, w[0], s, nofin, 0);
+      k_jacobi0<T, VW><<<nodegrid(g.n, ng), NB, 0, st>>>(g.n, S.invdiag, rl[l], gsl[l], c, w[0]);
       count_launch();
       count_bytes(level_family(g.n), (double)sizeof(T) * (double)g.n * (2.0 * s + 1.0));
     }
@@ -2143,6 +2252,13 @@ static void pcg_init(hp_problem *P, OpKind op, int s, cudaGraphConditionalHandle
   k_dot<T, VW><<<gr, NB, 0, st>>>(P->n, gs, r, r, s, make_fin(P, FIN_INIT));
   dot_finalize(make_fin(P, FIN_INIT), gr.x, s, st);
   count_bytes(BY_VECTOR, (double)sizeof(T) * (double)P->n * s);
+  if (op == OP_M) {  // <r, z> of the first iteration, where beta is 0 (the counter is at 0)
+    const Fin fin = make_fin(P, FIN_BETA);
+    k_dot_diag<T, VW><<<gr, NB, 0, st>>>(P->n, stencil_of<T>(P, op, 0).invdiag, r, gs, s, fin.part);
+    count_launch();
+    count_bytes(BY_VECTOR, (double)sizeof(T) * (double)P->n * (s + 1.0));
+    dot_finalize(fin, gr.x, s, st);
+  }
   k_pcg_cond<<<1, 256, 0, st>>>(P->sc.active.as<int>(), s, P->sc.iter.as<int>(), maxit, 0, h, use_handle);
   count_launch(2);
 }
@@ -2176,10 +2292,27 @@ static void pcg_body(hp_problem *P, OpKind op, int s, double tol2, cudaGraphCond
   T *p = W.p.template as<T>(), *q = W.q.template as<T>();
   const GridDesc &g0 = P->lv[0].g;
   const Stencil<T> &S0 = stencil_of<T>(P, op, 0);
-  int pr = prof_start(P, PROF_VCYCLE);
+  int pr = -1;
+  if (op == OP_M) {
+    k_p_update_diag<T, VW><<<nodegrid(n, ng), NB, 0, st>>>(n, gs, r, S0.invdiag, p, P->sc.beta.as<double>());
+    count_launch();
+    count_bytes(BY_VECTOR, (double)sizeof(T) * (double)n * (3.0 * s + 1.0));
+    st_launch<T, VW, M_APPLY_DOT>(g0, S0, p, gs, nullptr, 0, q, gs, s, T(0), make_fin(P, FIN_ALPHA), st);
+    const dim3 gu = nodegrid(n, ng);
+    const Fin frr = make_fin(P, FIN_RR, tol2), fbeta = make_fin(P, FIN_BETA_NEXT);
+    double *part2 = frr.part + (long)gu.x * round4(s);
+    k_cg_update_diag<T, VW><<<gu, NB, 0, st>>>(n, gs, p, q, x, r, S0.invdiag, P->sc.alpha.as<double>(), s, frr.part,
+                                               part2);
+    k_dot_finalize2<<<s, NB, 0, st>>>(frr.part, part2, gu.x, frr, fbeta);
+    count_bytes(BY_VECTOR, (double)sizeof(T) * (double)n * (6.0 * s + 1.0));
+    k_pcg_cond<<<1, 256, 0, st>>>(P->sc.active.as<int>(), s, P->sc.iter.as<int>(), maxit, 1, h, use_handle);
+    count_launch(3);
+    return;
+  }
+  pr = prof_start(P, PROF_VCYCLE);
   precondition<T, VW>(P, op, s, r, z, make_fin(P, FIN_BETA));
   prof_stop(P, pr);
-  if (op != OP_M && P->L == 1) {
+  if (P->L == 1) {
     const dim3 gr = nodegrid(n, ng);
     k_dot<T, VW><<<gr, NB, 0, st>>>(n, gs, r, z, s, make_fin(P, FIN_BETA));
     count_launch();
@@ -2304,7 +2437,7 @@ static int build_graph(hp_problem *P, OpKind op, int s, double tol, int maxit, P
 // launches of one PCG iteration (0 when the whole PCG is one launch per solve)
 static int kernels_per_iteration(const hp_problem *P, OpKind op, int tbytes, int vw, int s) {
   if (col_pcg_rule(P, op, tbytes, vw)) return 0;
-  if (op == OP_M) return 8;
+  if (op == OP_M) return 6;
   // V-cycle: per level above the one-launch coarse end (or the dense coarse solve) pre
   // (1 + nu - 2), resid, restrict, prolong, nu post; then 1; plus p update, matvec, cg
   // update, condition and three dot finalisations
@@ -2322,7 +2455,7 @@ static int kernels_per_iteration(const hp_problem *P, OpKind op, int tbytes, int
 // launches that start a PCG: the first residual's norm with its finalisation and the loop
 // condition, or the whole PCG in one launch
 static int kernels_per_pcg(const hp_problem *P, OpKind op, int tbytes, int vw) {
-  return col_pcg_rule(P, op, tbytes, vw) ? 1 : 3;
+  return col_pcg_rule(P, op, tbytes, vw) ? 1 : (op == OP_M ? 5 : 3);
 }
 
 // after a PCG: fails the solve if a tile kernel gave up waiting for its copies
