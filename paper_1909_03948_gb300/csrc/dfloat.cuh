@@ -108,6 +108,19 @@ __device__ __forceinline__ double f2d(float x) {
   return __hiloint2double((int)((u & 0x80000000u) | ((e + 896u) << 20) | (m >> 3)), (int)(m << 29));
 }
 
+// double -> float, rounded to nearest even, by bit manipulation (results in the normal float
+// range; anything else through the FP64 conversion)
+__device__ __forceinline__ float d2f(double x) {
+  const unsigned long long u = static_cast<unsigned long long>(__double_as_longlong(x));
+  const int eh = static_cast<int>((u >> 52) & 0x7ffu) - 896;  // float biased exponent
+  if (eh < 1 || eh > 253) return __double2float_rn(x);
+  const unsigned sgn = static_cast<unsigned>(u >> 32) & 0x80000000u;
+  const unsigned m = static_cast<unsigned>((u & 0xFFFFFFFFFFFFFull) >> 29);
+  const unsigned rest = static_cast<unsigned>(u) & 0x1FFFFFFFu;
+  const unsigned up = (rest > 0x10000000u || (rest == 0x10000000u && (m & 1u))) ? 1u : 0u;
+  return __uint_as_float(sgn | (((static_cast<unsigned>(eh) << 23) | m) + up));  // a carry raises the exponent
+}
+
 // double-float -> double: hi and lo widened exactly by bit manipulation, then one FP64
 // addition (the correctly rounded hi + lo)
 __device__ __forceinline__ double df2d(dfl v) { return f2d(v.hi) + f2d(v.lo); }

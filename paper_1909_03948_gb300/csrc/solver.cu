@@ -184,7 +184,7 @@ static void dot_finalize(const Fin &fin, unsigned nblk, int s, cudaStream_t st) 
 // and blocks, column groups over blockIdx.z.  Element (node i, group g) of a
 // block with group stride gs is at base + g*gs + i*VW.
 // ---------------------------------------------------------------------------
-enum { M_APPLY = 0, M_APPLY_DOT = 1, M_RESID = 2, M_JACOBI = 3, M_JACOBI_DOT = 4, M_JAC2 = 5, M_RESID_DOT = 6 };
+enum { M_APPLY = 0, M_APPLY_DOT = 1, M_RESID = 2, M_JACOBI = 3, M_JACOBI_DOT = 4, M_JAC2 = 5 };
 
 template <typename T, int VW, int D, bool FULL, int MODE>
 __global__ void __launch_bounds__(NB) k_st(GridDesc g, const T *__restrict__ diag, const T *__restrict__ invdiag,
@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(NB) k_st(GridDesc g, const T *__restrict__ dia
   const int i0 = blockIdx.x * 32 + lane;
   const int nrows = D == 2 ? g.np : g.np * g.np;
   const int grp = blockIdx.z;
-  constexpr bool DOT = (MODE == M_APPLY_DOT || MODE == M_JACOBI_DOT || MODE == M_RESID_DOT);
+  constexpr bool DOT = (MODE == M_APPLY_DOT || MODE == M_JACOBI_DOT);
   PK acc = PK::zero();
   for (int row = blockIdx.y * (NB / 32) + (threadIdx.x >> 5); row < nrows; row += gridDim.y * (NB / 32)) {
     if (i0 >= g.np) break;
@@ -259,12 +259,9 @@ __global__ void __launch_bounds__(NB) k_st(GridDesc g, const T *__restrict__ dia
           for (int q = 0; q < VW; ++q) acc.v[q] = fmadd(xc.v[q], out.v[q], acc.v[q]);
       } else {
         const PK bb = PK::ld(B + grp * gb + id * VW);
-        if (MODE == M_RESID || MODE == M_RESID_DOT) {
+        if (MODE == M_RESID) {
 #pragma unroll
           for (int q = 0; q < VW; ++q) out.v[q] = bb.v[q] - sx.v[q];
-          if (DOT)
-#pragma unroll
-            for (int q = 0; q < VW; ++q) acc.v[q] = fmadd(out.v[q], out.v[q], acc.v[q]);
         } else {
           const T wi = omega * invdiag[id];
 #pragma unroll
@@ -667,6 +664,86 @@ __global__ void __launch_bounds__(TL3_NT) k_st_tile3(const __grid_constant__ CUt
 // ---------------------------------------------------------------------------
 // grid transfer, coarse solve, vector kernels (grouped layout)
 // ---------------------------------------------------------------------------
+// FP64 stencils of column-major blocks (the refinement's residual and the operator
+// applications), one node per thread over the flattened grid, C64 columns per thread that
+// share the node's coefficients and addresses.  Bound by the FP64 pipe (2 lanes per clock and
+// SM): 15 or 17 operations per node and column over all Kuhn edges in 3D.  The row kernel gives
+// a row of 65 nodes three warps, the third with one lane, and pays for 96.  65^3 nodes, 120
+// columns: A x 1,310 -> 823 us (840 us is the pipe's time without the boundary), its residual
+// 1,545 -> 966; K's residual 829 -> 536.
+constexpr int C64 = 2;
+template <int D, bool FULL, bool RESID>
+__global__ void __launch_bounds__(NB) k_st64(GridDesc g, const double *__restrict__ diag,
+                                             const double *__restrict__ c, const double *__restrict__ X, long ldx,
+                                             const double *__restrict__ B, long ldb, double *__restrict__ Y, long ldy,
+                                             int s, double *part) {
+  constexpr int NF = FULL ? (1 << D) - 1 : D;
+  const int j0 = blockIdx.y * C64;
+  const double *x[C64];
+#pragma unroll
+  for (int q = 0; q < C64; ++q) x[q] = X + ldx * min(j0 + q, s - 1);
+  double acc[C64];
+#pragma unroll
+  for (int q = 0; q < C64; ++q) acc[q] = 0.0;
+  const unsigned np = (unsigned)g.np, n = (unsigned)g.n;
+  for (unsigned i = blockIdx.x * NB + threadIdx.x; i < n; i += gridDim.x * NB) {
+    const unsigned t = div_np(g, i), t2 = D == 2 ? 0u : div_np(g, t);
+    const int v[3] = {(int)(i - t * np), D == 2 ? (int)t : (int)(t - t2 * np), (int)t2};
+    double sx[C64];
+    const double dg = diag[i];
+#pragma unroll
+    for (int q = 0; q < C64; ++q) sx[q] = mulr(dg, x[q][i]);
+#pragma unroll
+    for (int f = 0; f < NF; ++f) {
+      const int b = FULL ? f + 1 : (1 << f);
+      bool fw = true, bw = true;
+#pragma unroll
+      for (int a = 0; a < D; ++a)
+        if ((b >> a) & 1) {
+          fw = fw && (v[a] < g.N);
+          bw = bw && (v[a] > 0);
+        }
+      const unsigned off = (unsigned)mask_offset(g, b);
+      const double *cf = c + (size_t)f * n;
+      if (fw) {
+        const double w = cf[i];
+#pragma unroll
+        for (int q = 0; q < C64; ++q) sx[q] = fmadd(w, x[q][i + off], sx[q]);
+      }
+      if (bw) {
+        const double w = cf[i - off];
+#pragma unroll
+        for (int q = 0; q < C64; ++q) sx[q] = fmadd(w, x[q][i - off], sx[q]);
+      }
+    }
+#pragma unroll
+    for (int q = 0; q < C64; ++q) {
+      if (j0 + q >= s) break;
+      double out = sx[q];
+      if (RESID) {
+        out = addr(B[ldb * (j0 + q) + i], -sx[q]);
+        acc[q] = fmadd(out, out, acc[q]);
+      }
+      Y[ldy * (j0 + q) + i] = out;
+    }
+  }
+  if (RESID) {  // per-column partials [column][block]
+    __shared__ double sh[NB / 32][C64];
+#pragma unroll
+    for (int q = 0; q < C64; ++q) {
+      const double w = warp_sum(acc[q]);
+      if ((threadIdx.x & 31) == 0) sh[threadIdx.x >> 5][q] = w;
+    }
+    __syncthreads();
+    if (threadIdx.x < C64 && j0 + (int)threadIdx.x < s) {
+      double t = 0.0;
+#pragma unroll
+      for (int w = 0; w < NB / 32; ++w) t += sh[w][threadIdx.x];
+      part[(long)(j0 + threadIdx.x) * gridDim.x + blockIdx.x] = t;
+    }
+  }
+}
+
 // Restriction = transpose of the P1 prolongation: r_c(J) = r_f(2J) +
 // 1/2 sum_{b != 0} [r_f(2J + b) + r_f(2J - b)] over the 2^D - 1 Kuhn edge
 // directions b; Dirichlet rows of the zero-BC space are zeroed.
@@ -1060,6 +1137,15 @@ __global__ void __launch_bounds__(NB) k_dot(long n, long gs, const T *__restrict
   dot_partial<T, VW>(acc, fin.part, grp, s, blockIdx.x, gridDim.x);
 }
 
+// Conversions between the inner precision and FP64 without the FP64 pipe, which runs at 1/64
+// of the FP32 rate and bounded the kernels that convert whole blocks (65^3 nodes, 120 columns:
+// x += d 202 -> 143 us, 97 us for its bytes; |r|-scaling 131 -> 104).  Same values.
+template <typename T> __device__ __forceinline__ T from64(double x);
+template <> __device__ __forceinline__ float from64<float>(double x) { return d2f(x); }
+template <> __device__ __forceinline__ double from64<double>(double x) { return x; }
+__device__ __forceinline__ double to64(float x) { return f2d(x); }
+__device__ __forceinline__ double to64(double x) { return x; }
+
 // <a, b> per column with the row kernels' grid and sums (k_st's dots): lanes along a row, a
 // thread's FP32 sum over its rows
 template <typename T, int VW>
@@ -1090,7 +1176,7 @@ __global__ void __launch_bounds__(NB) k_to_inner(long n, const double *__restric
 #pragma unroll
     for (int q = 0; q < VW; ++q) {
       const int col = grp * VW + q;
-      o.v[q] = col < s ? (T)(scale[col] * R[ldr * col + i]) : T(0);
+      o.v[q] = col < s ? from64<T>(scale[col] * R[ldr * col + i]) : T(0);
     }
     o.st(rt + grp * gs + i * VW);
   }
@@ -1112,7 +1198,7 @@ __global__ void __launch_bounds__(NB) k_to_inner_ctl(long n, const double *__res
 #pragma unroll
     for (int q = 0; q < VW; ++q) {
       const int col = grp * VW + q;
-      o.v[q] = col < s ? (T)(scale[col] * src[ldr * col + i]) : T(0);
+      o.v[q] = col < s ? from64<T>(scale[col] * src[ldr * col + i]) : T(0);
     }
     o.st(rt + grp * gs + i * VW);
   }
@@ -1186,7 +1272,7 @@ __global__ void __launch_bounds__(NB) k_accum(long n, const T *__restrict__ d, l
       const int col = grp * VW + q;
       if (col < s) {
         const double is = iscale[col];  // |r| of the column, 0 when it has converged
-        if (is != 0.0) X[ldx * col + i] += (double)v.v[q] * is;
+        if (is != 0.0) X[ldx * col + i] = fma(to64(v.v[q]), is, X[ldx * col + i]);
       }
     }
   }
@@ -1719,8 +1805,8 @@ static bool march_rule(const GridDesc &g, int ng) { return g.dim == 3 && g.n * n
 template <typename T, int VW, int MODE>
 static void st_launch(const GridDesc &g, const Stencil<T> &S, const T *X, long gx, const T *B, long gb, T *Y, long gy,
                       int s, T omega, const Fin &fin, cudaStream_t st, T omega2 = T(0)) {
-  count_bytes(sizeof(T) == 8 && MODE == M_RESID_DOT ? BY_REFINE : level_family(g.n), st_bytes<T, MODE>(g, S, s));
-  if constexpr (sizeof(T) == 4 && VW == 4 && MODE != M_RESID_DOT) {
+  count_bytes(level_family(g.n), st_bytes<T, MODE>(g, S, s));
+  if constexpr (sizeof(T) == 4 && VW == 4) {
     // tma_tiles 1: every eligible level; 2: the finest level only
     const bool tma = tl_tma == 1 || (tl_tma == 2 && g.n == tl_n0);
     if (tma && S.pk && !S.full && tile_grid(g) &&
@@ -1731,7 +1817,7 @@ static void st_launch(const GridDesc &g, const Stencil<T> &S, const T *X, long g
       return;
   }
   const int ng = (s + VW - 1) / VW;
-  if constexpr (sizeof(T) == 4 && VW == 4 && MODE != M_RESID_DOT && MODE != M_APPLY) {
+  if constexpr (sizeof(T) == 4 && VW == 4 && MODE != M_APPLY) {
     if (S.full && march_rule(g, ng)) {
       MarchArgs a{};
       a.diag = S.diag;
@@ -1770,7 +1856,7 @@ static void st_launch(const GridDesc &g, const Stencil<T> &S, const T *X, long g
                                                      omega2, fin);
   }
   count_launch();
-  if (MODE == M_APPLY_DOT || MODE == M_JACOBI_DOT || MODE == M_RESID_DOT) dot_finalize(fin, grid.x * grid.y, s, st);
+  if (MODE == M_APPLY_DOT || MODE == M_JACOBI_DOT) dot_finalize(fin, grid.x * grid.y, s, st);
 }
 
 template <typename T>
@@ -2527,9 +2613,31 @@ static int pcg(hp_problem *P, OpKind op, int s, double rtol, int maxit, int *its
   return *h_it >= maxit ? HP_ERR_NOT_CONVERGED : 0;
 }
 
+// Y = S X, or (RESID) Y = B - S X with the columns' |Y|^2 partials; returns the blocks per column
+template <bool RESID>
+static unsigned launch_st64(hp_problem *P, OpKind op, const double *X, long ldx, const double *B, long ldb, double *Y,
+                            long ldy, int s, double *part) {
+  const GridDesc &g = P->lv[0].g;
+  const Stencil<double> &S = stencil_of<double>(P, op, 0);
+  const int ng = (s + C64 - 1) / C64;
+  // about four rounds of the resident blocks, so that their last round costs little
+  const long cap = std::max<long>(1, 64l * NSM / ng);
+  const dim3 gr((unsigned)std::min<long>((g.n + NB - 1) / NB, cap), ng);
+  auto go = [&](auto k) { k<<<gr, NB, 0, P->st>>>(g, S.diag, S.c, X, ldx, B, ldb, Y, ldy, s, part); };
+  if (g.dim == 2) {
+    if (S.full) go(k_st64<2, true, RESID>);
+    else go(k_st64<2, false, RESID>);
+  } else {
+    if (S.full) go(k_st64<3, true, RESID>);
+    else go(k_st64<3, false, RESID>);
+  }
+  count_launch();
+  return gr.x;
+}
+
 int apply_op64(hp_problem *P, OpKind op, const double *X, long ldx, double *Y, long ldy, int s) {
-  st_launch<double, 1, M_APPLY>(P->lv[0].g, stencil_of<double>(P, op, 0), X, ldx, nullptr, 0, Y, ldy, s, 0.0, Fin{},
-                                P->st);
+  launch_st64<false>(P, op, X, ldx, nullptr, 0, Y, ldy, s, nullptr);
+  count_bytes(level_family(P->n), st_bytes<double, M_APPLY>(P->lv[0].g, stencil_of<double>(P, op, 0), s));
   return cuda_check(cudaGetLastError(), "apply");
 }
 
@@ -2555,8 +2663,10 @@ static bool use_df(const hp_problem *P, int tbytes, double rtol, int s) {
 static int residual64(hp_problem *P, OpKind op, const double *B, long ldb, const double *X, long ldx, double *R,
                       long ldr, int s) {
   const int pr = prof_start(P, PROF_RESID64);
-  st_launch<double, 1, M_RESID_DOT>(P->lv[0].g, stencil_of<double>(P, op, 0), X, ldx, B, ldb, R, ldr, s, 0.0,
-                                    make_fin(P, FIN_STORE, 0.0, P->sc.rr.as<double>()), P->st);
+  const Fin fin = make_fin(P, FIN_STORE, 0.0, P->sc.rr.as<double>());
+  const unsigned nblk = launch_st64<true>(P, op, X, ldx, B, ldb, R, ldr, s, fin.part);
+  count_bytes(BY_REFINE, st_bytes<double, M_RESID>(P->lv[0].g, stencil_of<double>(P, op, 0), s));
+  dot_finalize(fin, nblk, s, P->st);
   prof_stop(P, pr);
   return cuda_check(cudaGetLastError(), "residual");
 }
