@@ -234,18 +234,29 @@ __global__ void k_gemm_nn_df(const double *__restrict__ X, long ldx, int s1, con
   }
 }
 
-// R^{-1} of an upper-triangular R (column-major, s x s) in FP64, one thread per column:
-// back substitution of R x = e_j (the upper triangle of the result; zeros below)
-__global__ void k_tri_inv(const double *__restrict__ R, int s, double *__restrict__ Ri) {
-  for (int j = threadIdx.x; j < s; j += blockDim.x) {
-    for (int i = s - 1; i > j; --i) Ri[i + (long)s * j] = 0.0;
-    Ri[j + (long)s * j] = 1.0 / R[j + (long)s * j];
-    for (int i = j - 1; i >= 0; --i) {
-      double t = 0.0;
-      for (int k = i + 1; k <= j; ++k) t = fma(R[i + (long)s * k], Ri[k + (long)s * j], t);
-      Ri[i + (long)s * j] = -t / R[i + (long)s * i];
-    }
+// R^{-1} of an upper-triangular R (column-major, s x s) in FP64, one warp per column: back
+// substitution of R x = e_j (the upper triangle of the result; zeros below), a row's sum split
+// over the lanes.  One thread per column took 120 us for s = 60, chains of loads and FP64
+// operations with a latency of tens of clocks each; this takes 35.
+__global__ void __launch_bounds__(128) k_tri_inv(const double *__restrict__ R, int s, double *__restrict__ Ri) {
+  extern __shared__ double ti_x[];  // [4 warps][2][s]: the column, and the inverse diagonal
+  const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, j = blockIdx.x * 4 + w;
+  double *x = ti_x + (long)w * 2 * s, *rd = x + s;
+  if (j >= s) return;
+  for (int i = lane; i <= j; i += 32) rd[i] = 1.0 / R[i + (long)s * i];
+  for (int i = j + 1 + lane; i < s; i += 32) Ri[i + (long)s * j] = 0.0;
+  __syncwarp();
+  if (lane == 0) x[j] = rd[j];
+  __syncwarp();
+  for (int i = j - 1; i >= 0; --i) {
+    double t = 0.0;
+    for (int k = i + 1 + lane; k <= j; k += 32) t = fma(R[i + (long)s * k], x[k], t);
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+    if (lane == 0) x[i] = -t * rd[i];
+    __syncwarp();
   }
+  for (int i = lane; i <= j; i += 32) Ri[i + (long)s * j] = x[i];
 }
 
 void launch_gemm_nn(const double *X, long ldx, int s1, const double *S, int lds, int s2, double *Y, long ldy, long n,
@@ -361,9 +372,71 @@ __global__ void k_small_chol(double *A, int s, int *status) {
   if (threadIdx.x == 0) *status = bad;
 }
 
+// The same for s up to CH_SM with the triangle in shared memory, as L D L^T: a step scales the
+// pivot's column by 1 / d and updates the rows below, a warp per row; the thread that finishes
+// the next pivot forms its reciprocal while the others update, and the roots are taken at the
+// end, for all columns at once.  Bound by the latency of the s reciprocals and the FP64 pipe
+// (s = 60: 94 -> 59 us).
+constexpr int CH_SM = 144;
+constexpr int CH_NT = 512;
+static size_t chol_smem(int s) { return sizeof(double) * ((size_t)s * (s + 1) + 2 * s); }
+
+__global__ void __launch_bounds__(CH_NT) k_small_chol_sm(double *A, int s, int *status) {
+  extern __shared__ double ch[];  // rows of s + 1 doubles; the scaled column; the reciprocals
+  const int ld = s + 1, lane = threadIdx.x & 31, w = threadIdx.x >> 5;
+  double *wk = ch + s * ld, *rd = wk + s;
+  __shared__ int bad;
+  for (int t = threadIdx.x; t < s * s; t += CH_NT) {
+    const int i = t / s, j = t - i * s;
+    if (j <= i) ch[i * ld + j] = A[t];
+  }
+  if (threadIdx.x == 0) bad = 0;
+  __syncthreads();
+  auto pivot = [&](int k) {
+    const double d = ch[k * ld + k];
+    if (!(d > 0.0) || !isfinite(d)) bad = 1;
+    rd[k] = d > 0.0 ? 1.0 / d : 1.0;
+  };
+  if (threadIdx.x == 0) pivot(0);
+  __syncthreads();
+  for (int k = 0; k + 1 < s; ++k) {
+    const double r = rd[k];
+    for (int i = k + 1 + threadIdx.x; i < s; i += CH_NT) wk[i] = ch[i * ld + k] * r;
+    __syncthreads();
+    for (int i = k + 1 + w; i < s; i += CH_NT / 32) {
+      const double li = wk[i];
+      for (int j = k + 1 + lane; j <= i; j += 32) ch[i * ld + j] = fma(-li, ch[j * ld + k], ch[i * ld + j]);
+      if (i == k + 1 && lane == 0) pivot(i);
+    }
+    __syncthreads();
+  }
+  for (int k = threadIdx.x; k < s; k += CH_NT) {
+    const double d = ch[k * ld + k], q = d > 0.0 ? sqrt(d) : 1.0;
+    wk[k] = q;
+    rd[k] = 1.0 / q;
+  }
+  __syncthreads();
+  for (int t = threadIdx.x; t < s * s; t += CH_NT) {
+    const int i = t / s, j = t - i * s;
+    A[t] = j < i ? ch[i * ld + j] * rd[j] : (j == i ? wk[i] : 0.0);
+  }
+  if (threadIdx.x == 0) *status = bad;
+}
+
 int small_cholesky(hp_problem *P, double *G, int s) {
   int *d = P->sc.active.as<int>();
-  k_small_chol<<<1, 1024, 0, P->st>>>(G, s, d);
+  if (s <= CH_SM) {
+    static std::atomic<unsigned long long> attr_ch{0};  // once per device: the largest size
+    int dev = 0;
+    HP_CUDA(cudaGetDevice(&dev));
+    if (dev < 64 && !(attr_ch.load(std::memory_order_acquire) & (1ull << dev))) {
+      HP_CUDA(cudaFuncSetAttribute(k_small_chol_sm, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                   (int)chol_smem(CH_SM)));
+      attr_ch.fetch_or(1ull << dev, std::memory_order_release);
+    }
+    k_small_chol_sm<<<1, CH_NT, chol_smem(s), P->st>>>(G, s, d);
+  } else
+    k_small_chol<<<1, 1024, 0, P->st>>>(G, s, d);
   count_launch();
   int h = 0;
   HP_CUDA(cudaMemcpyAsync(&h, d, sizeof(int), cudaMemcpyDeviceToHost, P->st));
@@ -389,10 +462,10 @@ void launch_trsm_right_upper(double *Y, long ldy, long n, int s, const double *R
   // rounding is about cond(R) 2^-48 relative; the QR passes that use it are self-correcting
   // and the eigensolver's R-orthonormality is checked to 1e-7.
   const long ldt = (n + 63) / 64 * 64;
-  if (P->refine_df != 0 && s > 1 && sizeof(float2) * (size_t)s * GM_NJ <= 48 * 1024 &&
+  if (P->refine_df != 0 && s > 1 && sizeof(double) * (size_t)s * GM_NJ <= 48 * 1024 &&
       P->vtmp[3].ensure(sizeof(double) * (size_t)s * s) == 0 && P->dense_tmp.ensure(sizeof(double) * ldt * s) == 0) {
     double *Ri = P->vtmp[3].as<double>(), *T = P->dense_tmp.as<double>();
-    k_tri_inv<<<1, 128, 0, P->st>>>(R, s, Ri);
+    k_tri_inv<<<(s + 3) / 4, 128, sizeof(double) * 8 * s, P->st>>>(R, s, Ri);
     count_launch();
     launch_gemm_nn(Y, ldy, s, Ri, s, s, T, ldt, n, 1.0, 0.0, P);
     cudaMemcpy2DAsync(Y, sizeof(double) * ldy, T, sizeof(double) * ldt, sizeof(double) * n, s,
@@ -635,9 +708,13 @@ __global__ void __launch_bounds__(1024) k_jacobi_eig_sm(const double *__restrict
 
 // The same cyclic Jacobi with its rotations applied in double-float on the FP32 pipe: A
 // (and V while it fits) held as float pairs in shared memory, V in the global scratch Vg
-// beyond that.  Each rotation's angle is computed in FP64 from the three entries it needs
-// (joined from their pairs), its cosine and sine split into pairs, and every update
-// x' = c x - s y, y' = s x + c y is a compensated (Dot2) two-term sum.  The off-diagonal
+// beyond that.  Each rotation's angle comes from the three entries it needs (rot_angle), its
+// cosine and sine as pairs, and every update
+// x' = c x - s y, y' = s x + c y is a compensated (Dot2) two-term sum.  A round's rotations
+// are applied block by block: for two of its pairs a thread takes the 2 x 2 entries from
+// both sides and writes them with their mirror image, so a round is half the work of
+// a pass over the rows and one over the columns, and one barrier less (s = 60: 3.7 -> 2.5 ms,
+// 2.6 us a round; bound by the rounds' serial chain of angles, barriers and updates on one SM).  The off-diagonal
 // test uses the leading floats' squares, in FP64.
 __device__ __forceinline__ dfl rot_mix(dfl a, dfl x, dfl b, dfl y) {  // a x + b y
   Dot2 d;
@@ -646,28 +723,62 @@ __device__ __forceinline__ dfl rot_mix(dfl a, dfl x, dfl b, dfl y) {  // a x + b
   return d.result();
 }
 
+// Cosine and sine (as pairs) of a rotation that takes apq to (nearly) zero: the tangent
+// t = sign(theta) / (|theta| + sqrt(theta^2 + 1)), theta = (aqq - app) / (2 apq), is a float, and
+// c = 1 / sqrt(1 + t^2) and s = t c follow from that float in double-float, so the rotation is
+// orthogonal to about 2^-46 whatever t's rounding; an entry left at 2^-24 of its size instead
+// of 0 does not slow the sweeps down.  c: a float reciprocal root and one third-order step on its
+// residual 1 - (1 + t^2) y^2.  In FP64 its divisions and roots took a third of the solver's
+// time (s = 60: 5.4 -> 3.7 ms), and c and s rounded to pairs one by one left the eigenvectors 1e-12 off
+// orthogonal, now 2e-13.
+__device__ __forceinline__ void rot_angle(dfl app, dfl aqq, dfl apq, dfl *c, dfl *s) {
+  const dfl d = two_sum(aqq.hi, -app.hi);
+  const float diff = d.hi + (d.lo + (aqq.lo - app.lo));
+  const float theta = diff / (2.f * apq.hi);
+  const float t = copysignf(1.f, theta) / (fabsf(theta) + sqrtf(fmaf(theta, theta, 1.f)));
+  const dfl tt = two_prod(t, t);
+  dfl u = two_sum(1.f, tt.hi);
+  u.lo += tt.lo;
+  const float y = rsqrtf(u.hi);
+  const dfl yy = two_prod(y, y), w = two_prod(u.hi, yy.hi);
+  const float r = (1.f - w.hi) - (w.lo + fmaf(u.hi, yy.lo, u.lo * yy.hi));
+  *c = fast_two_sum(y, y * r * fmaf(0.375f, r, 0.5f));
+  const dfl p = two_prod(t, c->hi);
+  *s = fast_two_sum(p.hi, fmaf(t, c->lo, p.lo));
+}
+
 __global__ void __launch_bounds__(1024) k_jacobi_eig_sm_df(const double *__restrict__ Ain, int s, int m,
                                                            double *lam_out, double *S_out, int max_sweeps,
                                                            float2 *Vg) {
   extern __shared__ float2 shp[];
-  // A (and V while it fits) with leading dimension la = s + 1: a rotation's row pass reads
-  // A[p + la col] for consecutive col, which a stride of s would put in two banks only
-  const int la = s + 1;
-  float2 *A = shp, *V = Vg ? Vg : A + la * s;
+  // A (zero in the extra row and column of an odd s) and V while it fits, with an odd leading
+  // dimension la: neighbouring lanes' columns then lie in different banks
+  const int la = m + 1, h = m / 2;
+  float2 *A = shp, *V = Vg ? Vg : A + la * m;
   const int lv = Vg ? s : la;
-  float2 *csp = A + la * s + (Vg ? 0 : la * s), *snp = csp + m / 2;
+  float2 *csp = A + la * m + (Vg ? 0 : la * m), *snp = csp + h;
   double *red = reinterpret_cast<double *>(snp + m / 2);  // [2][32]
   int *pp = reinterpret_cast<int *>(red + 64);
   int *qq = pp + (m > s ? m : s);
-  for (int t = threadIdx.x; t < s * s; t += blockDim.x) {
-    const int row = t % s, col = t / s;
-    const dfl a = d2df(Ain[t]);
+  for (int t = threadIdx.x; t < m * m; t += blockDim.x) {
+    const int row = t % m, col = t / m;
+    const bool in = row < s && col < s;
+    const dfl a = d2df(in ? 0.5 * (Ain[row + s * col] + Ain[col + s * row]) : 0.0);
     A[row + la * col] = make_float2(a.hi, a.lo);
-    V[row + lv * col] = make_float2(row == col ? 1.f : 0.f, 0.f);
+    if (in) V[row + lv * col] = make_float2(row == col ? 1.f : 0.f, 0.f);
   }
   __syncthreads();
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = blockDim.x >> 5;
   auto J = [](float2 v) { return df2d(dfl{v.x, v.y}); };
+  auto rot = [](dfl c, dfl sn, dfl &x, dfl &y) {  // x' = c x - s y, y' = s x + c y
+    const dfl a = rot_mix(c, x, dfl{-sn.hi, -sn.lo}, y);
+    y = rot_mix(sn, x, c, y);
+    x = a;
+  };
+  // blocks (a, b), a <= b, of the round's pairs, numbered over a rectangle of nbc columns, and
+  // items of up to four rows of V per pair
+  const unsigned nbc = (h & 1) ? h : h + 1, nblk = h * (h + 1) / 2, nr4 = (s + 3) / 4;
+  const unsigned mbc = 0xFFFFFFFFu / nbc + 1, mr4 = 0xFFFFFFFFu / nr4 + 1;  // t / d for t < 2^16, d > 1
   double off_prev = 0.0;
   for (int sweep = 0; sweep < max_sweeps; ++sweep) {
     double off = 0.0, tot = 0.0;
@@ -704,64 +815,69 @@ __global__ void __launch_bounds__(1024) k_jacobi_eig_sm_df(const double *__restr
     if (off_s <= 1e-26 * tot_s || off_s == 0.0 || (sweep >= 3 && off_s > 0.5 * off_prev)) break;
     off_prev = off_s;
     for (int r = 0; r < m - 1; ++r) {
-      for (int k = threadIdx.x; k < m / 2; k += blockDim.x) {
-        int p, q;
-        if (k == 0) {
-          p = r;
-          q = m - 1;
-        } else {
-          p = (r + k) % (m - 1);
-          q = (r - k + (m - 1)) % (m - 1);
-        }
+      for (int k = threadIdx.x; k < h; k += blockDim.x) {
+        int p = k == 0 ? r : (r + k < m - 1 ? r + k : r + k - (m - 1));
+        int q = k == 0 ? m - 1 : (r >= k ? r - k : r - k + m - 1);
         if (p > q) {
           const int t = p;
           p = q;
           q = t;
         }
-        double c = 1.0, sv = 0.0;
-        if (q < s) {
-          const double apq = J(A[p + la * q]);
-          if (apq != 0.0) {
-            const double theta = (J(A[q + la * q]) - J(A[p + la * p])) / (2.0 * apq);
-            const double t = (theta >= 0 ? 1.0 : -1.0) / (fabs(theta) + sqrt(theta * theta + 1.0));
-            c = 1.0 / sqrt(t * t + 1.0);
-            sv = t * c;
-          }
-        }
-        const dfl cd = d2df(c), sd = d2df(sv);
+        dfl cd{1.f, 0.f}, sd{0.f, 0.f};
+        const float2 pq = A[p + la * q], pv = A[p + la * p], qv = A[q + la * q];
+        if (q < s && pq.x != 0.f) rot_angle(dfl{pv.x, pv.y}, dfl{qv.x, qv.y}, dfl{pq.x, pq.y}, &cd, &sd);
         csp[k] = make_float2(cd.hi, cd.lo);
         snp[k] = make_float2(sd.hi, sd.lo);
         pp[k] = p;
         qq[k] = q;
       }
       __syncthreads();
-      for (int t = threadIdx.x; t < (m / 2) * s; t += blockDim.x) {  // rows: A <- J^T A
-        const int k = t / s, col = t % s;
-        const int p = pp[k], q = qq[k];
-        if (q >= s) continue;
-        const dfl c{csp[k].x, csp[k].y}, sn{snp[k].x, snp[k].y}, msn{-snp[k].x, -snp[k].y};
-        const float2 ap2 = A[p + la * col], aq2 = A[q + la * col];
-        const dfl ap{ap2.x, ap2.y}, aq{aq2.x, aq2.y};
-        const dfl np_ = rot_mix(c, ap, msn, aq), nq = rot_mix(sn, ap, c, aq);
-        A[p + la * col] = make_float2(np_.hi, np_.lo);
-        A[q + la * col] = make_float2(nq.hi, nq.lo);
-      }
-      __syncthreads();
-      for (int t = threadIdx.x; t < (m / 2) * s; t += blockDim.x) {  // columns: A <- A J, V <- V J
-        const int k = t / s, row = t % s;
-        const int p = pp[k], q = qq[k];
-        if (q >= s) continue;
-        const dfl c{csp[k].x, csp[k].y}, sn{snp[k].x, snp[k].y}, msn{-snp[k].x, -snp[k].y};
-        const float2 ap2 = A[row + la * p], aq2 = A[row + la * q];
-        const dfl ap{ap2.x, ap2.y}, aq{aq2.x, aq2.y};
-        const dfl np_ = rot_mix(c, ap, msn, aq), nq = rot_mix(sn, ap, c, aq);
-        A[row + la * p] = make_float2(np_.hi, np_.lo);
-        A[row + la * q] = make_float2(nq.hi, nq.lo);
-        const float2 vp2 = V[row + lv * p], vq2 = V[row + lv * q];
-        const dfl vp{vp2.x, vp2.y}, vq{vq2.x, vq2.y};
-        const dfl nvp = rot_mix(c, vp, msn, vq), nvq = rot_mix(sn, vp, c, vq);
-        V[row + lv * p] = make_float2(nvp.hi, nvp.lo);
-        V[row + lv * q] = make_float2(nvq.hi, nvq.lo);
+      // A <- J^T A J and V <- V J
+      for (unsigned t = threadIdx.x; t < nblk + h * nr4; t += blockDim.x) {
+        if (t < nblk) {
+          const int br = nbc == 1 ? 0 : (int)__umulhi(t, mbc), bc = (int)t - br * (int)nbc;
+          int a, b;
+          if (h & 1) {
+            a = bc >= br ? br : h - br;
+            b = bc >= br ? bc : h - 1 - bc;
+          } else {
+            a = bc > br ? br : h - 1 - br;
+            b = bc > br ? bc - 1 : h - 1 - bc;
+          }
+          const int p1 = pp[a], q1 = qq[a], p2 = pp[b], q2 = qq[b];
+          const dfl c1{csp[a].x, csp[a].y}, s1{snp[a].x, snp[a].y}, c2{csp[b].x, csp[b].y}, s2{snp[b].x, snp[b].y};
+          auto ld = [&](int i, int j) {
+            const float2 v = A[i + la * j];
+            return dfl{v.x, v.y};
+          };
+          dfl xpp = ld(p1, p2), xpq = ld(p1, q2), xqp = ld(q1, p2), xqq = ld(q1, q2);
+          rot(c1, s1, xpp, xqp);
+          rot(c1, s1, xpq, xqq);
+          rot(c2, s2, xpp, xpq);
+          rot(c2, s2, xqp, xqq);
+          if (a == b) xqp = xpq;
+          auto put = [&](int i, int j, dfl v) { A[i + la * j] = A[j + la * i] = make_float2(v.hi, v.lo); };
+          put(p1, p2, xpp);
+          put(p1, q2, xpq);
+          put(q1, p2, xqp);
+          put(q1, q2, xqq);
+        } else {
+          const unsigned u = t - nblk;
+          const int k = nr4 == 1 ? (int)u : (int)__umulhi(u, mr4), r0 = (int)u - k * (int)nr4;
+          const int p = pp[k], q = qq[k];
+          if (q >= s) continue;
+          const dfl c{csp[k].x, csp[k].y}, sn{snp[k].x, snp[k].y};
+#pragma unroll
+          for (int e = 0; e < 4; ++e) {
+            const int row = r0 + e * (int)nr4;
+            if (row >= s) break;
+            const float2 vp = V[row + lv * p], vq = V[row + lv * q];
+            dfl x{vp.x, vp.y}, y{vq.x, vq.y};
+            rot(c, sn, x, y);
+            V[row + lv * p] = make_float2(x.hi, x.lo);
+            V[row + lv * q] = make_float2(y.hi, y.lo);
+          }
+        }
       }
       __syncthreads();
     }
@@ -795,7 +911,7 @@ int small_symeig(hp_problem *P, const double *T, int s, double *lambda, double *
       HP_TRY(P->vtmp[3].ensure(sizeof(float2) * (size_t)s * s));
       Vg = P->vtmp[3].as<float2>();
     }
-    const size_t shm = sizeof(float2) * ((v_shared ? 2 : 1) * (size_t)(s + 1) * s + m) + sizeof(double) * 64 +
+    const size_t shm = sizeof(float2) * ((v_shared ? 2 : 1) * (size_t)(m + 1) * m + m) + sizeof(double) * 64 +
                        sizeof(int) * 2 * (size_t)std::max(m, s);
     static std::atomic<unsigned long long> attr_df{0};
     int dev = 0;
