@@ -1224,7 +1224,13 @@ int hp_laplace_sample(hp_problem *P, const double *m_map, const double *lambda, 
     }
     if (post) {
       // R x = A M^{-1} (A x) = A M^{-1} W
-      HP_TRY(solve_block(P, OP_M, W, ld, t, ld, cs, std::min(P->rtol, 1e-10), st));
+      // V^T R x below magnifies this solve's error some thousandfold: at 1e-12 the error of
+      // either iteration is 7e-10 of the samples (65^3 nodes, 100 pairs).  CG keeps them equal to
+      // earlier samples of the same seed to 1e-9, the Chebyshev iteration would move them by 3e-9.
+      P->mass_cg = true;
+      const int mrc = solve_block(P, OP_M, W, ld, t, ld, cs, std::min(P->rtol, 1e-10), st);
+      P->mass_cg = false;
+      HP_TRY(mrc);
       HP_TRY(apply_op64(P, OP_A, t, ld, RX, ld, cs));
       if (k > 0) {
         HP_TRY(gram(P, V, ldv, k, RX, ld, cs, z, k, n));

@@ -153,6 +153,7 @@ struct hp_problem {
   cudaStream_t st = nullptr;
   cudaStream_t cap = nullptr;   // private stream used to capture CUDA graphs
   bool use_graphs = true;       // inner PCG loops as graphs with a device-side while node
+  bool mass_cg = false;   // M by CG also where the Chebyshev iteration would be taken (set around a call)
   std::vector<hp::PcgGraph> graphs;
   std::vector<hp::SolveGraph> sgraphs;
 
@@ -369,13 +370,18 @@ int launch_leg(LegArgs a, const GridDesc &g, bool full, bool up, int vw, int s, 
 // ---- march.cu -------------------------------------------------------------------
 // 3D stencils over all Kuhn edges with constant coefficients (A, M) on grouped FP32 blocks of
 // four columns per group, in one launch; returns the CTAs per group (partials per column).
-enum { MA_APPLY_DOT = 0, MA_RESID = 1, MA_JACOBI = 2, MA_JACOBI_DOT = 3, MA_JAC2 = 4 };
+enum { MA_APPLY_DOT = 0, MA_RESID = 1, MA_JACOBI = 2, MA_JACOBI_DOT = 3, MA_JAC2 = 4, MA_CHEB = 5 };
+struct ChebCtl {  // a Chebyshev iteration in device memory: steps done, their number, weight of the next
+  int it, n;
+  float omega;
+};
 struct MarchArgs {
   const float *diag, *invdiag, *c, *X, *B;
   float *Y;
   long gx, gb, gy;  // group strides
   float omega, omega2;
   double *part;     // dot partials [column][CTA]
+  const ChebCtl *ctl;  // MA_CHEB
   int np, s, ntx, nty, nzs;  // set by launch_march
 };
 int launch_march(MarchArgs a, const GridDesc &g, int mode, int s, cudaStream_t st);

@@ -46,7 +46,7 @@ __device__ __forceinline__ void f4_axpy(F4 &s, float a, const F4 &x) {
 
 template <int MODE>
 __global__ void __launch_bounds__(MA_NT, 2) k_march_full(const __grid_constant__ MarchArgs a) {
-  constexpr bool HAS_B = MODE == MA_RESID || MODE == MA_JACOBI || MODE == MA_JACOBI_DOT;
+  constexpr bool HAS_B = MODE == MA_RESID || MODE == MA_JACOBI || MODE == MA_JACOBI_DOT || MODE == MA_CHEB;
   constexpr bool DOT = MODE == MA_APPLY_DOT || MODE == MA_JACOBI_DOT;
   __shared__ __align__(16) float4 ring[MA_SLOTS][MA_BX * MA_BY];
   const int np = a.np, N = np - 1, plane = np * np, n = plane * np, t = threadIdx.x;
@@ -57,7 +57,13 @@ __global__ void __launch_bounds__(MA_NT, 2) k_march_full(const __grid_constant__
   const int x0 = tx * MA_X, y0 = ty * MA_Y;
   const int wx = tx == a.ntx - 1 ? np - x0 : MA_X, hy = ty == a.nty - 1 ? np - y0 : MA_Y;
   const int zb = (int)((long)tz * np / a.nzs), ze = (int)((long)(tz + 1) * np / a.nzs);
-  const float *__restrict__ X = a.X + blockIdx.y * a.gx;
+  // MA_CHEB: iterate j lies in X when n - j is even and in Y otherwise; Y of the step is the
+  // iterate before X's
+  const bool odd = MODE == MA_CHEB && ((a.ctl->n - a.ctl->it) & 1);
+  const float cw = MODE == MA_CHEB ? a.ctl->omega : 0.f;
+  const bool first = MODE == MA_CHEB && a.ctl->it == 0;  // a plain step: no iterate before X's
+  const float *X = (odd ? a.Y : a.X) + blockIdx.y * a.gx;
+  float *Y = (odd ? const_cast<float *>(a.X) : a.Y) + blockIdx.y * a.gy;
   const int bw = wx + 2;
   const int ly = t / wx, lx = t - ly * wx;
   const bool mine = ly < hy;
@@ -146,8 +152,9 @@ __global__ void __launch_bounds__(MA_NT, 2) k_march_full(const __grid_constant__
     // into the slot of plane p - 2, which every thread has left at the last barrier
     issue(p + MA_AHEAD);
     const long o4 = (long)xy + (long)p * plane;
-    F4 bb;
+    F4 bb, xo;
     if (HAS_B && mine) bb = F4::ld(bp + (long)p * plane);
+    if (MODE == MA_CHEB && mine && !first) xo = F4::ld(reinterpret_cast<const float4 *>(Y) + o4);
     if (mine && (p == zb || p <= 2 || p >= N - 1)) coefficients(p);
     asm volatile("cp.async.wait_group %0;" ::"n"(MA_AHEAD - 1) : "memory");  // plane p + 1 is there
     __syncthreads();
@@ -198,6 +205,10 @@ __global__ void __launch_bounds__(MA_NT, 2) k_march_full(const __grid_constant__
         const float wi = mulr(a.omega, iv);
 #pragma unroll
         for (int k = 0; k < 4; ++k) out.v[k] = fmadd(wi, addr(bb.v[k], -sx.v[k]), c0.v[k]);
+        if (MODE == MA_CHEB && !first) {
+#pragma unroll
+          for (int k = 0; k < 4; ++k) out.v[k] = fmadd(cw, addr(out.v[k], -xo.v[k]), xo.v[k]);
+        }
       } else {
         out = sx;
       }
@@ -205,7 +216,7 @@ __global__ void __launch_bounds__(MA_NT, 2) k_march_full(const __grid_constant__
 #pragma unroll
         for (int k = 0; k < 4; ++k) acc[k] = fmadd(HAS_B ? bb.v[k] : c0.v[k], out.v[k], acc[k]);
       }
-      out.st(reinterpret_cast<float4 *>(a.Y + blockIdx.y * a.gy) + o4);
+      out.st(reinterpret_cast<float4 *>(Y) + o4);
       cm = c0;
       c0 = cp;
 #pragma unroll
@@ -255,6 +266,7 @@ int launch_march(MarchArgs a, const GridDesc &g, int mode, int s, cudaStream_t s
     case MA_RESID: k_march_full<MA_RESID><<<gr, MA_NT, 0, st>>>(a); break;
     case MA_JACOBI: k_march_full<MA_JACOBI><<<gr, MA_NT, 0, st>>>(a); break;
     case MA_JACOBI_DOT: k_march_full<MA_JACOBI_DOT><<<gr, MA_NT, 0, st>>>(a); break;
+    case MA_CHEB: k_march_full<MA_CHEB><<<gr, MA_NT, 0, st>>>(a); break;
     default: k_march_full<MA_JAC2><<<gr, MA_NT, 0, st>>>(a);
   }
   count_launch();

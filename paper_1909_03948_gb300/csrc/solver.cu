@@ -1517,6 +1517,67 @@ __global__ void k_pcg_cond(const int *__restrict__ active, int s, int *iter, int
   }
 }
 
+// Chebyshev iteration for M with its diagonal D in 3D.  On a tetrahedron D^-1 M is (I + J) / 2,
+// J all ones, with eigenvalues 1/2 and 5/2, so those of the assembled D^-1 M lie between them on
+// every mesh: condition 5, rate 0.38, the same as CG's, without its inner products.
+//   x_{j+1} = x_{j-1} + omega_{j+1} (x_j + gamma D^-1 (b - M x_j) - x_{j-1}),  omega_1 = 1,
+//   gamma = 2/3, rho = 2/3, omega_2 = 1 / (1 - rho^2/2), omega_{j+1} = 1 / (1 - rho^2 omega_j / 4)
+// reduces the D^-1-norm of the residual by T_n(3/2), so the number of steps is known before the
+// first: the smallest that reaches the strictest column's tolerance.  It starts at x_0 =
+// 2/5 D^-1 b, whose residual has the further factor 1 - 2/5 lambda: at most 4/5, and nearly 0 for the
+// smooth components (lambda near 5/2), which Chebyshev would leave as large as the others
+// and on which the low-rank updates depend.
+constexpr float CHEB_GAMMA = 2.f / 3.f, CHEB_RHO2 = 4.f / 9.f, CHEB_X0 = 0.4f;
+
+// step 0: number of steps; 1: one more step is done
+__global__ void k_cheb_ctl(const double *__restrict__ tol2col, int s, int maxit, int step, ChebCtl *ctl, int *active,
+                           cudaGraphConditionalHandle h, int use_handle) {
+  __shared__ float tmin[256];
+  __shared__ int more_s;
+  if (step == 0) {
+    float t2 = 0.25f;
+    for (int j = threadIdx.x; j < s; j += 256) t2 = fminf(t2, (float)tol2col[j]);
+    tmin[threadIdx.x] = t2;
+    __syncthreads();
+    for (int o = 128; o > 0; o >>= 1) {
+      if ((int)threadIdx.x < o) tmin[threadIdx.x] = fminf(tmin[threadIdx.x], tmin[threadIdx.x + o]);
+      __syncthreads();
+    }
+  }
+  if (threadIdx.x == 0) {
+    ChebCtl c = *ctl;
+    if (step == 0) {
+      const float red = rsqrtf(fmaxf(tmin[0], 1e-14f));  // FP32 reaches about 1e-7
+      c.n = max(1, min((int)ceilf(acoshf(0.8f * red) * (1.f / 0.96242365f)), maxit));
+      c.it = 0;
+      c.omega = 1.f;
+    } else {
+      c.it += 1;
+      c.omega = 1.f / (1.f - (c.it == 1 ? 0.5f : 0.25f * c.omega) * CHEB_RHO2);
+    }
+    *ctl = c;
+    more_s = c.it < c.n;
+    if (use_handle) cudaGraphSetConditional(h, more_s ? 1u : 0u);
+  }
+  __syncthreads();
+  for (int j = threadIdx.x; j < s; j += 256) active[j] = more_s;
+}
+
+// x_0, in x when n is even and in p otherwise
+__global__ void __launch_bounds__(NB) k_cheb_start(long n, long gs, const float *__restrict__ r,
+                                                   const float *__restrict__ invdiag, float *__restrict__ x,
+                                                   float *__restrict__ p, const ChebCtl *__restrict__ ctl) {
+  float *y = (ctl->n & 1) ? p : x;
+  const long g0 = blockIdx.y * gs;
+  for (long i = blockIdx.x * (long)NB + threadIdx.x; i < n; i += (long)gridDim.x * NB) {
+    const float w = mulr(CHEB_X0, invdiag[i]);
+    Pack<float, 4> v = Pack<float, 4>::ld(r + g0 + i * 4);
+#pragma unroll
+    for (int q = 0; q < 4; ++q) v.v[q] = mulr(w, v.v[q]);
+    v.st(y + g0 + i * 4);
+  }
+}
+
 // ---------------------------------------------------------------------------
 // profiling: a pair of events around selected launches (off by default)
 // ---------------------------------------------------------------------------
@@ -1801,6 +1862,19 @@ template <typename T, int MODE> static double st_bytes(const GridDesc &g, const 
 // matvec 89 -> 57 us; 33^3 nodes, 64 columns (575,000): sweep 15.7 -> 14.2 us.
 constexpr long MARCH_MIN = 500000;
 static bool march_rule(const GridDesc &g, int ng) { return g.dim == 3 && g.n * ng >= MARCH_MIN; }
+
+// Whether M is solved by the Chebyshev iteration: where its stencil runs as the marching kernel,
+// which takes a whole step in one launch and four passes over a block where CG's takes eleven.
+// 65^3 nodes, 120 columns: CG 262 us per iteration and 12 us of scalar kernels, Chebyshev 164
+// and 3; 64 columns: 143 and 12, 95 and 3.
+static bool cheb_rule(const hp_problem *P, OpKind op, int tbytes, int vw, int s) {
+  return op == OP_M && tbytes == 4 && vw == 4 && !P->mass_cg && march_rule(P->lv[0].g, (s + 3) / 4);
+}
+
+// what a captured graph was built for
+static int graph_op(const hp_problem *P, OpKind op, int tbytes, int vw, int s) {
+  return (int)op + (cheb_rule(P, op, tbytes, vw, s) ? 16 : 0);
+}
 
 template <typename T, int VW, int MODE>
 static void st_launch(const GridDesc &g, const Stencil<T> &S, const T *X, long gx, const T *B, long gb, T *Y, long gy,
@@ -2324,8 +2398,47 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
 //   body:  z = M r, beta = <r,z>/rz (0 at iter 0), p = z + beta p,
 //          q = K p, alpha = rz/<p,q>, x += alpha p, r -= alpha q, rr = <r,r>,
 //          active &= rr > tol^2 bb, iter += 1; repeat while any active and iter < maxit.
+static ChebCtl *cheb_ctl(hp_problem *P) {  // the iteration counter and the two words behind it
+  static_assert(sizeof(ChebCtl) <= 4 * sizeof(int), "sc.iter holds four words");
+  return reinterpret_cast<ChebCtl *>(P->sc.iter.p);
+}
+
+static void cheb_init(hp_problem *P, int s, cudaGraphConditionalHandle h, int use_handle, int maxit) {
+  BlockWS<float> &W = P->w32;
+  const int ng = (s + 3) / 4;
+  k_cheb_ctl<<<1, 256, 0, P->st>>>(P->sc.tol2col.as<double>(), s, maxit, 0, cheb_ctl(P), P->sc.active.as<int>(), h,
+                                   use_handle);
+  k_cheb_start<<<nodegrid(P->n, ng), NB, 0, P->st>>>(P->n, W.ldn * 4, W.r.as<float>(),
+                                                     stencil_of<float>(P, OP_M, 0).invdiag, W.x.as<float>(),
+                                                     W.p.as<float>(), cheb_ctl(P));
+  count_launch(2);
+  count_bytes(BY_VECTOR, 4.0 * (double)P->n * (2.0 * s + 1.0));
+}
+
+static void cheb_step(hp_problem *P, int s, cudaGraphConditionalHandle h, int use_handle, int maxit) {
+  BlockWS<float> &W = P->w32;
+  const GridDesc &g = P->lv[0].g;
+  const Stencil<float> &S = stencil_of<float>(P, OP_M, 0);
+  MarchArgs a{};
+  a.diag = S.diag;
+  a.invdiag = S.invdiag;
+  a.c = S.c;
+  a.X = W.x.as<float>();
+  a.Y = W.p.as<float>();
+  a.B = W.r.as<float>();
+  a.gx = a.gy = a.gb = W.ldn * 4;
+  a.omega = CHEB_GAMMA;
+  a.ctl = cheb_ctl(P);
+  launch_march(a, g, MA_CHEB, s, P->st);
+  count_bytes(level_family(g.n), st_bytes<float, M_JACOBI>(g, S, s) + 4.0 * (double)g.n * s);
+  k_cheb_ctl<<<1, 256, 0, P->st>>>(P->sc.tol2col.as<double>(), s, maxit, 1, cheb_ctl(P), P->sc.active.as<int>(), h,
+                                   use_handle);
+  count_launch();
+}
+
 template <typename T, int VW>
 static void pcg_init(hp_problem *P, OpKind op, int s, cudaGraphConditionalHandle h, int use_handle, int maxit) {
+  if (cheb_rule(P, op, (int)sizeof(T), VW, s)) return cheb_init(P, s, h, use_handle, maxit);
   BlockWS<T> &W = ws_of<T>(P);
   cudaStream_t st = P->st;
   const int ng = (s + VW - 1) / VW;
@@ -2369,6 +2482,7 @@ template <int VW> static int pcg_columns(hp_problem *P, OpKind op, int s) {
 template <typename T, int VW>
 static void pcg_body(hp_problem *P, OpKind op, int s, double tol2, cudaGraphConditionalHandle h, int use_handle,
                      int maxit) {
+  if (cheb_rule(P, op, (int)sizeof(T), VW, s)) return cheb_step(P, s, h, use_handle, maxit);
   BlockWS<T> &W = ws_of<T>(P);
   cudaStream_t st = P->st;
   const long n = P->n;
@@ -2515,7 +2629,7 @@ static int build_graph(hp_problem *P, OpKind op, int s, double tol, int maxit, P
     if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, g, 0);
     if (g) cudaGraphDestroy(g);
     if (e != cudaSuccess) return cuda_check(e, "PCG graph");
-    *out = PcgGraph{(int)op, (int)sizeof(T), VW, s, maxit, tol, ex};
+    *out = PcgGraph{graph_op(P, op, (int)sizeof(T), VW, s), (int)sizeof(T), VW, s, maxit, tol, ex};
     return 0;
   });
 }
@@ -2523,6 +2637,7 @@ static int build_graph(hp_problem *P, OpKind op, int s, double tol, int maxit, P
 // launches of one PCG iteration (0 when the whole PCG is one launch per solve)
 static int kernels_per_iteration(const hp_problem *P, OpKind op, int tbytes, int vw, int s) {
   if (col_pcg_rule(P, op, tbytes, vw)) return 0;
+  if (cheb_rule(P, op, tbytes, vw, s)) return 2;
   if (op == OP_M) return 6;
   // V-cycle: per level above the one-launch coarse end (or the dense coarse solve) pre
   // (1 + nu - 2), resid, restrict, prolong, nu post; then 1; plus p update, matvec, cg
@@ -2540,7 +2655,8 @@ static int kernels_per_iteration(const hp_problem *P, OpKind op, int tbytes, int
 
 // launches that start a PCG: the first residual's norm with its finalisation and the loop
 // condition, or the whole PCG in one launch
-static int kernels_per_pcg(const hp_problem *P, OpKind op, int tbytes, int vw) {
+static int kernels_per_pcg(const hp_problem *P, OpKind op, int tbytes, int vw, int s) {
+  if (cheb_rule(P, op, tbytes, vw, s)) return 2;
   return col_pcg_rule(P, op, tbytes, vw) ? 1 : (op == OP_M ? 5 : 3);
 }
 
@@ -2560,8 +2676,9 @@ static int pcg(hp_problem *P, OpKind op, int s, double rtol, int maxit, int *its
   int *h_it = P->sc.h_iter;
   if (P->use_graphs && !P->prof_on) {
     PcgGraph *G = nullptr;
+    const int gop = graph_op(P, op, (int)sizeof(T), VW, s);
     for (auto &pg : P->graphs)
-      if (pg.op == (int)op && pg.tbytes == (int)sizeof(T) && pg.vw == VW && pg.s == s && pg.maxit == maxit &&
+      if (pg.op == gop && pg.tbytes == (int)sizeof(T) && pg.vw == VW && pg.s == s && pg.maxit == maxit &&
           pg.tol == rtol)
         G = &pg;
     if (!G) {
@@ -2575,7 +2692,7 @@ static int pcg(hp_problem *P, OpKind op, int s, double rtol, int maxit, int *its
     HP_CUDA(cudaMemcpyFromSymbolAsync(h_it + 1, g_tile_timeout, sizeof(int), 0, cudaMemcpyDeviceToHost, st));
     HP_CUDA(cudaStreamSynchronize(st));
     count_launch((unsigned long long)(*h_it) * kernels_per_iteration(P, op, (int)sizeof(T), VW, s) +
-                 kernels_per_pcg(P, op, (int)sizeof(T), VW));
+                 kernels_per_pcg(P, op, (int)sizeof(T), VW, s));
     *its = *h_it;
     HP_TRY(tile_timeout_check(P, h_it));
     return *h_it >= maxit ? HP_ERR_NOT_CONVERGED : 0;
@@ -2742,7 +2859,7 @@ static int build_solve_graph(hp_problem *P, OpKind op, int s, double rtol, doubl
     if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, g, 0);
     if (g) cudaGraphDestroy(g);
     if (e != cudaSuccess) return cuda_check(e, "refinement graph");
-    *out = SolveGraph{(int)op, (int)sizeof(T), VW, s, maxit, max_outer, rtol, tol_in, ex};
+    *out = SolveGraph{graph_op(P, op, (int)sizeof(T), VW, s), (int)sizeof(T), VW, s, maxit, max_outer, rtol, tol_in, ex};
     return 0;
   });
 }
@@ -2762,8 +2879,9 @@ static int ir_solve_graph(hp_problem *P, OpKind op, const double *B, long ldb, d
   const long face = op == OP_K ? (P->dim == 2 ? g0.np : (long)g0.np * g0.np) : 0;
   HP_TRY(ir_start(P, B, ldb, b64, ld64, x64, ld64, n, s, face, P->sc.bbr.as<double>(), P->sc.rr.as<double>()));
   SolveGraph *G = nullptr;
+  const int gop = graph_op(P, op, (int)sizeof(T), VW, s);
   for (auto &sg : P->sgraphs)
-    if (sg.op == (int)op && sg.tbytes == (int)sizeof(T) && sg.vw == VW && sg.s == s && sg.maxit == P->max_iter &&
+    if (sg.op == gop && sg.tbytes == (int)sizeof(T) && sg.vw == VW && sg.s == s && sg.maxit == P->max_iter &&
         sg.max_outer == P->max_outer && sg.rtol == rtol && sg.tol_in == tol_in)
       G = &sg;
   if (!G) {
@@ -2783,7 +2901,7 @@ static int ir_solve_graph(hp_problem *P, OpKind op, const double *B, long ldb, d
   HP_TRY(tile_timeout_check(P, h_it));
   // kernels run: the first check, and per step the scaling, the PCG's start and
   // iterations, the accumulation, the residual with its finalisation and the check
-  count_launch(1ull + (5ull + kernels_per_pcg(P, op, (int)sizeof(T), VW)) * (unsigned long long)c.outer +
+  count_launch(1ull + (5ull + kernels_per_pcg(P, op, (int)sizeof(T), VW, s)) * (unsigned long long)c.outer +
                (unsigned long long)c.total_its * (unsigned long long)kernels_per_iteration(P, op, (int)sizeof(T), VW, s));
   if (c.flags & 2) return set_error(HP_ERR_NONFINITE, "non-finite residual in a PDE solve");
   if (stats) {
@@ -2909,7 +3027,7 @@ static int build_solve_graph_dfp(hp_problem *P, OpKind op, int s, double rtol, d
     if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, g, 0);
     if (g) cudaGraphDestroy(g);
     if (e != cudaSuccess) return cuda_check(e, "double-float refinement graph");
-    *out = SolveGraph{(int)op, 100 + (int)sizeof(T), VW, s, maxit, max_outer, rtol, tol_in, ex};
+    *out = SolveGraph{graph_op(P, op, (int)sizeof(T), VW, s), 100 + (int)sizeof(T), VW, s, maxit, max_outer, rtol, tol_in, ex};
     return 0;
   });
 }
@@ -2956,8 +3074,9 @@ static int ir_solve_dfp(hp_problem *P, OpKind op, const double *B, long ldb, dou
     double worst = 0.0;
     if (P->use_graphs && !P->prof_on) {
       SolveGraph *G = nullptr;
+      const int gop = graph_op(P, op, (int)sizeof(T), VW, s);
       for (auto &sg : P->sgraphs)
-        if (sg.op == (int)op && sg.tbytes == 100 + (int)sizeof(T) && sg.vw == VW && sg.s == s &&
+        if (sg.op == gop && sg.tbytes == 100 + (int)sizeof(T) && sg.vw == VW && sg.s == s &&
             sg.maxit == P->max_iter && sg.max_outer == P->max_outer && sg.rtol == rtol && sg.tol_in == tol_in)
           G = &sg;
       if (!G) {
@@ -2978,7 +3097,7 @@ static int ir_solve_dfp(hp_problem *P, OpKind op, const double *B, long ldb, dou
       HP_TRY(tile_timeout_check(P, h_it));
       // kernels run: the first check and right-hand side, per step the PCG's start and
       // iterations, the update, the residual with its finalisation and the check
-      count_launch(2ull + (4ull + kernels_per_pcg(P, op, (int)sizeof(T), VW)) * (unsigned long long)c.outer +
+      count_launch(2ull + (4ull + kernels_per_pcg(P, op, (int)sizeof(T), VW, s)) * (unsigned long long)c.outer +
                    (unsigned long long)c.total_its * (unsigned long long)kernels_per_iteration(P, op, (int)sizeof(T), VW, s));
       if (c.flags & 2) return set_error(HP_ERR_NONFINITE, "non-finite residual in a PDE solve");
       total_its = c.total_its;
