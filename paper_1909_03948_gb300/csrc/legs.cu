@@ -204,8 +204,9 @@ __global__ void __launch_bounds__(LEG_NT, VW == 4 ? 2 : 3) k_leg_down(const __gr
   float *v = A, *o = B;
   if (mine) {
     C.init(a, x0, y0, halo, strip, col);
-    C.load(a, a.r + grp * a.gs, r);
   }
+  pdl_enter();  // the coefficients are older than the kernel before this one
+  if (mine) C.load(a, a.r + grp * a.gs, r);
   if (a.nu >= 2) {
     // two sweeps from zero (k_st's M_JAC2): e1 = w1 D^-1 r, x = e1 + w2 D^-1 (r - S e1), the
     // neighbours entering as (c w1 / diag) r
@@ -337,6 +338,9 @@ __global__ void __launch_bounds__(LEG_NT, VW == 4 ? 2 : 3) k_leg_up(const __grid
   leg_pad<VW>(a, o);
   if (mine) {
     C.init(a, x0, y0, halo, strip, col);
+  }
+  pdl_enter();  // as in k_leg_down
+  if (mine) {
     C.load(a, a.xin + grp * a.gs, x);
     C.load(a, a.r + grp * a.gs, r);
     // x += P e_c (see k_prolong_add): e_c at the coarse node below, or the mean with its
@@ -454,7 +458,7 @@ int launch_leg(LegArgs a, const GridDesc &g, bool full, bool up, int vw, int s, 
   else
     k = full ? (up ? (dot ? (K)k_leg_up<1, true, true> : (K)k_leg_up<1, true, false>) : (K)k_leg_down<1, true>)
              : (up ? (dot ? (K)k_leg_up<1, false, true> : (K)k_leg_up<1, false, false>) : (K)k_leg_down<1, false>);
-  k<<<dim3(a.ntx * a.nty, (s + vw - 1) / vw), nt, shm, st>>>(a);
+  pdl_launch(k, dim3(a.ntx * a.nty, (s + vw - 1) / vw), nt, shm, st, a);
   count_launch();
   return cuda_check(cudaGetLastError(), "level leg");
 }

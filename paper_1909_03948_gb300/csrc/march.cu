@@ -46,6 +46,7 @@ __device__ __forceinline__ void f4_axpy(F4 &s, float a, const F4 &x) {
 
 template <int MODE>
 __global__ void __launch_bounds__(MA_NT, 2) k_march_full(const __grid_constant__ MarchArgs a) {
+  pdl_enter();
   constexpr bool HAS_B = MODE == MA_RESID || MODE == MA_JACOBI || MODE == MA_JACOBI_DOT || MODE == MA_CHEB;
   constexpr bool DOT = MODE == MA_APPLY_DOT || MODE == MA_JACOBI_DOT;
   __shared__ __align__(16) float4 ring[MA_SLOTS][MA_BX * MA_BY];
@@ -262,12 +263,12 @@ int launch_march(MarchArgs a, const GridDesc &g, int mode, int s, cudaStream_t s
   a.nzs = march_segs(g, ng, a.ntx * a.nty);
   const dim3 gr(a.ntx * a.nty * a.nzs, ng);
   switch (mode) {
-    case MA_APPLY_DOT: k_march_full<MA_APPLY_DOT><<<gr, MA_NT, 0, st>>>(a); break;
-    case MA_RESID: k_march_full<MA_RESID><<<gr, MA_NT, 0, st>>>(a); break;
-    case MA_JACOBI: k_march_full<MA_JACOBI><<<gr, MA_NT, 0, st>>>(a); break;
-    case MA_JACOBI_DOT: k_march_full<MA_JACOBI_DOT><<<gr, MA_NT, 0, st>>>(a); break;
-    case MA_CHEB: k_march_full<MA_CHEB><<<gr, MA_NT, 0, st>>>(a); break;
-    default: k_march_full<MA_JAC2><<<gr, MA_NT, 0, st>>>(a);
+    case MA_APPLY_DOT: pdl_launch(k_march_full<MA_APPLY_DOT>, gr, MA_NT, 0, st, a); break;
+    case MA_RESID: pdl_launch(k_march_full<MA_RESID>, gr, MA_NT, 0, st, a); break;
+    case MA_JACOBI: pdl_launch(k_march_full<MA_JACOBI>, gr, MA_NT, 0, st, a); break;
+    case MA_JACOBI_DOT: pdl_launch(k_march_full<MA_JACOBI_DOT>, gr, MA_NT, 0, st, a); break;
+    case MA_CHEB: pdl_launch(k_march_full<MA_CHEB>, gr, MA_NT, 0, st, a); break;
+    default: pdl_launch(k_march_full<MA_JAC2>, gr, MA_NT, 0, st, a);
   }
   count_launch();
   return (int)gr.x;

@@ -150,6 +150,7 @@ __device__ __forceinline__ void dot_partial(const Pack<T, VW> &acc, double *part
 }
 
 __global__ void k_dot_finalize(const double *__restrict__ part, unsigned nblk, Fin fin) {
+  pdl_enter();
   const int col = blockIdx.x;
   double sum = 0.0;
   for (unsigned b = threadIdx.x; b < nblk; b += NB) sum += part[(long)col * nblk + b];
@@ -160,6 +161,7 @@ __global__ void k_dot_finalize(const double *__restrict__ part, unsigned nblk, F
 // two products at once: fin's partials, then fin2's
 __global__ void k_dot_finalize2(const double *__restrict__ part, const double *__restrict__ part2, unsigned nblk,
                                 Fin fin, Fin fin2) {
+  pdl_enter();
   const int col = blockIdx.x;
   double sum = 0.0, sum2 = 0.0;
   for (unsigned b = threadIdx.x; b < nblk; b += NB) {
@@ -175,7 +177,7 @@ __global__ void k_dot_finalize2(const double *__restrict__ part, const double *_
 }
 
 static void dot_finalize(const Fin &fin, unsigned nblk, int s, cudaStream_t st) {
-  k_dot_finalize<<<s, NB, 0, st>>>(fin.part, nblk, fin);
+  pdl_launch(k_dot_finalize, s, NB, 0, st, fin.part, nblk, fin);
   count_launch();
 }
 
@@ -191,6 +193,7 @@ __global__ void __launch_bounds__(NB) k_st(GridDesc g, const T *__restrict__ dia
                                            const T *__restrict__ c, const T *__restrict__ X, long gx,
                                            const T *__restrict__ B, long gb, T *__restrict__ Y, long gy, int s,
                                            T omega, T omega2, Fin fin) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   const int lane = threadIdx.x & 31;
   const int i0 = blockIdx.x * 32 + lane;
@@ -677,6 +680,7 @@ __global__ void __launch_bounds__(NB) k_st64(GridDesc g, const double *__restric
                                              const double *__restrict__ c, const double *__restrict__ X, long ldx,
                                              const double *__restrict__ B, long ldb, double *__restrict__ Y, long ldy,
                                              int s, double *part) {
+  pdl_enter();
   constexpr int NF = FULL ? (1 << D) - 1 : D;
   const int j0 = blockIdx.y * C64;
   const double *x[C64];
@@ -750,6 +754,7 @@ __global__ void __launch_bounds__(NB) k_st64(GridDesc g, const double *__restric
 template <typename T, int VW, int D>
 __global__ void __launch_bounds__(NB) k_restrict(GridDesc gf, GridDesc gc, const T *__restrict__ rf, long gsf,
                                                  T *__restrict__ rc, long gsc, int zero_dirichlet) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   // one coarse node per thread over the flattened grid (every lane busy whatever np is)
   const unsigned I = blockIdx.x * NB + threadIdx.x;
@@ -783,6 +788,7 @@ __global__ void __launch_bounds__(NB) k_restrict(GridDesc gf, GridDesc gc, const
 template <typename T, int VW, int D>
 __global__ void __launch_bounds__(NB) k_prolong_add(GridDesc gf, GridDesc gc, const T *__restrict__ ec, long gsc,
                                                     T *__restrict__ ef, long gsf) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   // one fine node per thread over the flattened grid (every lane busy whatever np is)
   const unsigned i = blockIdx.x * NB + threadIdx.x;
@@ -842,6 +848,7 @@ __global__ void __launch_bounds__(NB) k_resid_restrict(GridDesc gf, GridDesc gc,
                                                        const T *__restrict__ c, const T *__restrict__ e,
                                                        const T *__restrict__ bf, long gsf, T *__restrict__ rc,
                                                        long gsc, int zero_dirichlet) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   const int I0 = blockIdx.x * 32 + (threadIdx.x & 31);
   const int row = blockIdx.y * (NB / 32) + (threadIdx.x >> 5);
@@ -895,6 +902,7 @@ __global__ void __launch_bounds__(NB) k_prolong_sweep(GridDesc gf, GridDesc gc, 
                                                       const T *__restrict__ x, const T *__restrict__ ec,
                                                       long gsc, const T *__restrict__ bf, T *__restrict__ y,
                                                       long gsf, T omega) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   constexpr int NF = FULL ? (1 << D) - 1 : D;
   const int lane = threadIdx.x & 31;
@@ -960,6 +968,7 @@ __global__ void __launch_bounds__(NB) k_prolong_sweep(GridDesc gf, GridDesc gc, 
 template <typename T, int VW>
 __global__ void __launch_bounds__(256) k_coarse_apply(const T *__restrict__ inv, int nc, const T *__restrict__ R,
                                                       long gsr, T *__restrict__ E, long gse) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   extern __shared__ unsigned char smem_raw[];
   T *r = reinterpret_cast<T *>(smem_raw);
@@ -994,6 +1003,7 @@ __global__ void __launch_bounds__(256) k_coarse_apply(const T *__restrict__ inv,
 template <typename T, int VW>
 __global__ void __launch_bounds__(NB) k_jacobi0(long n, const T *__restrict__ invdiag, const T *__restrict__ B, long gs,
                                                 T *__restrict__ Y, T omega) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   const int grp = blockIdx.y;
   for (long i = blockIdx.x * (long)NB + threadIdx.x; i < n; i += (long)gridDim.x * NB) {
@@ -1010,6 +1020,7 @@ template <typename T, int VW>
 __global__ void __launch_bounds__(NB) k_cg_update(long n, long gs, const T *__restrict__ p, const T *__restrict__ q,
                                                   T *__restrict__ x, T *__restrict__ r,
                                                   const double *__restrict__ alpha, int s, Fin fin) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   const int grp = blockIdx.y;
   PK acc = PK::zero();
@@ -1042,6 +1053,7 @@ __global__ void __launch_bounds__(NB) k_cg_update_diag(long n, long gs, const T 
                                                        const T *__restrict__ invdiag,
                                                        const double *__restrict__ alpha, int s, double *part,
                                                        double *part2) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   const int grp = blockIdx.y;
   PK acc = PK::zero(), acc2 = PK::zero();
@@ -1072,6 +1084,7 @@ template <typename T, int VW>
 __global__ void __launch_bounds__(NB) k_p_update_diag(long n, long gs, const T *__restrict__ r,
                                                       const T *__restrict__ invdiag, T *__restrict__ p,
                                                       const double *__restrict__ beta) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   const int grp = blockIdx.y;
   T b[VW];
@@ -1092,6 +1105,7 @@ __global__ void __launch_bounds__(NB) k_p_update_diag(long n, long gs, const T *
 template <typename T, int VW>
 __global__ void __launch_bounds__(NB) k_dot_diag(long n, const T *__restrict__ invdiag, const T *__restrict__ R,
                                                  long gs, int s, double *part) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   const int grp = blockIdx.y;
   PK acc = PK::zero();
@@ -1107,6 +1121,7 @@ __global__ void __launch_bounds__(NB) k_dot_diag(long n, const T *__restrict__ i
 template <typename T, int VW>
 __global__ void __launch_bounds__(NB) k_p_update(long n, long gs, const T *__restrict__ z, T *__restrict__ p,
                                                  const double *__restrict__ beta) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   const int grp = blockIdx.y;
   T b[VW];
@@ -1126,6 +1141,7 @@ __global__ void __launch_bounds__(NB) k_p_update(long n, long gs, const T *__res
 template <typename T, int VW>
 __global__ void __launch_bounds__(NB) k_dot(long n, long gs, const T *__restrict__ a, const T *__restrict__ b, int s,
                                             Fin fin) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   const int grp = blockIdx.y;
   PK acc = PK::zero();
@@ -1151,6 +1167,7 @@ __device__ __forceinline__ double to64(double x) { return x; }
 template <typename T, int VW>
 __global__ void __launch_bounds__(NB) k_row_dot(GridDesc g, const T *__restrict__ a, const T *__restrict__ b, long gs,
                                                 int s, Fin fin) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   const int i0 = blockIdx.x * 32 + (threadIdx.x & 31), grp = blockIdx.z;
   const int nrows = g.dim == 2 ? g.np : g.np * g.np;
@@ -1169,6 +1186,7 @@ __global__ void __launch_bounds__(NB) k_row_dot(GridDesc g, const T *__restrict_
 template <typename T, int VW>
 __global__ void __launch_bounds__(NB) k_to_inner(long n, const double *__restrict__ R, long ldr,
                                                  const double *__restrict__ scale, int s, T *__restrict__ rt, long gs) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   const int grp = blockIdx.y;
   for (long i = blockIdx.x * (long)NB + threadIdx.x; i < n; i += (long)gridDim.x * NB) {
@@ -1190,6 +1208,7 @@ __global__ void __launch_bounds__(NB) k_to_inner_ctl(long n, const double *__res
                                                      const RefineCtl *__restrict__ ctl,
                                                      const double *__restrict__ scale, int s, T *__restrict__ rt,
                                                      long gs) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   const double *src = ctl->outer == 1 ? B0 : R;
   const int grp = blockIdx.y;
@@ -1214,6 +1233,7 @@ __global__ void k_refine_ctl(int s, const double *__restrict__ rr, const double 
                              double tol_in, double *__restrict__ scale, double *__restrict__ iscale,
                              double *__restrict__ tol2col, const int *__restrict__ pcg_iter, int after_body,
                              int max_outer, RefineCtl *ctl, cudaGraphConditionalHandle h) {
+  pdl_enter();
   __shared__ int nact_s, bad_s;
   __shared__ double worst_s[256];
   if (threadIdx.x == 0) nact_s = bad_s = 0;
@@ -1263,6 +1283,7 @@ __global__ void k_refine_ctl(int s, const double *__restrict__ rr, const double 
 template <typename T, int VW>
 __global__ void __launch_bounds__(NB) k_accum(long n, const T *__restrict__ d, long gs, const double *__restrict__ iscale,
                                               int s, double *__restrict__ X, long ldx) {
+  pdl_enter();
   using PK = Pack<T, VW>;
   const int grp = blockIdx.y;
   for (long i = blockIdx.x * (long)NB + threadIdx.x; i < n; i += (long)gridDim.x * NB) {
@@ -1504,6 +1525,7 @@ __global__ void __launch_bounds__(NB) k_df_out_dfp(const float4 *__restrict__ Xp
 // graph mode the decision drives the device-side while loop.
 __global__ void k_pcg_cond(const int *__restrict__ active, int s, int *iter, int maxit, int bump,
                            cudaGraphConditionalHandle h, int use_handle) {
+  pdl_enter();
   __shared__ int any;
   if (threadIdx.x == 0) any = 0;
   __syncthreads();
@@ -1532,6 +1554,7 @@ constexpr float CHEB_GAMMA = 2.f / 3.f, CHEB_RHO2 = 4.f / 9.f, CHEB_X0 = 0.4f;
 // step 0: number of steps; 1: one more step is done
 __global__ void k_cheb_ctl(const double *__restrict__ tol2col, int s, int maxit, int step, ChebCtl *ctl, int *active,
                            cudaGraphConditionalHandle h, int use_handle) {
+  pdl_enter();
   __shared__ float tmin[256];
   __shared__ int more_s;
   if (step == 0) {
@@ -1567,6 +1590,7 @@ __global__ void k_cheb_ctl(const double *__restrict__ tol2col, int s, int maxit,
 __global__ void __launch_bounds__(NB) k_cheb_start(long n, long gs, const float *__restrict__ r,
                                                    const float *__restrict__ invdiag, float *__restrict__ x,
                                                    float *__restrict__ p, const ChebCtl *__restrict__ ctl) {
+  pdl_enter();
   float *y = (ctl->n & 1) ? p : x;
   const long g0 = blockIdx.y * gs;
   for (long i = blockIdx.x * (long)NB + threadIdx.x; i < n; i += (long)gridDim.x * NB) {
@@ -1916,17 +1940,17 @@ static void st_launch(const GridDesc &g, const Stencil<T> &S, const T *X, long g
   const dim3 grid = rowgrid_capped(g, ng);
   if (g.dim == 2) {
     if (S.full)
-      k_st<T, VW, 2, true, MODE><<<grid, NB, 0, st>>>(g, S.diag, S.invdiag, S.c, X, gx, B, gb, Y, gy, s, omega,
+      pdl_launch(k_st<T, VW, 2, true, MODE>, grid, NB, 0, st, g, S.diag, S.invdiag, S.c, X, gx, B, gb, Y, gy, s, omega,
                                                      omega2, fin);
     else
-      k_st<T, VW, 2, false, MODE><<<grid, NB, 0, st>>>(g, S.diag, S.invdiag, S.c, X, gx, B, gb, Y, gy, s, omega,
+      pdl_launch(k_st<T, VW, 2, false, MODE>, grid, NB, 0, st, g, S.diag, S.invdiag, S.c, X, gx, B, gb, Y, gy, s, omega,
                                                      omega2, fin);
   } else {
     if (S.full)
-      k_st<T, VW, 3, true, MODE><<<grid, NB, 0, st>>>(g, S.diag, S.invdiag, S.c, X, gx, B, gb, Y, gy, s, omega,
+      pdl_launch(k_st<T, VW, 3, true, MODE>, grid, NB, 0, st, g, S.diag, S.invdiag, S.c, X, gx, B, gb, Y, gy, s, omega,
                                                      omega2, fin);
     else
-      k_st<T, VW, 3, false, MODE><<<grid, NB, 0, st>>>(g, S.diag, S.invdiag, S.c, X, gx, B, gb, Y, gy, s, omega,
+      pdl_launch(k_st<T, VW, 3, false, MODE>, grid, NB, 0, st, g, S.diag, S.invdiag, S.c, X, gx, B, gb, Y, gy, s, omega,
                                                      omega2, fin);
   }
   count_launch();
@@ -2202,7 +2226,7 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
   const int L = P->L;
   if (L == 1) {  // the coarse solve is the whole preconditioner; the caller forms <r, z>
     const int nc = (int)P->lv[0].g.n;
-    k_coarse_apply<T, VW><<<dim3((nc + 31) / 32, ng), 256, sizeof(T) * nc * VW, st>>>(coarse_inv<T>(P, op), nc, r0,
+    pdl_launch(k_coarse_apply<T, VW>, dim3((nc + 31) / 32, ng), 256, sizeof(T) * nc * VW, st, coarse_inv<T>(P, op), nc, r0,
                                                                                        gs0, z0, gs0);
     count_launch();
     count_bytes(BY_STENCILC, (double)sizeof(T) * ((double)nc * nc + 2.0 * nc * s));
@@ -2253,7 +2277,7 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
     if (nu >= 2) {
       st_launch<T, VW, M_JAC2>(g, S, rl[l], gsl[l], nullptr, 0, c, gsl[l], s, w[0], nofin, st, w[1]);
     } else {
-      k_jacobi0<T, VW><<<nodegrid(g.n, ng), NB, 0, st>>>(g.n, S.invdiag, rl[l], gsl[l], c, w[0]);
+      pdl_launch(k_jacobi0<T, VW>, nodegrid(g.n, ng), NB, 0, st, g.n, S.invdiag, rl[l], gsl[l], c, w[0]);
       count_launch();
       count_bytes(level_family(g.n), (double)sizeof(T) * (double)g.n * (2.0 * s + 1.0));
     }
@@ -2272,14 +2296,14 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
       const int zd = op == OP_K;
       if (g.dim == 2) {
         if (S.full)
-          k_resid_restrict<T, VW, 2, true><<<gr, NB, 0, st>>>(g, gc, S.diag, S.c, c, rl[l], gsl[l], rc, gsl[l + 1], zd);
+          pdl_launch(k_resid_restrict<T, VW, 2, true>, gr, NB, 0, st, g, gc, S.diag, S.c, c, rl[l], gsl[l], rc, gsl[l + 1], zd);
         else
-          k_resid_restrict<T, VW, 2, false><<<gr, NB, 0, st>>>(g, gc, S.diag, S.c, c, rl[l], gsl[l], rc, gsl[l + 1], zd);
+          pdl_launch(k_resid_restrict<T, VW, 2, false>, gr, NB, 0, st, g, gc, S.diag, S.c, c, rl[l], gsl[l], rc, gsl[l + 1], zd);
       } else {
         if (S.full)
-          k_resid_restrict<T, VW, 3, true><<<gr, NB, 0, st>>>(g, gc, S.diag, S.c, c, rl[l], gsl[l], rc, gsl[l + 1], zd);
+          pdl_launch(k_resid_restrict<T, VW, 3, true>, gr, NB, 0, st, g, gc, S.diag, S.c, c, rl[l], gsl[l], rc, gsl[l + 1], zd);
         else
-          k_resid_restrict<T, VW, 3, false><<<gr, NB, 0, st>>>(g, gc, S.diag, S.c, c, rl[l], gsl[l], rc, gsl[l + 1], zd);
+          pdl_launch(k_resid_restrict<T, VW, 3, false>, gr, NB, 0, st, g, gc, S.diag, S.c, c, rl[l], gsl[l], rc, gsl[l + 1], zd);
       }
       count_launch();
       count_bytes(BY_TRANSFER, (double)sizeof(T) * ((2.0 * s + 1.0 + S.nf) * (double)g.n + (double)s * gc.n));
@@ -2288,9 +2312,9 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
       st_launch<T, VW, M_RESID>(g, S, c, gsl[l], rl[l], gsl[l], o, gsl[l], s, om, nofin, st);
       prof_stop(P, pr);
       if (g.dim == 2)
-        k_restrict<T, VW, 2><<<flatgrid(gc, ng), NB, 0, st>>>(g, gc, o, gsl[l], rc, gsl[l + 1], op == OP_K);
+        pdl_launch(k_restrict<T, VW, 2>, flatgrid(gc, ng), NB, 0, st, g, gc, o, gsl[l], rc, gsl[l + 1], op == OP_K);
       else
-        k_restrict<T, VW, 3><<<flatgrid(gc, ng), NB, 0, st>>>(g, gc, o, gsl[l], rc, gsl[l + 1], op == OP_K);
+        pdl_launch(k_restrict<T, VW, 3>, flatgrid(gc, ng), NB, 0, st, g, gc, o, gsl[l], rc, gsl[l + 1], op == OP_K);
       count_launch();
       count_bytes(BY_TRANSFER, (double)sizeof(T) * s * ((double)g.n + (double)gc.n));
     }
@@ -2310,7 +2334,7 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
   } else {
     const int lc = L - 1;
     const int nc = (int)P->lv[lc].g.n;
-    k_coarse_apply<T, VW><<<dim3((nc + 31) / 32, ng), 256, sizeof(T) * nc * VW, st>>>(coarse_inv<T>(P, op), nc,
+    pdl_launch(k_coarse_apply<T, VW>, dim3((nc + 31) / 32, ng), 256, sizeof(T) * nc * VW, st, coarse_inv<T>(P, op), nc,
                                                                                        rl[lc], gsl[lc], ea[lc], gsl[lc]);
     count_launch();
     count_bytes(BY_STENCILC, (double)sizeof(T) * ((double)nc * nc + 2.0 * nc * s));
@@ -2340,7 +2364,7 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
           dot_finalize(fin, leg_tiles(g), s, st);
         } else if (l == 0) {
           const dim3 gr = rowgrid_capped(g, ng);
-          k_row_dot<T, VW><<<gr, NB, 0, st>>>(g, rl[0], cur[0], gsl[0], s, fin);
+          pdl_launch(k_row_dot<T, VW>, gr, NB, 0, st, g, rl[0], cur[0], gsl[0], s, fin);
           count_launch();
           count_bytes(BY_VECTOR, 8.0 * s * (double)g.n);
           dot_finalize(fin, gr.x * gr.y, s, st);
@@ -2355,17 +2379,17 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
       const T *ec = cur[l + 1];
       if (g.dim == 2) {
         if (S.full)
-          k_prolong_sweep<T, VW, 2, true><<<gr, NB, 0, st>>>(g, gc, S.diag, S.invdiag, S.c, c, ec, gsl[l + 1], rl[l],
+          pdl_launch(k_prolong_sweep<T, VW, 2, true>, gr, NB, 0, st, g, gc, S.diag, S.invdiag, S.c, c, ec, gsl[l + 1], rl[l],
                                                              o, gsl[l], w[nu - 1]);
         else
-          k_prolong_sweep<T, VW, 2, false><<<gr, NB, 0, st>>>(g, gc, S.diag, S.invdiag, S.c, c, ec, gsl[l + 1], rl[l],
+          pdl_launch(k_prolong_sweep<T, VW, 2, false>, gr, NB, 0, st, g, gc, S.diag, S.invdiag, S.c, c, ec, gsl[l + 1], rl[l],
                                                               o, gsl[l], w[nu - 1]);
       } else {
         if (S.full)
-          k_prolong_sweep<T, VW, 3, true><<<gr, NB, 0, st>>>(g, gc, S.diag, S.invdiag, S.c, c, ec, gsl[l + 1], rl[l],
+          pdl_launch(k_prolong_sweep<T, VW, 3, true>, gr, NB, 0, st, g, gc, S.diag, S.invdiag, S.c, c, ec, gsl[l + 1], rl[l],
                                                              o, gsl[l], w[nu - 1]);
         else
-          k_prolong_sweep<T, VW, 3, false><<<gr, NB, 0, st>>>(g, gc, S.diag, S.invdiag, S.c, c, ec, gsl[l + 1], rl[l],
+          pdl_launch(k_prolong_sweep<T, VW, 3, false>, gr, NB, 0, st, g, gc, S.diag, S.invdiag, S.c, c, ec, gsl[l + 1], rl[l],
                                                               o, gsl[l], w[nu - 1]);
       }
       count_launch();
@@ -2374,9 +2398,9 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
       k0 = 1;
     } else {
       if (g.dim == 2)
-        k_prolong_add<T, VW, 2><<<flatgrid(g, ng), NB, 0, st>>>(g, gc, cur[l + 1], gsl[l + 1], cur[l], gsl[l]);
+        pdl_launch(k_prolong_add<T, VW, 2>, flatgrid(g, ng), NB, 0, st, g, gc, cur[l + 1], gsl[l + 1], cur[l], gsl[l]);
       else
-        k_prolong_add<T, VW, 3><<<flatgrid(g, ng), NB, 0, st>>>(g, gc, cur[l + 1], gsl[l + 1], cur[l], gsl[l]);
+        pdl_launch(k_prolong_add<T, VW, 3>, flatgrid(g, ng), NB, 0, st, g, gc, cur[l + 1], gsl[l + 1], cur[l], gsl[l]);
       count_launch();
       count_bytes(BY_TRANSFER, (double)sizeof(T) * s * (2.0 * (double)g.n + (double)gc.n));
     }
@@ -2406,9 +2430,9 @@ static ChebCtl *cheb_ctl(hp_problem *P) {  // the iteration counter and the two 
 static void cheb_init(hp_problem *P, int s, cudaGraphConditionalHandle h, int use_handle, int maxit) {
   BlockWS<float> &W = P->w32;
   const int ng = (s + 3) / 4;
-  k_cheb_ctl<<<1, 256, 0, P->st>>>(P->sc.tol2col.as<double>(), s, maxit, 0, cheb_ctl(P), P->sc.active.as<int>(), h,
+  pdl_launch(k_cheb_ctl, 1, 256, 0, P->st, P->sc.tol2col.as<double>(), s, maxit, 0, cheb_ctl(P), P->sc.active.as<int>(), h,
                                    use_handle);
-  k_cheb_start<<<nodegrid(P->n, ng), NB, 0, P->st>>>(P->n, W.ldn * 4, W.r.as<float>(),
+  pdl_launch(k_cheb_start, nodegrid(P->n, ng), NB, 0, P->st, P->n, W.ldn * 4, W.r.as<float>(),
                                                      stencil_of<float>(P, OP_M, 0).invdiag, W.x.as<float>(),
                                                      W.p.as<float>(), cheb_ctl(P));
   count_launch(2);
@@ -2431,7 +2455,7 @@ static void cheb_step(hp_problem *P, int s, cudaGraphConditionalHandle h, int us
   a.ctl = cheb_ctl(P);
   launch_march(a, g, MA_CHEB, s, P->st);
   count_bytes(level_family(g.n), st_bytes<float, M_JACOBI>(g, S, s) + 4.0 * (double)g.n * s);
-  k_cheb_ctl<<<1, 256, 0, P->st>>>(P->sc.tol2col.as<double>(), s, maxit, 1, cheb_ctl(P), P->sc.active.as<int>(), h,
+  pdl_launch(k_cheb_ctl, 1, 256, 0, P->st, P->sc.tol2col.as<double>(), s, maxit, 1, cheb_ctl(P), P->sc.active.as<int>(), h,
                                    use_handle);
   count_launch();
 }
@@ -2448,17 +2472,17 @@ static void pcg_init(hp_problem *P, OpKind op, int s, cudaGraphConditionalHandle
   cudaMemsetAsync(P->sc.iter.p, 0, sizeof(int), st);
   T *r = W.r.template as<T>();
   const dim3 gr = nodegrid(P->n, ng);
-  k_dot<T, VW><<<gr, NB, 0, st>>>(P->n, gs, r, r, s, make_fin(P, FIN_INIT));
+  pdl_launch(k_dot<T, VW>, gr, NB, 0, st, P->n, gs, r, r, s, make_fin(P, FIN_INIT));
   dot_finalize(make_fin(P, FIN_INIT), gr.x, s, st);
   count_bytes(BY_VECTOR, (double)sizeof(T) * (double)P->n * s);
   if (op == OP_M) {  // <r, z> of the first iteration, where beta is 0 (the counter is at 0)
     const Fin fin = make_fin(P, FIN_BETA);
-    k_dot_diag<T, VW><<<gr, NB, 0, st>>>(P->n, stencil_of<T>(P, op, 0).invdiag, r, gs, s, fin.part);
+    pdl_launch(k_dot_diag<T, VW>, gr, NB, 0, st, P->n, stencil_of<T>(P, op, 0).invdiag, r, gs, s, fin.part);
     count_launch();
     count_bytes(BY_VECTOR, (double)sizeof(T) * (double)P->n * (s + 1.0));
     dot_finalize(fin, gr.x, s, st);
   }
-  k_pcg_cond<<<1, 256, 0, st>>>(P->sc.active.as<int>(), s, P->sc.iter.as<int>(), maxit, 0, h, use_handle);
+  pdl_launch(k_pcg_cond, 1, 256, 0, st, P->sc.active.as<int>(), s, P->sc.iter.as<int>(), maxit, 0, h, use_handle);
   count_launch(2);
 }
 
@@ -2494,18 +2518,18 @@ static void pcg_body(hp_problem *P, OpKind op, int s, double tol2, cudaGraphCond
   const Stencil<T> &S0 = stencil_of<T>(P, op, 0);
   int pr = -1;
   if (op == OP_M) {
-    k_p_update_diag<T, VW><<<nodegrid(n, ng), NB, 0, st>>>(n, gs, r, S0.invdiag, p, P->sc.beta.as<double>());
+    pdl_launch(k_p_update_diag<T, VW>, nodegrid(n, ng), NB, 0, st, n, gs, r, S0.invdiag, p, P->sc.beta.as<double>());
     count_launch();
     count_bytes(BY_VECTOR, (double)sizeof(T) * (double)n * (3.0 * s + 1.0));
     st_launch<T, VW, M_APPLY_DOT>(g0, S0, p, gs, nullptr, 0, q, gs, s, T(0), make_fin(P, FIN_ALPHA), st);
     const dim3 gu = nodegrid(n, ng);
     const Fin frr = make_fin(P, FIN_RR, tol2), fbeta = make_fin(P, FIN_BETA_NEXT);
     double *part2 = frr.part + (long)gu.x * round4(s);
-    k_cg_update_diag<T, VW><<<gu, NB, 0, st>>>(n, gs, p, q, x, r, S0.invdiag, P->sc.alpha.as<double>(), s, frr.part,
+    pdl_launch(k_cg_update_diag<T, VW>, gu, NB, 0, st, n, gs, p, q, x, r, S0.invdiag, P->sc.alpha.as<double>(), s, frr.part,
                                                part2);
-    k_dot_finalize2<<<s, NB, 0, st>>>(frr.part, part2, gu.x, frr, fbeta);
+    pdl_launch(k_dot_finalize2, s, NB, 0, st, frr.part, part2, gu.x, frr, fbeta);
     count_bytes(BY_VECTOR, (double)sizeof(T) * (double)n * (6.0 * s + 1.0));
-    k_pcg_cond<<<1, 256, 0, st>>>(P->sc.active.as<int>(), s, P->sc.iter.as<int>(), maxit, 1, h, use_handle);
+    pdl_launch(k_pcg_cond, 1, 256, 0, st, P->sc.active.as<int>(), s, P->sc.iter.as<int>(), maxit, 1, h, use_handle);
     count_launch(3);
     return;
   }
@@ -2514,12 +2538,12 @@ static void pcg_body(hp_problem *P, OpKind op, int s, double tol2, cudaGraphCond
   prof_stop(P, pr);
   if (P->L == 1) {
     const dim3 gr = nodegrid(n, ng);
-    k_dot<T, VW><<<gr, NB, 0, st>>>(n, gs, r, z, s, make_fin(P, FIN_BETA));
+    pdl_launch(k_dot<T, VW>, gr, NB, 0, st, n, gs, r, z, s, make_fin(P, FIN_BETA));
     count_launch();
     count_bytes(BY_VECTOR, (double)sizeof(T) * (double)n * 2.0 * s);
     dot_finalize(make_fin(P, FIN_BETA), gr.x, s, st);
   }
-  k_p_update<T, VW><<<nodegrid(n, ng), NB, 0, st>>>(n, gs, z, p, P->sc.beta.as<double>());
+  pdl_launch(k_p_update<T, VW>, nodegrid(n, ng), NB, 0, st, n, gs, z, p, P->sc.beta.as<double>());
   count_launch();
   count_bytes(BY_VECTOR, (double)sizeof(T) * (double)n * 3.0 * s);
   pr = prof_start(P, PROF_MATVEC);
@@ -2527,11 +2551,11 @@ static void pcg_body(hp_problem *P, OpKind op, int s, double tol2, cudaGraphCond
   prof_stop(P, pr);
   pr = prof_start(P, PROF_CG_UPDATE);
   const dim3 gu = nodegrid(n, ng);
-  k_cg_update<T, VW><<<gu, NB, 0, st>>>(n, gs, p, q, x, r, P->sc.alpha.as<double>(), s, make_fin(P, FIN_RR, tol2));
+  pdl_launch(k_cg_update<T, VW>, gu, NB, 0, st, n, gs, p, q, x, r, P->sc.alpha.as<double>(), s, make_fin(P, FIN_RR, tol2));
   dot_finalize(make_fin(P, FIN_RR, tol2), gu.x, s, st);
   count_bytes(BY_VECTOR, (double)sizeof(T) * (double)n * 6.0 * s);
   prof_stop(P, pr);
-  k_pcg_cond<<<1, 256, 0, st>>>(P->sc.active.as<int>(), s, P->sc.iter.as<int>(), maxit, 1, h, use_handle);
+  pdl_launch(k_pcg_cond, 1, 256, 0, st, P->sc.active.as<int>(), s, P->sc.iter.as<int>(), maxit, 1, h, use_handle);
   count_launch(2);
 }
 
@@ -2740,7 +2764,7 @@ static unsigned launch_st64(hp_problem *P, OpKind op, const double *X, long ldx,
   // about four rounds of the resident blocks, so that their last round costs little
   const long cap = std::max<long>(1, 64l * NSM / ng);
   const dim3 gr((unsigned)std::min<long>((g.n + NB - 1) / NB, cap), ng);
-  auto go = [&](auto k) { k<<<gr, NB, 0, P->st>>>(g, S.diag, S.c, X, ldx, B, ldb, Y, ldy, s, part); };
+  auto go = [&](auto k) { pdl_launch(k, gr, NB, 0, P->st, g, S.diag, S.c, X, ldx, B, ldb, Y, ldy, s, part); };
   if (g.dim == 2) {
     if (S.full) go(k_st64<2, true, RESID>);
     else go(k_st64<2, false, RESID>);
@@ -2829,7 +2853,7 @@ static int build_solve_graph(hp_problem *P, OpKind op, int s, double rtol, doubl
     if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(cs, g, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
     if (e == cudaSuccess) {
       cudaMemsetAsync(ctl, 0, sizeof(RefineCtl), cs);
-      k_refine_ctl<<<1, 256, 0, cs>>>(s, rr, bb, rtol, tol_in, scale, iscale, tol2col, iter, 0, max_outer, ctl, ho);
+      pdl_launch(k_refine_ctl, 1, 256, 0, cs, s, rr, bb, rtol, tol_in, scale, iscale, tol2col, iter, 0, max_outer, ctl, ho);
       e = end_capture(g, true);
     }
     if (e == cudaSuccess) {
@@ -2843,16 +2867,16 @@ static int build_solve_graph(hp_problem *P, OpKind op, int s, double rtol, doubl
     }
     if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(cs, body, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
     if (e == cudaSuccess) {
-      k_to_inner_ctl<T, VW><<<nodegrid(n, ng), NB, 0, cs>>>(n, b64, r64, ld64, ctl, scale, s, W.r.template as<T>(),
+      pdl_launch(k_to_inner_ctl<T, VW>, nodegrid(n, ng), NB, 0, cs, n, b64, r64, ld64, ctl, scale, s, W.r.template as<T>(),
                                                             gs);
       e = end_capture(body, true);
     }
     if (e == cudaSuccess) e = append_pcg<T, VW>(P, op, s, tol_in, maxit, body, leaf, &pw);
     if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(cs, body, &pw, nullptr, 1, cudaStreamCaptureModeRelaxed);
     if (e == cudaSuccess) {
-      k_accum<T, VW><<<nodegrid(n, ng), NB, 0, cs>>>(n, W.x.template as<T>(), gs, iscale, s, x64, ld64);
+      pdl_launch(k_accum<T, VW>, nodegrid(n, ng), NB, 0, cs, n, W.x.template as<T>(), gs, iscale, s, x64, ld64);
       const int rc = residual64(P, op, b64, ld64, x64, ld64, r64, ld64, s);
-      k_refine_ctl<<<1, 256, 0, cs>>>(s, rr, bb, rtol, tol_in, scale, iscale, tol2col, iter, 1, max_outer, ctl, ho);
+      pdl_launch(k_refine_ctl, 1, 256, 0, cs, s, rr, bb, rtol, tol_in, scale, iscale, tol2col, iter, 1, max_outer, ctl, ho);
       e = end_capture(body, false);
       if (e == cudaSuccess && rc) e = cudaErrorUnknown;
     }
@@ -2999,7 +3023,7 @@ static int build_solve_graph_dfp(hp_problem *P, OpKind op, int s, double rtol, d
     if (e == cudaSuccess) e = cudaStreamBeginCaptureToGraph(cs, g, nullptr, nullptr, 0, cudaStreamCaptureModeRelaxed);
     if (e == cudaSuccess) {
       cudaMemsetAsync(ctl, 0, sizeof(RefineCtl), cs);
-      k_refine_ctl<<<1, 256, 0, cs>>>(s, rr, bb, rtol, tol_in, scale, iscale, tol2col, iter, 0, max_outer, ctl, ho);
+      pdl_launch(k_refine_ctl, 1, 256, 0, cs, s, rr, bb, rtol, tol_in, scale, iscale, tol2col, iter, 0, max_outer, ctl, ho);
       launch_first_inner_dfp(P, Bp, ldp, s, rt, gs);
       const cudaError_t el = capture_leaf(cs, &leaf);
       cudaGraph_t gg = g;
@@ -3020,7 +3044,7 @@ static int build_solve_graph_dfp(hp_problem *P, OpKind op, int s, double rtol, d
     if (e == cudaSuccess) {
       launch_accum_dfp(P, d, gs, s, Xp, ldp);
       launch_resid_dfp(P, op, Xp, Bp, ldp, rt, gs, s, bb);
-      k_refine_ctl<<<1, 256, 0, cs>>>(s, rr, bb, rtol, tol_in, scale, iscale, tol2col, iter, 1, max_outer, ctl, ho);
+      pdl_launch(k_refine_ctl, 1, 256, 0, cs, s, rr, bb, rtol, tol_in, scale, iscale, tol2col, iter, 1, max_outer, ctl, ho);
       cudaGraph_t bg = body;
       e = cudaStreamEndCapture(cs, &bg);
     }
@@ -3235,7 +3259,7 @@ static int ir_solve(hp_problem *P, OpKind op, const double *B, long ldb, double 
     HP_CUDA(cudaMemcpyAsync(P->sc.tol2col.p, htol2.data(), sizeof(double) * s, cudaMemcpyHostToDevice, st));
     // the first residual of a solve from zero is b64 (r64 not yet written)
     const double *rsrc = (outer == 0 && !warm) ? b64 : r64;
-    k_to_inner<T, VW><<<nodegrid(n, ng), NB, 0, st>>>(n, rsrc, ld64, P->sc.scale.as<double>(), s,
+    pdl_launch(k_to_inner<T, VW>, nodegrid(n, ng), NB, 0, st, n, rsrc, ld64, P->sc.scale.as<double>(), s,
                                                       W.r.template as<T>(), gs);
     count_launch();
     count_bytes(BY_REFINE, (8.0 + sizeof(T)) * (double)n * s);  // read the FP64 residual, write the inner one
@@ -3245,7 +3269,7 @@ static int ir_solve(hp_problem *P, OpKind op, const double *B, long ldb, double 
     if (prc && prc != HP_ERR_NOT_CONVERGED) return prc;
     total_its += its;
     prof_spin(P);
-    k_accum<T, VW><<<nodegrid(n, ng), NB, 0, st>>>(n, W.x.template as<T>(), gs, P->sc.iscale.as<double>(), s, X,
+    pdl_launch(k_accum<T, VW>, nodegrid(n, ng), NB, 0, st, n, W.x.template as<T>(), gs, P->sc.iscale.as<double>(), s, X,
                                                    ldx);
     count_launch();
     count_bytes(BY_REFINE, (16.0 + sizeof(T)) * (double)n * s);  // read the correction, read and write x
