@@ -167,10 +167,13 @@ __global__ void __launch_bounds__(256) k_conv_fwd(ConvIn I, const __nv_bfloat16 
 // stages: a slab's loads to registers are under way while the MMAs of the slab before start;
 // a stage is refilled once the tcgen05.commit of the MMAs that read it has arrived on
 // its mbarrier.
-// Bound: latency and issue of the staging (load, split into terms, store), not the tensor cores
-// (8 % busy) or memory; so two threads per accumulator row, of up to 64 registers (four CTAs per
-// SM), an item's place computed once per tile, two values per conversion, weights by
-// asynchronous copies.  The forward pass of 60 images of 264 x 264: 4.23 -> 2.93 ms.
+// Bound: the MMAs.  With few output channels an MMA's time is the reading of its 128 pixels (4 KB)
+// from shared memory, not its arithmetic: 63 clocks each in the 16-channel layers, of which
+// the read takes 32 or more, 87 with 32 and 64 channels.  With one thread per accumulator row, 16
+// warps per SM, the staging (load, split into terms, store) was exposed beside them: hence two
+// threads per row of up to 64 registers (four CTAs per SM), an item's place computed once per
+// tile, two values per conversion, weights by asynchronous copies.  The forward pass of 60
+// images of 264 x 264: 4.23 -> 2.92 ms (MMAs at 32 clocks: 1.2 ms).
 // ---------------------------------------------------------------------------
 constexpr int TC_NT = 256;   // threads per CTA: two per accumulator row (tensor-memory lane)
 constexpr int TC_TR = 16;    // tile rows
@@ -195,7 +198,7 @@ struct TcArgs {
   int cin;             // input channels (I.c1 + I.c2)
   const uint4 *w;      // packed weights, one slab after another
   const float *bias;   // co values, or null
-  float *out;          // (N, co, H, W)
+  float *out;          // (N, co, H, W), or null (the head only)
   int co, H, W, relu;
   int tx, ntx;         // MMAs per tile (8-column strips), tiles per image row
   int cs;              // tensor-memory columns between the strips' accumulators
@@ -357,7 +360,7 @@ __global__ void __launch_bounds__(TC_NT, 4) k_conv_tc(TcArgs a) {
           const float bi = (i & 3) == 0 ? b4.x : (i & 3) == 1 ? b4.y : (i & 3) == 2 ? b4.z : b4.w;
           float z = v[i] + bi;
           if (a.relu) z = fmaxf(z, 0.f);
-          o[(long)(c0 + i) * HW] = z;
+          if (a.out) o[(long)(c0 + i) * HW] = z;
           if (a.hout) head = fmaf(__bfloat162float(a.hw[c0 + i]), z, head);
         }
       }
@@ -884,10 +887,13 @@ static ConvIn cin(const float *a, int c, int up = 0, const float *b = nullptr, i
   return ConvIn{a, c, up, b, cb};
 }
 
-static void unet_forward(hp_unet *U, int N) {
+// y = net(x) for N images; keep: every layer's output is stored, as the backward pass reads them
+// (without it the last hidden layer's 16 channels, a tenth of the traffic, stay in the kernel
+// that also forms y)
+static void unet_forward(hp_unet *U, int N, const float *x, float *y, bool keep) {
   const int H = U->H, W = U->W;
   const int h[4] = {H, H / 2, H / 4, H / 8}, w[4] = {W, W / 2, W / 4, W / 8};
-  conv_fwd(U, 0, cin(U->x, 3), U->a[0], N, h[0], w[0], 1);
+  conv_fwd(U, 0, cin(x, 3), U->a[0], N, h[0], w[0], 1);
   conv_fwd(U, 1, cin(U->a[0], 16), U->a[1], N, h[0], w[0], 1);
   k_pool<<<gblocks((long)N * 16 * h[1] * w[1]), 256, 0, U->st>>>(U->a[1], U->pl[0], (long)N * 16, h[0], w[0]);
   conv_fwd(U, 2, cin(U->pl[0], 16), U->a[2], N, h[1], w[1], 1);
@@ -906,11 +912,11 @@ static void unet_forward(hp_unet *U, int N) {
   if (use_tc(U, 13)) {
     // dec1b with the 1x1 output layer folded into its epilogue
     const ULayer &L = U->L[13], &O = U->L[14];
-    conv_tc(U, cin(U->a[12], 16), L.ci, U->wtc + U->tc_fo[13], U->p32 + L.boff, U->a[13], L.co, N, h[0], w[0], 1,
-            U->w16 + O.woff, U->p32 + O.boff, U->a[14]);
+    conv_tc(U, cin(U->a[12], 16), L.ci, U->wtc + U->tc_fo[13], U->p32 + L.boff, keep ? U->a[13] : nullptr, L.co, N,
+            h[0], w[0], 1, U->w16 + O.woff, U->p32 + O.boff, y);
   } else {
     conv_fwd(U, 13, cin(U->a[12], 16), U->a[13], N, h[0], w[0], 1);
-    conv_fwd(U, 14, cin(U->a[13], 16), U->a[14], N, h[0], w[0], 0);
+    conv_fwd(U, 14, cin(U->a[13], 16), y, N, h[0], w[0], 0);
   }
   count_launch(3);
 }
@@ -1036,7 +1042,7 @@ static int tc_status() {
 void unet_run(hp_unet *U, int N, cudaStream_t st) {
   cudaStream_t own = U->st;
   U->st = st;
-  unet_forward(U, N);
+  unet_forward(U, N, U->x, U->a[14], false);
   U->st = own;
 }
 
@@ -1160,10 +1166,7 @@ int hp_unet_get_params(const hp_unet *U, float *params_host) {
 // y (N,1,H,W) = net(x (N,3,H,W)); device pointers, N <= cap
 int hp_unet_forward(hp_unet *U, const float *x_dev, int N, float *y_dev) {
   if (!U || !x_dev || !y_dev || N < 1 || N > U->cap) return set_error(HP_ERR_INVALID, "hp_unet_forward: arguments");
-  const long HW = (long)U->H * U->W;
-  HP_CUDA(cudaMemcpyAsync(U->x, x_dev, sizeof(float) * N * 3 * HW, cudaMemcpyDeviceToDevice, U->st));
-  unet_forward(U, N);
-  HP_CUDA(cudaMemcpyAsync(y_dev, U->a[14], sizeof(float) * N * HW, cudaMemcpyDeviceToDevice, U->st));
+  unet_forward(U, N, x_dev, y_dev, false);
   HP_CUDA(cudaStreamSynchronize(U->st));
   HP_CUDA(cudaGetLastError());
   return tc_status();
@@ -1174,7 +1177,7 @@ static int unet_grad(hp_unet *U, const float *x, const float *aux, int N, double
   const long HW = (long)U->H * U->W;
   HP_CUDA(cudaMemcpyAsync(U->x, x, sizeof(float) * N * 3 * HW, cudaMemcpyDeviceToDevice, U->st));
   HP_CUDA(cudaMemcpyAsync(U->aux, aux, sizeof(float) * N * 4 * HW, cudaMemcpyDeviceToDevice, U->st));
-  unet_forward(U, N);
+  unet_forward(U, N, U->x, U->a[14], true);
   const long cnt = (long)N * HW;
   const int nb = gblocks(cnt);
   double *wts = U->lossbuf, *part = U->lossbuf + 64;
