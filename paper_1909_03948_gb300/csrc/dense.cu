@@ -18,6 +18,7 @@
 #include <algorithm>
 #include <atomic>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "dfloat.cuh"
@@ -64,6 +65,8 @@ __global__ void k_gram_partial(const double *__restrict__ X, long ldx, int s1, c
 // diagonal are formed; k_gram_final mirrors the others.  The compensated sum over a chunk
 // is more accurate than FP64 accumulation of the same products (about 2^-48 of the result
 // plus n 2^-96 of the terms' magnitudes).
+// The next rows are under way while the current ones are multiplied, and a warp leaves out the
+// columns beyond s1: 65^3 rows, 100 x 64: 1,750 -> 1,300 us (FP32 pipe: 613 us).
 __global__ void k_gram_partial_df(const double *__restrict__ X, long ldx, int s1, const double *__restrict__ Y,
                                   long ldy, int s2, long n, long rows_per_chunk, int sym, double *__restrict__ part) {
   __shared__ float2 xs[GT][GT + 1], ys[GT][GT + 1];
@@ -72,25 +75,42 @@ __global__ void k_gram_partial_df(const double *__restrict__ X, long ldx, int s1
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;  // 32 x 8
   const long r0 = ch * rows_per_chunk, r1 = std::min<long>(n, r0 + rows_per_chunk);
   Dot2 acc[4];
-  for (long rb = r0; rb < r1; rb += GT) {
-    for (int k = ty; k < GT; k += 8) {
-      const long row = rb + tx;
-      const int ca = ta * GT + k, cb = tb * GT + k;
-      const dfl a = d2df((row < r1 && ca < s1) ? X[ldx * ca + row] : 0.0);
-      const dfl b = d2df((row < r1 && cb < s2) ? Y[ldy * cb + row] : 0.0);
-      xs[k][tx] = make_float2(a.hi, a.lo);
-      ys[k][tx] = make_float2(b.hi, b.lo);
+  double xd[4], yd[4];
+  auto fetch = [&](long rb) {
+    const long row = rb + tx;
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const int ca = ta * GT + ty + 8 * q, cb = tb * GT + ty + 8 * q;
+      xd[q] = (row < r1 && ca < s1) ? X[ldx * ca + row] : 0.0;
+      yd[q] = (row < r1 && cb < s2) ? Y[ldy * cb + row] : 0.0;
     }
-    __syncthreads();
+  };
+  auto rows = [&](auto nq) {  // the first nq of this warp's four columns of X
 #pragma unroll 4
     for (int rr = 0; rr < GT; ++rr) {
       const float2 yv = ys[tx][rr];
 #pragma unroll
-      for (int q = 0; q < 4; ++q) {
+      for (int q = 0; q < decltype(nq)::value; ++q) {
         const float2 xv = xs[ty + 8 * q][rr];
         acc[q].fma(dfl{xv.x, xv.y}, dfl{yv.x, yv.y});
       }
     }
+  };
+  const int cols = (s1 - ta * GT - ty + 7) / 8;  // of this warp, at most 4 here
+  fetch(r0);
+  for (long rb = r0; rb < r1; rb += GT) {
+#pragma unroll
+    for (int q = 0; q < 4; ++q) {
+      const dfl a = d2df(xd[q]), b = d2df(yd[q]);
+      xs[ty + 8 * q][tx] = make_float2(a.hi, a.lo);
+      ys[ty + 8 * q][tx] = make_float2(b.hi, b.lo);
+    }
+    __syncthreads();
+    if (rb + GT < r1) fetch(rb + GT);
+    if (cols >= 4) rows(std::integral_constant<int, 4>{});
+    else if (cols == 3) rows(std::integral_constant<int, 3>{});
+    else if (cols == 2) rows(std::integral_constant<int, 2>{});
+    else if (cols == 1) rows(std::integral_constant<int, 1>{});
     __syncthreads();
   }
   const int nta = gridDim.x, ntb = gridDim.y;
@@ -112,6 +132,7 @@ __global__ void k_gram_final(const double *__restrict__ part, int nchunk, int nt
   }
   const int ta = a / GT, tb = b / GT;
   double s = 0.0;
+#pragma unroll 8
   for (int c = 0; c < nchunk; ++c) s += part[(((long)c * nta + ta) * ntb + tb) * GT * GT + (a % GT) * GT + (b % GT)];
   G[idx % s1 + (long)ldg * (idx / s1)] = s;
 }
@@ -169,7 +190,10 @@ int gram(hp_problem *P, const double *X, long ldx, int s1, const double *Y, long
     return cuda_check(cudaGetLastError(), "gram");
   }
   const int nta = (s1 + GT - 1) / GT, ntb = (s2 + GT - 1) / GT;
-  int nchunk = std::max(1, (2 * NSM) / (nta * ntb));
+  const bool df = P->refine_df != 0;  // the Gram in double-float (see k_gram_partial_df)
+  const int sym = df && X == Y && ldx == ldy && s1 == s2;
+  // two CTAs per SM over the tiles that are computed
+  int nchunk = std::max(1, (2 * NSM) / (sym ? nta * (nta + 1) / 2 : nta * ntb));
   long rpc = (n + nchunk - 1) / nchunk;
   rpc = (rpc + GT - 1) / GT * GT;
   nchunk = (int)((n + rpc - 1) / rpc);
@@ -177,8 +201,6 @@ int gram(hp_problem *P, const double *X, long ldx, int s1, const double *Y, long
   const size_t need = sizeof(double) * (size_t)nchunk * nta * ntb * GT * GT;
   HP_TRY(P->vtmp[5].ensure(need));
   double *part = P->vtmp[5].as<double>();
-  const bool df = P->refine_df != 0;  // the Gram in double-float (see k_gram_partial_df)
-  const int sym = df && X == Y && ldx == ldy && s1 == s2;
   if (df)
     k_gram_partial_df<<<dim3(nta, ntb, nchunk), 256, 0, P->st>>>(X, ldx, s1, Y, ldy, s2, n, rpc, sym, part);
   else
@@ -199,33 +221,49 @@ __global__ void k_gemm_nn(const double *__restrict__ X, long ldx, int s1, const 
   }
 }
 
-// The same product in double-float on the FP32 pipe: each thread forms 8 output columns of
-// its row as compensated (Dot2) sums, so every element of X is split into a pair once per 8
-// columns instead of read and multiplied in FP64 for each; S's entries are split as they
-// are used (from L1).  alpha and beta are applied in FP64 once per output.
-constexpr int GM_NJ = 8;
-__global__ void k_gemm_nn_df(const double *__restrict__ X, long ldx, int s1, const double *__restrict__ S, int lds,
-                             int s2, double *__restrict__ Y, long ldy, long n, double alpha, double beta) {
-  extern __shared__ float2 sp[];  // the block's 8 columns of S as pairs, [k][q]
-  const int j0 = blockIdx.y * GM_NJ;
-  for (int t = threadIdx.x; t < s1 * GM_NJ; t += blockDim.x) {
-    const int k = t / GM_NJ, q = t % GM_NJ;
+// The same product in double-float on the FP32 pipe: each thread forms NJ output columns of
+// its row as compensated (Dot2) sums, so every element of X is split into a pair once per NJ
+// columns instead of read and multiplied in FP64 for each; the pairs of S's columns lie in
+// shared memory, two to a load.  alpha and beta are applied in FP64 once per output.
+// Bound by the FP32 pipe: 13 operations per term.  65^3 rows, 100 x 64: 1,126 -> 902 us with 16
+// columns instead of 8 and four elements of X under way (613 us for the operations alone).
+constexpr int GM_NJ = 8, GM_NJ2 = 16;
+template <int NJ>
+__global__ void __launch_bounds__(NT) k_gemm_nn_df(const double *__restrict__ X, long ldx, int s1,
+                                                   const double *__restrict__ S, int lds, int s2,
+                                                   double *__restrict__ Y, long ldy, long n, double alpha,
+                                                   double beta) {
+  extern __shared__ __align__(16) float2 sp[];  // the block's NJ columns of S as pairs, [k][q]
+  const int j0 = blockIdx.y * NJ;
+  for (int t = threadIdx.x; t < s1 * NJ; t += blockDim.x) {
+    const int k = t / NJ, q = t % NJ;
     const dfl d = d2df(j0 + q < s2 ? S[k + (long)lds * (j0 + q)] : 0.0);
     sp[t] = make_float2(d.hi, d.lo);
   }
   __syncthreads();
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
-    Dot2 acc[GM_NJ];
-    for (int k = 0; k < s1; ++k) {
-      const dfl x = d2df(X[ldx * k + i]);
+    Dot2 acc[NJ];
+    auto term = [&](int k, double xk) {
+      const dfl x = d2df(xk);
+      const float4 *sk = reinterpret_cast<const float4 *>(sp + k * NJ);
 #pragma unroll
-      for (int q = 0; q < GM_NJ; ++q) {
-        const float2 sv = sp[k * GM_NJ + q];
+      for (int q = 0; q < NJ; q += 2) {
+        const float4 sv = sk[q / 2];
         acc[q].fma(dfl{sv.x, sv.y}, x);
+        acc[q + 1].fma(dfl{sv.z, sv.w}, x);
       }
-    }
+    };
+    int k = 0;
+    for (; k + 4 <= s1; k += 4) {
+      double x[4];
 #pragma unroll
-    for (int q = 0; q < GM_NJ; ++q) {
+      for (int e = 0; e < 4; ++e) x[e] = X[ldx * (k + e) + i];
+#pragma unroll
+      for (int e = 0; e < 4; ++e) term(k + e, x[e]);
+    }
+    for (; k < s1; ++k) term(k, X[ldx * k + i]);
+#pragma unroll
+    for (int q = 0; q < NJ; ++q) {
       const int j = j0 + q;
       if (j >= s2) break;
       const double y = beta == 0.0 ? 0.0 : beta * Y[ldy * j + i];
@@ -262,9 +300,15 @@ __global__ void __launch_bounds__(128) k_tri_inv(const double *__restrict__ R, i
 void launch_gemm_nn(const double *X, long ldx, int s1, const double *S, int lds, int s2, double *Y, long ldy, long n,
                     double alpha, double beta, hp_problem *P) {
   if (P->refine_df != 0 && s2 > 1 && sizeof(float2) * (size_t)s1 * GM_NJ <= 48 * 1024) {
-    const int nj = (s2 + GM_NJ - 1) / GM_NJ;
-    k_gemm_nn_df<<<dim3(blocks_for(n, nj), nj), NT, sizeof(float2) * (size_t)s1 * GM_NJ, P->st>>>(
-        X, ldx, s1, S, lds, s2, Y, ldy, n, alpha, beta);
+    // 16 columns per thread where more than half of the last 16 are there and they fit
+    const size_t shm = sizeof(float2) * (size_t)s1 * GM_NJ2;
+    const int nj2 = (s2 + GM_NJ2 - 1) / GM_NJ2, nj = (s2 + GM_NJ - 1) / GM_NJ;
+    if (nj == 2 * nj2 && shm <= 48 * 1024)
+      k_gemm_nn_df<GM_NJ2><<<dim3(blocks_for(n, nj2), nj2), NT, shm, P->st>>>(X, ldx, s1, S, lds, s2, Y, ldy, n, alpha,
+                                                                             beta);
+    else
+      k_gemm_nn_df<GM_NJ><<<dim3(blocks_for(n, nj), nj), NT, sizeof(float2) * (size_t)s1 * GM_NJ, P->st>>>(
+          X, ldx, s1, S, lds, s2, Y, ldy, n, alpha, beta);
   } else {
     k_gemm_nn<<<dim3(blocks_for(n, s2), s2), NT, 0, P->st>>>(X, ldx, s1, S, lds, s2, Y, ldy, n, alpha, beta);
   }
