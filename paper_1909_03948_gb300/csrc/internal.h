@@ -375,6 +375,8 @@ int launch_leg(LegArgs a, const GridDesc &g, bool full, bool up, int vw, int s, 
 // pdl_enter() in all its threads.  A solve is a chain of hundreds of launches of a few us: one
 // column on 257^2 nodes 1.76 -> 1.70 ms, a 3D block of 24^3 cells' full Hessian 3.71 -> 3.49 ms,
 // a gradient on 257^2 nodes 4.17 -> 3.97 ms.
+// Not for kernels of very many short CTAs: the wait costs each of them some hundred clocks
+// (k_prolong_add, 64,000 CTAs of one node per thread: 44 -> 72 us).
 template <class... P, class... A>
 inline void pdl_launch(void (*k)(P...), dim3 grid, dim3 block, size_t shm, cudaStream_t st, A &&...args) {
   cudaLaunchAttribute at{};

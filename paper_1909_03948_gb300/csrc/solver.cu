@@ -788,7 +788,6 @@ __global__ void __launch_bounds__(NB) k_restrict(GridDesc gf, GridDesc gc, const
 template <typename T, int VW, int D>
 __global__ void __launch_bounds__(NB) k_prolong_add(GridDesc gf, GridDesc gc, const T *__restrict__ ec, long gsc,
                                                     T *__restrict__ ef, long gsf) {
-  pdl_enter();
   using PK = Pack<T, VW>;
   // one fine node per thread over the flattened grid (every lane busy whatever np is)
   const unsigned i = blockIdx.x * NB + threadIdx.x;
@@ -2398,9 +2397,9 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
       k0 = 1;
     } else {
       if (g.dim == 2)
-        pdl_launch(k_prolong_add<T, VW, 2>, flatgrid(g, ng), NB, 0, st, g, gc, cur[l + 1], gsl[l + 1], cur[l], gsl[l]);
+        k_prolong_add<T, VW, 2><<<flatgrid(g, ng), NB, 0, st>>>(g, gc, cur[l + 1], gsl[l + 1], cur[l], gsl[l]);
       else
-        pdl_launch(k_prolong_add<T, VW, 3>, flatgrid(g, ng), NB, 0, st, g, gc, cur[l + 1], gsl[l + 1], cur[l], gsl[l]);
+        k_prolong_add<T, VW, 3><<<flatgrid(g, ng), NB, 0, st>>>(g, gc, cur[l + 1], gsl[l + 1], cur[l], gsl[l]);
       count_launch();
       count_bytes(BY_TRANSFER, (double)sizeof(T) * s * (2.0 * (double)g.n + (double)gc.n));
     }
