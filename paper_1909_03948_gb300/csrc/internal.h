@@ -372,7 +372,11 @@ int launch_leg(LegArgs a, const GridDesc &g, bool full, bool up, int vw, int s, 
 // the stream drains, and wait in pdl_enter() until it has completed and its writes are
 // visible.  They are let in only after pdl_enter() of every CTA of the kernel before, so what is
 // read ahead of pdl_enter() must be older than that kernel.  Each kernel launched this way calls
-// pdl_enter() in all its threads.  A solve is a chain of hundreds of launches of a few us: one
+// pdl_enter() in all its threads, and reads what the solve writes through ordinary loads: the
+// kernel is resident while the one before it still stores, and a non-coherent load (__ldg, or
+// what the compiler makes of a const __restrict__ parameter) is only defined, and only kept behind
+// the wait, for data that is constant over the kernel's whole life.  The stencils and the
+// coarse inverse, written when a point is set, are.  A solve is a chain of hundreds of launches of a few us: one
 // column on 257^2 nodes 1.76 -> 1.70 ms, a 3D block of 24^3 cells' full Hessian 3.71 -> 3.49 ms,
 // a gradient on 257^2 nodes 4.17 -> 3.97 ms.
 // Not for kernels of very many short CTAs: the wait costs each of them some hundred clocks

@@ -36,17 +36,12 @@ template <int VW> struct LegV;  // VW values of one node
 template <> struct LegV<1> {
   float v[1];
   __device__ __forceinline__ static LegV ld(const float *p) { return {{*p}}; }
-  __device__ __forceinline__ static LegV ldg(const float *p) { return {{__ldg(p)}}; }
   __device__ __forceinline__ void st(float *p) const { *p = v[0]; }
 };
 template <> struct LegV<4> {
   float v[4];
   __device__ __forceinline__ static LegV ld(const float *p) {
     const float4 t = *reinterpret_cast<const float4 *>(p);
-    return {{t.x, t.y, t.z, t.w}};
-  }
-  __device__ __forceinline__ static LegV ldg(const float *p) {
-    const float4 t = __ldg(reinterpret_cast<const float4 *>(p));
     return {{t.x, t.y, t.z, t.w}};
   }
   __device__ __forceinline__ void st(float *p) const {
@@ -104,7 +99,7 @@ template <int VW, bool FULL> struct LegStrip {
   // strip values of the block at base (group's first value), zero outside the grid
   __device__ __forceinline__ void load(const LegArgs &a, const float *base, V x[LEG_N]) const {
 #pragma unroll
-    for (int k = 0; k < LEG_N; ++k) x[k] = V::ldg(base + (long)node(a, gx, gy + k) * VW);
+    for (int k = 0; k < LEG_N; ++k) x[k] = V::ld(base + (long)node(a, gx, gy + k) * VW);
 #pragma unroll
     for (int k = 0; k < LEG_N; ++k)
 #pragma unroll
@@ -352,8 +347,8 @@ __global__ void __launch_bounds__(LEG_NT, VW == 4 ? 2 : 3) k_leg_up(const __grid
 #pragma unroll
     for (int k = 0; k < LEG_N; ++k) {
       const int Y = min(max(C.gy + k, 0), np - 1), ic = (X >> 1) + npc * (Y >> 1);
-      e0[k] = V::ldg(ec + (long)ic * VW);
-      e1[k] = V::ldg(ec + (long)(ic + (X & 1) + (Y & 1) * npc) * VW);
+      e0[k] = V::ld(ec + (long)ic * VW);
+      e1[k] = V::ld(ec + (long)(ic + (X & 1) + (Y & 1) * npc) * VW);
     }
 #pragma unroll
     for (int k = 0; k < LEG_N; ++k) {

@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(MA_NT, 2) k_march_full(const __grid_constant__
     }
   }
   float acc[4] = {0.f, 0.f, 0.f, 0.f};
-  const float4 *__restrict__ bp = reinterpret_cast<const float4 *>(a.B + blockIdx.y * a.gb) + xy;
+  const float4 *bp = reinterpret_cast<const float4 *>(a.B + blockIdx.y * a.gb) + xy;
   for (int p = zb; p < ze; ++p) {
     // into the slot of plane p - 2, which every thread has left at the last barrier
     issue(p + MA_AHEAD);

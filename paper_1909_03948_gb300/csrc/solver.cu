@@ -149,7 +149,7 @@ __device__ __forceinline__ void dot_partial(const Pack<T, VW> &acc, double *part
   }
 }
 
-__global__ void k_dot_finalize(const double *__restrict__ part, unsigned nblk, Fin fin) {
+__global__ void k_dot_finalize(const double *part, unsigned nblk, Fin fin) {
   pdl_enter();
   const int col = blockIdx.x;
   double sum = 0.0;
@@ -159,7 +159,7 @@ __global__ void k_dot_finalize(const double *__restrict__ part, unsigned nblk, F
 }
 
 // two products at once: fin's partials, then fin2's
-__global__ void k_dot_finalize2(const double *__restrict__ part, const double *__restrict__ part2, unsigned nblk,
+__global__ void k_dot_finalize2(const double *part, const double *part2, unsigned nblk,
                                 Fin fin, Fin fin2) {
   pdl_enter();
   const int col = blockIdx.x;
@@ -190,8 +190,8 @@ enum { M_APPLY = 0, M_APPLY_DOT = 1, M_RESID = 2, M_JACOBI = 3, M_JACOBI_DOT = 4
 
 template <typename T, int VW, int D, bool FULL, int MODE>
 __global__ void __launch_bounds__(NB) k_st(GridDesc g, const T *__restrict__ diag, const T *__restrict__ invdiag,
-                                           const T *__restrict__ c, const T *__restrict__ X, long gx,
-                                           const T *__restrict__ B, long gb, T *__restrict__ Y, long gy, int s,
+                                           const T *__restrict__ c, const T *X, long gx,
+                                           const T *B, long gb, T *__restrict__ Y, long gy, int s,
                                            T omega, T omega2, Fin fin) {
   pdl_enter();
   using PK = Pack<T, VW>;
@@ -677,8 +677,8 @@ __global__ void __launch_bounds__(TL3_NT) k_st_tile3(const __grid_constant__ CUt
 constexpr int C64 = 2;
 template <int D, bool FULL, bool RESID>
 __global__ void __launch_bounds__(NB) k_st64(GridDesc g, const double *__restrict__ diag,
-                                             const double *__restrict__ c, const double *__restrict__ X, long ldx,
-                                             const double *__restrict__ B, long ldb, double *__restrict__ Y, long ldy,
+                                             const double *__restrict__ c, const double *X, long ldx,
+                                             const double *B, long ldb, double *__restrict__ Y, long ldy,
                                              int s, double *part) {
   pdl_enter();
   constexpr int NF = FULL ? (1 << D) - 1 : D;
@@ -752,7 +752,7 @@ __global__ void __launch_bounds__(NB) k_st64(GridDesc g, const double *__restric
 // 1/2 sum_{b != 0} [r_f(2J + b) + r_f(2J - b)] over the 2^D - 1 Kuhn edge
 // directions b; Dirichlet rows of the zero-BC space are zeroed.
 template <typename T, int VW, int D>
-__global__ void __launch_bounds__(NB) k_restrict(GridDesc gf, GridDesc gc, const T *__restrict__ rf, long gsf,
+__global__ void __launch_bounds__(NB) k_restrict(GridDesc gf, GridDesc gc, const T *rf, long gsf,
                                                  T *__restrict__ rc, long gsc, int zero_dirichlet) {
   pdl_enter();
   using PK = Pack<T, VW>;
@@ -844,8 +844,8 @@ __device__ __forceinline__ Pack<T, VW> stencil_at(const GridDesc &g, const T *__
 // residual is never stored.  One coarse node per thread.
 template <typename T, int VW, int D, bool FULL>
 __global__ void __launch_bounds__(NB) k_resid_restrict(GridDesc gf, GridDesc gc, const T *__restrict__ diag,
-                                                       const T *__restrict__ c, const T *__restrict__ e,
-                                                       const T *__restrict__ bf, long gsf, T *__restrict__ rc,
+                                                       const T *__restrict__ c, const T *e,
+                                                       const T *bf, long gsf, T *__restrict__ rc,
                                                        long gsc, int zero_dirichlet) {
   pdl_enter();
   using PK = Pack<T, VW>;
@@ -898,8 +898,8 @@ __global__ void __launch_bounds__(NB) k_resid_restrict(GridDesc gf, GridDesc gc,
 template <typename T, int VW, int D, bool FULL>
 __global__ void __launch_bounds__(NB) k_prolong_sweep(GridDesc gf, GridDesc gc, const T *__restrict__ diag,
                                                       const T *__restrict__ invdiag, const T *__restrict__ c,
-                                                      const T *__restrict__ x, const T *__restrict__ ec,
-                                                      long gsc, const T *__restrict__ bf, T *__restrict__ y,
+                                                      const T *x, const T *ec,
+                                                      long gsc, const T *bf, T *__restrict__ y,
                                                       long gsf, T omega) {
   pdl_enter();
   using PK = Pack<T, VW>;
@@ -965,7 +965,7 @@ __global__ void __launch_bounds__(NB) k_prolong_sweep(GridDesc gf, GridDesc gc, 
 // dense coarse-grid inverse: e = A_c^{-1} r.  blockIdx.x = chunk of 32 rows (lanes),
 // blockIdx.y = column group; the 8 warps of a block split the k sum, then add.
 template <typename T, int VW>
-__global__ void __launch_bounds__(256) k_coarse_apply(const T *__restrict__ inv, int nc, const T *__restrict__ R,
+__global__ void __launch_bounds__(256) k_coarse_apply(const T *__restrict__ inv, int nc, const T *R,
                                                       long gsr, T *__restrict__ E, long gse) {
   pdl_enter();
   using PK = Pack<T, VW>;
@@ -1000,7 +1000,7 @@ __global__ void __launch_bounds__(256) k_coarse_apply(const T *__restrict__ inv,
 
 // 1-D node kernels: blockIdx.x over nodes (NB each), blockIdx.y = group
 template <typename T, int VW>
-__global__ void __launch_bounds__(NB) k_jacobi0(long n, const T *__restrict__ invdiag, const T *__restrict__ B, long gs,
+__global__ void __launch_bounds__(NB) k_jacobi0(long n, const T *__restrict__ invdiag, const T *B, long gs,
                                                 T *__restrict__ Y, T omega) {
   pdl_enter();
   using PK = Pack<T, VW>;
@@ -1016,9 +1016,9 @@ __global__ void __launch_bounds__(NB) k_jacobi0(long n, const T *__restrict__ in
 }
 
 template <typename T, int VW>
-__global__ void __launch_bounds__(NB) k_cg_update(long n, long gs, const T *__restrict__ p, const T *__restrict__ q,
+__global__ void __launch_bounds__(NB) k_cg_update(long n, long gs, const T *p, const T *q,
                                                   T *__restrict__ x, T *__restrict__ r,
-                                                  const double *__restrict__ alpha, int s, Fin fin) {
+                                                  const double *alpha, int s, Fin fin) {
   pdl_enter();
   using PK = Pack<T, VW>;
   const int grp = blockIdx.y;
@@ -1047,10 +1047,10 @@ __global__ void __launch_bounds__(NB) k_cg_update(long n, long gs, const T *__re
 // pass per iteration (38 us of 370 for 65^3 nodes and 120 columns) and two launches less; the
 // products and sums are those of k_jacobi0.
 template <typename T, int VW>
-__global__ void __launch_bounds__(NB) k_cg_update_diag(long n, long gs, const T *__restrict__ p,
-                                                       const T *__restrict__ q, T *__restrict__ x, T *__restrict__ r,
+__global__ void __launch_bounds__(NB) k_cg_update_diag(long n, long gs, const T *p,
+                                                       const T *q, T *__restrict__ x, T *__restrict__ r,
                                                        const T *__restrict__ invdiag,
-                                                       const double *__restrict__ alpha, int s, double *part,
+                                                       const double *alpha, int s, double *part,
                                                        double *part2) {
   pdl_enter();
   using PK = Pack<T, VW>;
@@ -1080,9 +1080,9 @@ __global__ void __launch_bounds__(NB) k_cg_update_diag(long n, long gs, const T 
 }
 
 template <typename T, int VW>
-__global__ void __launch_bounds__(NB) k_p_update_diag(long n, long gs, const T *__restrict__ r,
+__global__ void __launch_bounds__(NB) k_p_update_diag(long n, long gs, const T *r,
                                                       const T *__restrict__ invdiag, T *__restrict__ p,
-                                                      const double *__restrict__ beta) {
+                                                      const double *beta) {
   pdl_enter();
   using PK = Pack<T, VW>;
   const int grp = blockIdx.y;
@@ -1102,7 +1102,7 @@ __global__ void __launch_bounds__(NB) k_p_update_diag(long n, long gs, const T *
 
 // <r, D^-1 r> partials (the first product of that PCG)
 template <typename T, int VW>
-__global__ void __launch_bounds__(NB) k_dot_diag(long n, const T *__restrict__ invdiag, const T *__restrict__ R,
+__global__ void __launch_bounds__(NB) k_dot_diag(long n, const T *__restrict__ invdiag, const T *R,
                                                  long gs, int s, double *part) {
   pdl_enter();
   using PK = Pack<T, VW>;
@@ -1118,8 +1118,8 @@ __global__ void __launch_bounds__(NB) k_dot_diag(long n, const T *__restrict__ i
 }
 
 template <typename T, int VW>
-__global__ void __launch_bounds__(NB) k_p_update(long n, long gs, const T *__restrict__ z, T *__restrict__ p,
-                                                 const double *__restrict__ beta) {
+__global__ void __launch_bounds__(NB) k_p_update(long n, long gs, const T *z, T *__restrict__ p,
+                                                 const double *beta) {
   pdl_enter();
   using PK = Pack<T, VW>;
   const int grp = blockIdx.y;
@@ -1138,7 +1138,7 @@ __global__ void __launch_bounds__(NB) k_p_update(long n, long gs, const T *__res
 
 // <a, b> per column (a == b: squared norm)
 template <typename T, int VW>
-__global__ void __launch_bounds__(NB) k_dot(long n, long gs, const T *__restrict__ a, const T *__restrict__ b, int s,
+__global__ void __launch_bounds__(NB) k_dot(long n, long gs, const T *a, const T *b, int s,
                                             Fin fin) {
   pdl_enter();
   using PK = Pack<T, VW>;
@@ -1164,7 +1164,7 @@ __device__ __forceinline__ double to64(double x) { return x; }
 // <a, b> per column with the row kernels' grid and sums (k_st's dots): lanes along a row, a
 // thread's FP32 sum over its rows
 template <typename T, int VW>
-__global__ void __launch_bounds__(NB) k_row_dot(GridDesc g, const T *__restrict__ a, const T *__restrict__ b, long gs,
+__global__ void __launch_bounds__(NB) k_row_dot(GridDesc g, const T *a, const T *b, long gs,
                                                 int s, Fin fin) {
   pdl_enter();
   using PK = Pack<T, VW>;
@@ -1183,8 +1183,8 @@ __global__ void __launch_bounds__(NB) k_row_dot(GridDesc g, const T *__restrict_
 
 // r_T (grouped) = scale * r64 (column-major); columns >= s and converged ones are 0
 template <typename T, int VW>
-__global__ void __launch_bounds__(NB) k_to_inner(long n, const double *__restrict__ R, long ldr,
-                                                 const double *__restrict__ scale, int s, T *__restrict__ rt, long gs) {
+__global__ void __launch_bounds__(NB) k_to_inner(long n, const double *R, long ldr,
+                                                 const double *scale, int s, T *__restrict__ rt, long gs) {
   pdl_enter();
   using PK = Pack<T, VW>;
   const int grp = blockIdx.y;
@@ -1202,10 +1202,10 @@ __global__ void __launch_bounds__(NB) k_to_inner(long n, const double *__restric
 // The same scaling inside a graph-driven refinement: the first step (ctl->outer == 1,
 // counted before the step runs) starts from x = 0, so its residual is b0 itself.
 template <typename T, int VW>
-__global__ void __launch_bounds__(NB) k_to_inner_ctl(long n, const double *__restrict__ B0,
-                                                     const double *__restrict__ R, long ldr,
-                                                     const RefineCtl *__restrict__ ctl,
-                                                     const double *__restrict__ scale, int s, T *__restrict__ rt,
+__global__ void __launch_bounds__(NB) k_to_inner_ctl(long n, const double *B0,
+                                                     const double *R, long ldr,
+                                                     const RefineCtl *ctl,
+                                                     const double *scale, int s, T *__restrict__ rt,
                                                      long gs) {
   pdl_enter();
   using PK = Pack<T, VW>;
@@ -1228,9 +1228,9 @@ __global__ void __launch_bounds__(NB) k_to_inner_ctl(long n, const double *__res
 // of margin); then the loop condition: another step while a column is open, a
 // non-finite residual or max_outer steps end the loop with a flag.  after_body adds the
 // inner iterations of the step that just ran.
-__global__ void k_refine_ctl(int s, const double *__restrict__ rr, const double *__restrict__ bb, double rtol,
+__global__ void k_refine_ctl(int s, const double *rr, const double *bb, double rtol,
                              double tol_in, double *__restrict__ scale, double *__restrict__ iscale,
-                             double *__restrict__ tol2col, const int *__restrict__ pcg_iter, int after_body,
+                             double *__restrict__ tol2col, const int *pcg_iter, int after_body,
                              int max_outer, RefineCtl *ctl, cudaGraphConditionalHandle h) {
   pdl_enter();
   __shared__ int nact_s, bad_s;
@@ -1280,7 +1280,7 @@ __global__ void k_refine_ctl(int s, const double *__restrict__ rr, const double 
 
 // X (column-major FP64) += d / scale for the columns with scale != 0
 template <typename T, int VW>
-__global__ void __launch_bounds__(NB) k_accum(long n, const T *__restrict__ d, long gs, const double *__restrict__ iscale,
+__global__ void __launch_bounds__(NB) k_accum(long n, const T *d, long gs, const double *iscale,
                                               int s, double *__restrict__ X, long ldx) {
   pdl_enter();
   using PK = Pack<T, VW>;
@@ -1522,7 +1522,7 @@ __global__ void __launch_bounds__(NB) k_df_out_dfp(const float4 *__restrict__ Xp
 
 // End of a PCG iteration: count it and decide whether another one runs.  In
 // graph mode the decision drives the device-side while loop.
-__global__ void k_pcg_cond(const int *__restrict__ active, int s, int *iter, int maxit, int bump,
+__global__ void k_pcg_cond(const int *active, int s, int *iter, int maxit, int bump,
                            cudaGraphConditionalHandle h, int use_handle) {
   pdl_enter();
   __shared__ int any;
@@ -1551,7 +1551,7 @@ __global__ void k_pcg_cond(const int *__restrict__ active, int s, int *iter, int
 constexpr float CHEB_GAMMA = 2.f / 3.f, CHEB_RHO2 = 4.f / 9.f, CHEB_X0 = 0.4f;
 
 // step 0: number of steps; 1: one more step is done
-__global__ void k_cheb_ctl(const double *__restrict__ tol2col, int s, int maxit, int step, ChebCtl *ctl, int *active,
+__global__ void k_cheb_ctl(const double *tol2col, int s, int maxit, int step, ChebCtl *ctl, int *active,
                            cudaGraphConditionalHandle h, int use_handle) {
   pdl_enter();
   __shared__ float tmin[256];
@@ -1586,9 +1586,9 @@ __global__ void k_cheb_ctl(const double *__restrict__ tol2col, int s, int maxit,
 }
 
 // x_0, in x when n is even and in p otherwise
-__global__ void __launch_bounds__(NB) k_cheb_start(long n, long gs, const float *__restrict__ r,
+__global__ void __launch_bounds__(NB) k_cheb_start(long n, long gs, const float *r,
                                                    const float *__restrict__ invdiag, float *__restrict__ x,
-                                                   float *__restrict__ p, const ChebCtl *__restrict__ ctl) {
+                                                   float *__restrict__ p, const ChebCtl *ctl) {
   pdl_enter();
   float *y = (ctl->n & 1) ? p : x;
   const long g0 = blockIdx.y * gs;

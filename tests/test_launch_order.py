@@ -1,0 +1,42 @@
+"""Kernels that may be resident while the kernel before them still runs (they call pdl_enter())
+read what other kernels of a solve write through ordinary loads: a const __restrict__ pointer
+or __ldg lets the compiler use non-coherent loads, whose data has to be constant over the
+kernel's whole life and which nothing keeps behind the wait.  Only the stencils' coefficients
+and the dense coarse inverse are that old.  Read from the source: no GPU shows a missed order
+reliably."""
+import os
+import re
+
+import pytest
+
+CSRC = os.path.join(os.path.dirname(os.path.dirname(os.path.abspath(__file__))), "paper_1909_03948_gb300", "csrc")
+SETUP = {"diag", "invdiag", "c", "inv"}     # written when a problem or its point is set
+
+
+def source(name):
+    with open(os.path.join(CSRC, name)) as f:
+        return re.sub(r"//.*", "", f.read())
+
+
+def kernels():
+    for name in sorted(os.listdir(CSRC)):
+        if name.endswith(".cu"):
+            for k in re.finditer(r"__global__.*?\n}\n", source(name), re.S):
+                if "pdl_enter()" in k.group(0):
+                    yield pytest.param(k.group(0), id=re.search(r"\b(k_\w+)\(", k.group(0)).group(1))
+
+
+def test_kernels_found():
+    assert len(list(kernels())) >= 26
+
+
+@pytest.mark.parametrize("text", list(kernels()))
+def test_noncoherent_pointers_are_setup_data(text):
+    names = set(re.findall(r"const\s+\w+\s*\*\s*__restrict__\s+(\w+)", text))
+    assert names <= SETUP, names - SETUP
+
+
+@pytest.mark.parametrize("name", ["legs.cu", "march.cu"])
+def test_noncoherent_loads_are_setup_data(name):
+    args = re.findall(r"__ldg\(\s*([\w.]+)", source(name))
+    assert args and all(a.split(".")[-1] in SETUP for a in args), args
