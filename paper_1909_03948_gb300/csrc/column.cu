@@ -733,6 +733,8 @@ __device__ __forceinline__ void col_pcg(const ColArgs &a, int col, ColScal &sc) 
     });
     flat_dot([&](dfl rr) { sc.active = df2d(rr) > sc.stop; });
   }
+  // no copy outlives the CTA: a column without an iteration has not waited for the triangle yet
+  asm volatile("cp.async.wait_all;" ::: "memory");
   col_nodes<D, NPT>(n, [&](int, int id) { dst[(long)id * vw] = X[id]; });
   if (threadIdx.x == 0) atomicMax(a.iter, it);
 }

@@ -3,7 +3,8 @@ read what other kernels of a solve write through ordinary loads: a const __restr
 or __ldg lets the compiler use non-coherent loads, whose data has to be constant over the
 kernel's whole life and which nothing keeps behind the wait.  Only the stencils' coefficients
 and the dense coarse inverse are that old.  Read from the source: no GPU shows a missed order
-reliably."""
+reliably.  The same goes for asynchronous copies into the shared memory of a CTA that ends
+without having waited for them."""
 import os
 import re
 
@@ -40,3 +41,14 @@ def test_noncoherent_pointers_are_setup_data(text):
 def test_noncoherent_loads_are_setup_data(name):
     args = re.findall(r"__ldg\(\s*([\w.]+)", source(name))
     assert args and all(a.split(".")[-1] in SETUP for a in args), args
+
+
+def test_column_kernel_waits_for_its_copies_on_every_path():
+    """k_colpcg starts the copy of the coarse inverse's triangle before it knows whether its column
+    iterates at all (a zero right-hand side, or one that converged a refinement step ago, does
+    not), and the V-cycle, which waits for the copy, only runs in the loop."""
+    text = source("column.cu")
+    body = text[text.index("void col_pcg("):text.index("k_colpcg(")]
+    loop = body.index("for (; sc.active && it < maxit; ++it)")
+    assert "col_begin(a)" in text[text.index("k_colpcg("):]
+    assert "cp.async.wait_all" in body[loop:]
