@@ -807,24 +807,23 @@ template <int D> static bool col_layout(ColArgs &a, bool pcg) {
   return off <= CAP;
 }
 
-static int col_launch(void (*k)(const ColArgs), const ColArgs &a, int dim, int cols, cudaStream_t st) {
+static void col_launch(void (*k)(const ColArgs), const ColArgs &a, int dim, int cols, cudaStream_t st) {
   // the opt-in shared-memory size, once per kernel and device (setting it twice is harmless)
   static std::atomic<unsigned long long> done[8];
   static void (*const ks[8])(const ColArgs) = {k_vtail<2, false>, k_vtail<2, true>, k_vtail<3, false>, k_vtail<3, true>,
                                                k_colpcg<2, false>, k_colpcg<2, true>, k_colpcg<3, false>,
                                                k_colpcg<3, true>};
   int dev = 0;
-  HP_CUDA(cudaGetDevice(&dev));
+  if (cudaGetDevice(&dev) != cudaSuccess) return;
   for (int i = 0; i < 8; ++i) {
     if (ks[i] != k) continue;
     if (dev >= 64 || !(done[i].load(std::memory_order_acquire) & (1ull << dev))) {
-      HP_CUDA(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, COL_SMEM));
+      if (cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, COL_SMEM) != cudaSuccess) return;
       if (dev < 64) done[i].fetch_or(1ull << dev, std::memory_order_release);
     }
   }
   k<<<cols, dim == 2 ? col_nt<2>() : col_nt<3>(), sizeof(float) * a.nfloats, st>>>(a);
   count_launch();
-  return cuda_check(cudaGetLastError(), "column kernel");
 }
 
 bool col_fits(const ColArgs &in, bool pcg) {
@@ -832,18 +831,18 @@ bool col_fits(const ColArgs &in, bool pcg) {
   return a.lv[a.l0].n <= COL_MAXN && (a.lv[a.l0].g.dim == 2 ? col_layout<2>(a, pcg) : col_layout<3>(a, pcg));
 }
 
-int launch_vtail(ColArgs a, int dim, bool full, int cols, cudaStream_t st) {
+void launch_vtail(ColArgs a, int dim, bool full, int cols, cudaStream_t st) {
   (void)(dim == 2 ? col_layout<2>(a, false) : col_layout<3>(a, false));
-  return col_launch(dim == 2 ? (full ? k_vtail<2, true> : k_vtail<2, false>)
-                             : (full ? k_vtail<3, true> : k_vtail<3, false>),
-                    a, dim, cols, st);
+  col_launch(dim == 2 ? (full ? k_vtail<2, true> : k_vtail<2, false>)
+                      : (full ? k_vtail<3, true> : k_vtail<3, false>),
+             a, dim, cols, st);
 }
 
-int launch_colpcg(ColArgs a, int dim, bool full, int cols, cudaStream_t st) {
+void launch_colpcg(ColArgs a, int dim, bool full, int cols, cudaStream_t st) {
   (void)(dim == 2 ? col_layout<2>(a, true) : col_layout<3>(a, true));
-  return col_launch(dim == 2 ? (full ? k_colpcg<2, true> : k_colpcg<2, false>)
-                             : (full ? k_colpcg<3, true> : k_colpcg<3, false>),
-                    a, dim, cols, st);
+  col_launch(dim == 2 ? (full ? k_colpcg<2, true> : k_colpcg<2, false>)
+                      : (full ? k_colpcg<3, true> : k_colpcg<3, false>),
+             a, dim, cols, st);
 }
 
 }  // namespace hp

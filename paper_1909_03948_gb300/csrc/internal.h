@@ -345,8 +345,10 @@ struct ColArgs {
   int nfloats, nclear, offx, offp, offs, offc, offt, tn;
 };
 bool col_fits(const ColArgs &a, bool pcg);
-int launch_vtail(ColArgs a, int dim, bool full, int cols, cudaStream_t st);
-int launch_colpcg(ColArgs a, int dim, bool full, int cols, cudaStream_t st);
+// A refused launch (or set-up of one) is left pending in cudaGetLastError, as by every launch of a
+// solve: the PCG's caller fails the solve, or the capture, on it.
+void launch_vtail(ColArgs a, int dim, bool full, int cols, cudaStream_t st);
+void launch_colpcg(ColArgs a, int dim, bool full, int cols, cudaStream_t st);
 
 // ---- legs.cu --------------------------------------------------------------------
 // One leg of a 2D level's part of the V-cycle in one launch (FP32; see legs.cu).
@@ -365,7 +367,7 @@ struct LegArgs {
 };
 constexpr int LEG_MAXNU = 3;       // most sweeps of a leg
 int leg_tiles(const GridDesc &g);  // CTAs per column group (partials per column)
-int launch_leg(LegArgs a, const GridDesc &g, bool full, bool up, int vw, int s, cudaStream_t st);
+void launch_leg(LegArgs a, const GridDesc &g, bool full, bool up, int vw, int s, cudaStream_t st);
 
 // ---- launches that overlap the end of the kernel before them --------------------
 // Programmatic dependent launch: the kernel's CTAs may be set up while the kernel before it in

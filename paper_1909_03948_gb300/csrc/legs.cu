@@ -432,7 +432,7 @@ int leg_tiles(const GridDesc &g) {
   return ntx * nty;
 }
 
-int launch_leg(LegArgs a, const GridDesc &g, bool full, bool up, int vw, int s, cudaStream_t st) {
+void launch_leg(LegArgs a, const GridDesc &g, bool full, bool up, int vw, int s, cudaStream_t st) {
   const int halo = up ? a.nu : a.nu + 1;
   a.np = g.np;
   a.npc = g.N / 2 + 1;
@@ -456,7 +456,6 @@ int launch_leg(LegArgs a, const GridDesc &g, bool full, bool up, int vw, int s, 
              : (up ? (dot ? (K)k_leg_up<1, false, true> : (K)k_leg_up<1, false, false>) : (K)k_leg_down<1, false>);
   pdl_launch(k, dim3(a.ntx * a.nty, (s + vw - 1) / vw), nt, shm, st, a);
   count_launch();
-  return cuda_check(cudaGetLastError(), "level leg");
 }
 
 }  // namespace hp

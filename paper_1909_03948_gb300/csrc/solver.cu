@@ -2487,7 +2487,7 @@ static void pcg_init(hp_problem *P, OpKind op, int s, cudaGraphConditionalHandle
 
 // The PCG of every column in one launch (column.cu), the iteration count of the slowest in
 // sc.iter.
-template <int VW> static int pcg_columns(hp_problem *P, OpKind op, int s) {
+template <int VW> static void pcg_columns(hp_problem *P, OpKind op, int s) {
   BlockWS<float> &W = P->w32;
   cudaMemsetAsync(P->sc.iter.p, 0, sizeof(int), P->st);
   ColArgs a;
@@ -2499,7 +2499,7 @@ template <int VW> static int pcg_columns(hp_problem *P, OpKind op, int s) {
   a.open = tl_open;
   a.iter = P->sc.iter.as<int>();
   count_bytes(BY_VECTOR, 8.0 * (double)P->n * s);  // r read, x written: the rest stays on chip
-  return launch_colpcg(a, P->dim, stencil_of<float>(P, op, 0).full, (s + VW - 1) / VW * VW, P->st);
+  launch_colpcg(a, P->dim, stencil_of<float>(P, op, 0).full, (s + VW - 1) / VW * VW, P->st);
 }
 
 template <typename T, int VW>
@@ -2577,6 +2577,13 @@ static cudaError_t capture_leaf(cudaStream_t st, cudaGraphNode_t *leaf) {
   return cudaSuccess;
 }
 
+// A launch refused during the capture leaves its error pending and its node out of the graph:
+// such a graph is not instantiated (it would be kept, and replayed without that node).
+static cudaError_t instantiate(cudaGraphExec_t *ex, cudaGraph_t g) {
+  const cudaError_t e = cudaGetLastError();
+  return e != cudaSuccess ? e : cudaGraphInstantiate(ex, g, 0);
+}
+
 // Appends the PCG to graph g after node dep (none if null): the captured init, then a
 // conditional WHILE node whose body is one PCG iteration; *last receives the while node.
 // Capture runs on P->cap with P->st pointed at it by the caller.
@@ -2589,11 +2596,11 @@ static cudaError_t append_pcg(hp_problem *P, OpKind op, int s, double tol, int m
       e = cudaStreamBeginCaptureToGraph(P->cap, g, dep ? &dep : nullptr, nullptr, dep ? 1 : 0,
                                         cudaStreamCaptureModeRelaxed);
       if (e != cudaSuccess) return e;
-      const int rc = pcg_columns<VW>(P, op, s);
+      pcg_columns<VW>(P, op, s);
       const cudaError_t el = capture_leaf(P->cap, last);
       cudaGraph_t gg = g;
       e = cudaStreamEndCapture(P->cap, &gg);
-      return el != cudaSuccess ? el : e != cudaSuccess ? e : rc ? cudaErrorUnknown : cudaSuccess;
+      return el != cudaSuccess ? el : e;
     }
   }
   cudaGraphConditionalHandle h;
@@ -2649,7 +2656,7 @@ static int build_graph(hp_problem *P, OpKind op, int s, double tol, int maxit, P
     cudaGraphNode_t last = nullptr;
     if (e == cudaSuccess) e = append_pcg<T, VW>(P, op, s, tol, maxit, g, nullptr, &last);
     cudaGraphExec_t ex = nullptr;
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, g, 0);
+    if (e == cudaSuccess) e = instantiate(&ex, g);
     if (g) cudaGraphDestroy(g);
     if (e != cudaSuccess) return cuda_check(e, "PCG graph");
     *out = PcgGraph{graph_op(P, op, (int)sizeof(T), VW, s), (int)sizeof(T), VW, s, maxit, tol, ex};
@@ -2722,7 +2729,8 @@ static int pcg(hp_problem *P, OpKind op, int s, double rtol, int maxit, int *its
   }
   if constexpr (sizeof(T) == 4) {
     if (col_pcg_rule(P, op, 4, VW)) {
-      HP_TRY((pcg_columns<VW>(P, op, s)));
+      pcg_columns<VW>(P, op, s);
+      HP_CUDA(cudaGetLastError());
       HP_CUDA(cudaMemcpyAsync(h_it, P->sc.iter.p, sizeof(int), cudaMemcpyDeviceToHost, st));
       HP_CUDA(cudaStreamSynchronize(st));
       *its = *h_it;
@@ -2738,6 +2746,7 @@ static int pcg(hp_problem *P, OpKind op, int s, double rtol, int maxit, int *its
   for (;;) {
     prof_spin(P);
     pcg_body<T, VW>(P, op, s, tol2, 0, 0, maxit);
+    HP_CUDA(cudaGetLastError());
     HP_CUDA(cudaMemcpyAsync(hact, P->sc.active.p, sizeof(int) * s, cudaMemcpyDeviceToHost, st));
     HP_CUDA(cudaMemcpyAsync(h_it, P->sc.iter.p, sizeof(int), cudaMemcpyDeviceToHost, st));
     HP_CUDA(cudaStreamSynchronize(st));
@@ -2879,7 +2888,7 @@ static int build_solve_graph(hp_problem *P, OpKind op, int s, double rtol, doubl
       e = end_capture(body, false);
       if (e == cudaSuccess && rc) e = cudaErrorUnknown;
     }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, g, 0);
+    if (e == cudaSuccess) e = instantiate(&ex, g);
     if (g) cudaGraphDestroy(g);
     if (e != cudaSuccess) return cuda_check(e, "refinement graph");
     *out = SolveGraph{graph_op(P, op, (int)sizeof(T), VW, s), (int)sizeof(T), VW, s, maxit, max_outer, rtol, tol_in, ex};
@@ -3047,7 +3056,7 @@ static int build_solve_graph_dfp(hp_problem *P, OpKind op, int s, double rtol, d
       cudaGraph_t bg = body;
       e = cudaStreamEndCapture(cs, &bg);
     }
-    if (e == cudaSuccess) e = cudaGraphInstantiate(&ex, g, 0);
+    if (e == cudaSuccess) e = instantiate(&ex, g);
     if (g) cudaGraphDestroy(g);
     if (e != cudaSuccess) return cuda_check(e, "double-float refinement graph");
     *out = SolveGraph{graph_op(P, op, (int)sizeof(T), VW, s), 100 + (int)sizeof(T), VW, s, maxit, max_outer, rtol, tol_in, ex};
