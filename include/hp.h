@@ -342,9 +342,15 @@ typedef struct {
                       length that fills the GPU's last wave of CTAs better); 2: the same on
                       the finest level only (the coarser levels keep the row kernels); 0:
                       every warp loads its own row of nodes */
-  int smem_tail;   /* accepted (0..15) and kept, without effect: FP32 solves run the coarse
-                      end of the V-cycle, and the whole PCG of a problem that fits, with one
-                      CTA per column wherever that is the faster form */
+  int smem_tail;   /* where FP32 solves may run several steps of a multigrid level as one launch
+                      (a 2D level's two legs, the coarse end of the V-cycle in one CTA per
+                      column, the whole PCG of a problem that fits in one): 0 and 1, on
+                      every level where that was measured to be the faster form; k >= 2, on
+                      levels k and coarser only, the finer ones run one launch per step; 15:
+                      nowhere.  The results are the same bit for bit, but for a whole PCG in
+                      one CTA that holds the coarsest grid's inverse as a triangle (symmetric
+                      to the last bit, which the square inverse is not): there the
+                      preconditioner rounds differently */
   int refine_df;   /* arithmetic of the FP64 iterative refinement around FP32 inner solves
                       (the residual b - K x with its norm, the scaling into the inner
                       precision and the update x += d): 0 FP64 instructions; 1 (default)
@@ -363,8 +369,8 @@ int hp_get_tuning(const hp_problem *P, hp_tuning *t);
 /* Times one block of nrhs Gauss-Newton Hessian actions at the current point
  * (CUDA events, the mean of reps timed runs after a warm-up per candidate) over a
  * small candidate set by coordinate descent in two passes (smoother, column
- * chunk, fused transfers, tiled kernels, grid cap; a candidate must
- * be at least 1 % faster to be taken) and applies the fastest.  best / best_ms
+ * chunk, fused transfers, one launch per level leg or per step, tiled kernels, grid cap; a
+ * candidate must be at least 1 % faster to be taken) and applies the fastest.  best / best_ms
  * (HOST, may be NULL) receive it.  Needs hp_set_point first; allocates its test
  * block (setup-time call). */
 int hp_autotune(hp_problem *P, int nrhs, int reps, hp_tuning *best, double *best_ms);

@@ -20,7 +20,10 @@
 // that a stencil needs no boundary tests: a coupling that leaves the grid is zero (the
 // stencils store it so), a neighbour index that leaves the array reads the padding, and one
 // that wraps to another row meets a zero coupling.  Every value is formed by the operations
-// of the per-level kernels in their order, so a solve has the same bits either way.
+// of the per-level kernels in their order, so a solve has the same bits either way, with one
+// exception: where the coarse inverse is held as its lower triangle, an entry above the diagonal
+// is the one below it, and the square matrix of the per-level kernels, computed column by column,
+// is symmetric to rounding only.
 #include <algorithm>
 #include <atomic>
 #include <cstring>

@@ -147,7 +147,7 @@ struct hp_problem {
   int fuse_transfer = 0;        // residual + restriction and prolongation + first post sweep fused (tuning)
   double cheb_alpha = 10.0;     // Chebyshev interval [lmax / alpha, lmax]             (tuning)
   int tma_tiles = 0;            // 2D stiffness levels as TMA-tiled stencil kernels       (tuning)
-  int smem_tail = 0;            // kept for callers, without effect                              (tuning)
+  int smem_tail = 0;            // 0, 1 anywhere; k: several steps of a level per launch from level k on (tuning)
   int refine_df = 1;            // FP64 refinement arithmetic in double-float on the FP32 pipe:
                                 // 0 never, 1 for tolerances >= DF_MIN_RTOL, 2 always (tuning)
   cudaStream_t st = nullptr;

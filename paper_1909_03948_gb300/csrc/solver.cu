@@ -2104,6 +2104,9 @@ static bool tiled_level(const hp_problem *P, OpKind op, int l, int vw) {
   return on && op == OP_K && vw == 4 && P->lv[l].K32.pk && (tile_grid(P->lv[l].g) || tile3_grid(P->lv[l].g));
 }
 
+// whether the level may run several of its steps per launch (tuning smem_tail)
+static bool joined_level(const hp_problem *P, int l) { return P->smem_tail < 2 || l >= P->smem_tail; }
+
 // The part of an FP32 solve that runs with one CTA per column (column.cu): fills the
 // arguments for the levels from l0 down.
 static void col_args(const hp_problem *P, OpKind op, int vw, int s, int l0, ColArgs *a) {
@@ -2134,12 +2137,13 @@ static void col_args(const hp_problem *P, OpKind op, int vw, int s, int l0, ColA
 }
 
 // first level whose cycle runs with one CTA per column: the finest that fits (at most
-// COL_MAXN nodes) and is not asked to run as TMA tiles; L if there is none (and in FP64)
+// COL_MAXN nodes) and is not asked to run as TMA tiles or step by step; L if there is none
+// (and in FP64)
 static int col_level(const hp_problem *P, OpKind op, int tbytes, int vw) {
   const int L = op == OP_M ? 1 : P->L;
   if (tbytes != 4) return L;
   int l = L;
-  while (l > 0 && P->lv[l - 1].g.n <= COL_MAXN && !tiled_level(P, op, l - 1, vw)) {
+  while (l > 0 && P->lv[l - 1].g.n <= COL_MAXN && joined_level(P, l - 1) && !tiled_level(P, op, l - 1, vw)) {
     ColArgs a;
     col_args(P, op, vw, 1, l - 1, &a);
     if (!col_fits(a, l == 1)) break;
@@ -2172,9 +2176,11 @@ static int tail_level(const hp_problem *P, OpKind op, int tbytes, int vw) {
 }
 
 // Whether a level's legs run as one launch each (legs.cu): FP32, 2D, up to LEG_MAXNU sweeps
-// (the halo), neither asked to run as TMA tiles nor with the transfers fused the other way.
+// (the halo), neither asked to run as TMA tiles or step by step nor with the transfers fused
+// the other way.
 static bool leg_level(const hp_problem *P, OpKind op, int l, int tbytes, int vw) {
-  return tbytes == 4 && P->dim == 2 && nu_at(P, l) <= LEG_MAXNU && !fuse_at(P, l) && !tiled_level(P, op, l, vw);
+  return tbytes == 4 && P->dim == 2 && joined_level(P, l) && nu_at(P, l) <= LEG_MAXNU && !fuse_at(P, l) &&
+         !tiled_level(P, op, l, vw);
 }
 
 // Algorithmic bytes of the V-cycle's levels l0 .. L-1 as the per-level kernels would move

@@ -2,8 +2,8 @@
 //
 // Knobs: the V-cycle's smoother (nu sweeps, damped Jacobi with omega or Chebyshev
 // weights on [lmax / alpha, lmax]), the RHS column chunk processed per solve (0 = all
-// columns at once), fused grid transfers, the shared-memory coarse tail, the TMA-tiled
-// stencil kernels, the double-float refinement and the grid-size cap of the node
+// columns at once), fused grid transfers, one launch per level leg (or coarse end) or per
+// step, the TMA-tiled stencil kernels, the double-float refinement and the grid-size cap of the node
 // kernels.  hp_autotune times one block of Gauss-Newton Hessian actions at the current
 // linearisation point (CUDA events on the problem's stream) for each candidate, by
 // coordinate descent over the groups of knobs, and keeps the fastest.  Every candidate
@@ -149,6 +149,12 @@ static int autotune_on(hp_problem *P, const double *X, int ldx, int nrhs, int re
       if (ft == cur.fuse_transfer) continue;
       hp_tuning t = cur;
       t.fuse_transfer = ft;
+      if ((rc = consider(t))) return cleanup(rc);
+    }
+    for (int st : {0, HP_MAXL - 1}) {
+      if ((st >= 2) == (cur.smem_tail >= 2)) continue;
+      hp_tuning t = cur;
+      t.smem_tail = st;
       if ((rc = consider(t))) return cleanup(rc);
     }
     for (int tt : {0, 1, 2}) {
