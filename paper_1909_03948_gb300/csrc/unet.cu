@@ -479,8 +479,7 @@ __global__ void __launch_bounds__(256) k_conv_bwd_data(const float *__restrict__
 // flight at once, the two resident blocks covering each other's loads -- and a lane then
 // marches down its column keeping the K x K input window and the GW_C K^2 sums in registers:
 // K + GW_C shared-memory loads per GW_C K^2 multiply-adds.  A lane sums up to GW_HELD sets in
-// FP32 (288 terms; the previous form up to 324 for the same batch), the lanes are added in
-// FP32 and everything above in FP64.
+// FP32, the lanes are added in pairs of floats and everything above in FP64.
 // k_conv_bwd_weight_final: adds the chunks (FP64), and the bias gradient's per-image sums.
 //
 // Bound: the FP32 pipes and the issue slots (16 images of 72^2 pixels: 3.4 G multiply-adds).
@@ -488,7 +487,7 @@ __global__ void __launch_bounds__(256) k_conv_bwd_data(const float *__restrict__
 // ms for that batch's 15 layers and the bias sums 1.3 ms; the marching lanes with plain loads
 // 2.6 ms (each row waited for its loads from L2).
 constexpr int GW_C = 8, GW_ROWS = 18, GW_WARPS = 8;
-constexpr int GW_HELD = 16;  // sets whose FP32 sums a lane carries on
+constexpr int GW_HELD = 16;  // most sets whose FP32 sums a lane carries on
 constexpr int GW_INW = 48;   // floats per staged input row: 32 lanes and the units' halos
 
 struct GwArgs {
@@ -498,25 +497,42 @@ struct GwArgs {
   int per, sw;           // units per warp, columns per unit
   int strips, segs;      // units per image row and column
   int units, sets;       // units in all, sets of `per` units
+  int held;              // sets whose FP32 sums a lane carries on
   double *part;          // [chunk][co][ci][K^2]
 };
 
 // Sums of NV values over the warp's lanes (NV a power of two up to 32): the value with index
-// lane % NV, by halving the values at each exchange (31 shuffles for 32 values).
-template <int NV> __device__ __forceinline__ float gw_lane_sums(float (&v)[32], int lane) {
+// lane % NV, by halving the values at each exchange (31 pairs exchanged for 32 values).  The sums
+// are kept in pairs of floats (two_sum, about 48 bits): FP64 additions here would cost a block
+// as much as its multiply-adds, and FP32 ones would round once per exchange.
+template <int NV> __device__ __forceinline__ double gw_lane_sums(float (&v)[32], int lane) {
+  float c[NV > 1 ? NV / 2 : 1];  // the low parts
+  bool low = false;              // (known at compile time in each unrolled step)
 #pragma unroll
   for (int o = NV / 2; o > 0; o >>= 1) {
     const bool up = lane & o;
 #pragma unroll
     for (int i = 0; i < o; ++i) {
       const float keep = up ? v[i + o] : v[i], send = up ? v[i] : v[i + o];
-      v[i] = keep + __shfl_xor_sync(0xffffffffu, send, o);
+      const dfl t = two_sum(keep, __shfl_xor_sync(0xffffffffu, send, o));
+      v[i] = t.hi;
+      if (low) {
+        const float kc = up ? c[i + o] : c[i], sc = up ? c[i] : c[i + o];
+        c[i] = t.lo + (kc + __shfl_xor_sync(0xffffffffu, sc, o));
+      } else {
+        c[i] = t.lo;
+      }
     }
+    low = true;
   }
-  float r = v[0];
+  float r = v[0], rc = low ? c[0] : 0.f;
 #pragma unroll
-  for (int o = NV; o < 32; o <<= 1) r += __shfl_xor_sync(0xffffffffu, r, o);
-  return r;
+  for (int o = NV; o < 32; o <<= 1) {
+    const dfl t = two_sum(r, __shfl_xor_sync(0xffffffffu, r, o));
+    rc = t.lo + (rc + __shfl_xor_sync(0xffffffffu, rc, o));
+    r = t.hi;
+  }
+  return rc == rc ? (double)r + (double)rc : (double)r;  // an infinite sum has no low part
 }
 
 template <int K, int C>
@@ -556,7 +572,7 @@ __global__ void __launch_bounds__(32 * GW_WARPS, 2) k_conv_bwd_weight(GwArgs a) 
         const int j = t * 32 + i < NV ? t * 32 + i : 0;
         v[i] = acc[j / KK][j % KK];
       }
-      tot[t] += (double)(t + 1 < NT32 ? gw_lane_sums<32>(v, lane) : gw_lane_sums<LAST>(v, lane));
+      tot[t] += t + 1 < NT32 ? gw_lane_sums<32>(v, lane) : gw_lane_sums<LAST>(v, lane);
     }
     clear();
   };
@@ -636,7 +652,7 @@ __global__ void __launch_bounds__(32 * GW_WARPS, 2) k_conv_bwd_weight(GwArgs a) 
       }
     }
     __syncthreads();
-    if (++held == GW_HELD) {
+    if (++held == a.held) {
       flush();
       held = 0;
     }
@@ -669,8 +685,8 @@ __global__ void __launch_bounds__(256) k_conv_bwd_weight_final(const double *__r
 }
 
 // dz = da [a > 0] in place (relu; linear layers keep da) and the sum of each plane (n, c) of
-// dz into bpart[n][c]: one block per plane, the sums in pairs of floats per thread (two_sum)
-// and FP64 across them
+// dz into bpart[n][c]: one block per plane, the sums in pairs of floats per thread (two_sum; an
+// infinite sum has no low part) and FP64 across them
 __global__ void __launch_bounds__(256) k_relu_back_bias(float *__restrict__ da, const float *__restrict__ a, int HW,
                                                         double *__restrict__ bpart) {
   float *d = da + (long)blockIdx.x * HW;
@@ -686,7 +702,7 @@ __global__ void __launch_bounds__(256) k_relu_back_bias(float *__restrict__ da, 
     s = t.hi;
     c += t.lo;
   }
-  const double sum = block_sum<256>((double)s + (double)c);
+  const double sum = block_sum<256>(c == c ? (double)s + (double)c : (double)s);
   if (threadIdx.x == 0) bpart[blockIdx.x] = sum;
 }
 
@@ -964,6 +980,9 @@ static void conv_bwd(hp_unet *U, int li, ConvIn I, float *d, const float *a_out,
   g.segs = (H + GW_ROWS - 1) / GW_ROWS;
   g.units = N * g.strips * g.segs;
   g.sets = (g.units + g.per - 1) / g.per;
+  // FP32 sums of at most 288 terms, and of fewer for small batches of small images: no longer than
+  // when the batch's pixels are divided among 256 threads (but one set at least)
+  g.held = (int)std::max<long>(1, std::min<long>(GW_HELD, (long)N * H * W / (256 * GW_ROWS)));
   g.part = part;
   const int blocks = gw_blocks(L);
   const long cnt = (long)L.co * L.ci * L.k * L.k;
