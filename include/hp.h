@@ -347,10 +347,7 @@ typedef struct {
                       column, the whole PCG of a problem that fits in one): 0 and 1, on
                       every level where that was measured to be the faster form; k >= 2, on
                       levels k and coarser only, the finer ones run one launch per step; 15:
-                      nowhere.  The results are the same bit for bit, but for a whole PCG in
-                      one CTA that holds the coarsest grid's inverse as a triangle (symmetric
-                      to the last bit, which the square inverse is not): there the
-                      preconditioner rounds differently */
+                      nowhere.  Every value gives the same results bit for bit */
   int refine_df;   /* arithmetic of the FP64 iterative refinement around FP32 inner solves
                       (the residual b - K x with its norm, the scaling into the inner
                       precision and the update x += d): 0 FP64 instructions; 1 (default)

@@ -20,10 +20,8 @@
 // that a stencil needs no boundary tests: a coupling that leaves the grid is zero (the
 // stencils store it so), a neighbour index that leaves the array reads the padding, and one
 // that wraps to another row meets a zero coupling.  Every value is formed by the operations
-// of the per-level kernels in their order, so a solve has the same bits either way, with one
-// exception: where the coarse inverse is held as its lower triangle, an entry above the diagonal
-// is the one below it, and the square matrix of the per-level kernels, computed column by column,
-// is symmetric to rounding only.
+// of the per-level kernels in their order, so a solve has the same bits either way (the square
+// coarse inverse is made symmetric to the last bit where its triangle may be held here).
 #include <algorithm>
 #include <atomic>
 #include <cstring>
@@ -832,6 +830,11 @@ static void col_launch(void (*k)(const ColArgs), const ColArgs &a, int dim, int 
 bool col_fits(const ColArgs &in, bool pcg) {
   ColArgs a = in;
   return a.lv[a.l0].n <= COL_MAXN && (a.lv[a.l0].g.dim == 2 ? col_layout<2>(a, pcg) : col_layout<3>(a, pcg));
+}
+
+bool col_holds(const ColArgs &in) {
+  ColArgs a = in;
+  return a.lv[0].n <= COL_MAXN && (a.lv[0].g.dim == 2 ? col_layout<2>(a, true) : col_layout<3>(a, true)) && a.tn > 0;
 }
 
 void launch_vtail(ColArgs a, int dim, bool full, int cols, cudaStream_t st) {

@@ -558,14 +558,17 @@ __global__ void __launch_bounds__(1024) k_dense_cholesky32(GridDesc g, const flo
 // L y = e_j from row j on (rows above are zero), then L^T x = y, each row's sum split over
 // the 32 lanes and reduced.  L is held in shared memory: a row is a chain of loads, lane sums,
 // five shuffles and a division, and with L read from L2 the chains took 500 us.  x goes out
-// as row j of inv32 (the inverse is symmetric) and its entries from j on as column j of tri32.
+// as row j of inv32 (the inverse is symmetric) and its entries from j on as column j of tri32;
+// with sym, the entries from j on as row and column j of inv32, so that the square and the
+// triangle hold the same numbers (see col_holds_triangle).
 constexpr int CI_W = 16;  // columns per CTA
 static size_t inv32_smem(long nc) {
   return sizeof(float) * ((size_t)(nc * (nc + 1) / 2 + 3) / 4 * 4 + (size_t)CI_W * nc);
 }
 
 __global__ void __launch_bounds__(32 * CI_W) k_dense_inverse32(const float *__restrict__ Lg, int nc,
-                                                               float *__restrict__ inv32, float *__restrict__ tri32) {
+                                                               float *__restrict__ inv32, float *__restrict__ tri32,
+                                                               bool sym) {
   extern __shared__ __align__(16) float L[];
   const int lane = threadIdx.x & 31, w = threadIdx.x >> 5, nt4 = (nc * (nc + 1) / 2 + 3) / 4;
   for (int t = threadIdx.x; t < nt4; t += 32 * CI_W)
@@ -596,16 +599,22 @@ __global__ void __launch_bounds__(32 * CI_W) k_dense_inverse32(const float *__re
     __syncwarp();
   }
   for (int i = lane; i < nc; i += 32) {
-    inv32[(long)j * nc + i] = x[i];
-    if (i >= j) tri32[tri_at(i, j)] = x[i];
+    if (i >= j || !sym) inv32[(long)j * nc + i] = x[i];
+    if (i < j) continue;
+    if (sym) inv32[(long)i * nc + j] = x[i];
+    tri32[tri_at(i, j)] = x[i];
   }
 }
 
 // lower triangle of the symmetric FP32 inverse, row i at i (i + 1) / 2 (the one-CTA coarse
-// solve holds it in shared memory: half the square)
-__global__ void k_pack_tri(const float *__restrict__ inv, int nc, float *__restrict__ tri) {
+// solve holds it in shared memory: half the square); sym: and into the upper one
+__global__ void k_pack_tri(float *inv, int nc, float *__restrict__ tri, bool sym) {
   const int i = blockIdx.x;
-  for (int j = threadIdx.x; j <= i; j += blockDim.x) tri[(long)i * (i + 1) / 2 + j] = inv[(long)j * nc + i];
+  for (int j = threadIdx.x; j <= i; j += blockDim.x) {
+    const float v = inv[(long)j * nc + i];
+    tri[(long)i * (i + 1) / 2 + j] = v;
+    if (sym) inv[(long)i * nc + j] = v;
+  }
 }
 
 int coarse_setup(hp_problem *P, OpKind op) {
@@ -614,6 +623,7 @@ int coarse_setup(hp_problem *P, OpKind op) {
   const Stencil<double> &S = op == OP_K ? lc.K64 : lc.A64;
   const long nc = lc.g.n;
   int *dstat = P->sc.active.as<int>();
+  const bool sym = col_holds_triangle(P, op);
   constexpr size_t SMEM32 = 222 * 1024;
   if (P->precision == HP_FP32_IR && std::max(chol32_smem(nc), inv32_smem(nc)) <= SMEM32) {
     // only inv32 is used by FP32 inner solves: factor and invert in FP32 (inv64 is
@@ -634,7 +644,7 @@ int coarse_setup(hp_problem *P, OpKind op) {
     else
       k_dense_cholesky32<3><<<1, 1024, chol32_smem(nc), P->st>>>(lc.g, S32.diag, S32.c, S32.nf, S32.full, L32, dstat);
     k_dense_inverse32<<<(int)((nc + CI_W - 1) / CI_W), 32 * CI_W, inv32_smem(nc), P->st>>>(L32, (int)nc, C.inv32,
-                                                                                           C.tri32);
+                                                                                           C.tri32, sym);
     C.fp64_valid = false;
     count_launch(2);
   } else {
@@ -646,7 +656,7 @@ int coarse_setup(hp_problem *P, OpKind op) {
       k_dense_from_stencil<3><<<nb, 256, 0, P->st>>>(lc.g, S.diag, S.c, S.nf, S.full, C.dense);
     k_dense_cholesky<<<1, 1024, 0, P->st>>>(C.dense, (int)nc, dstat);
     k_dense_inverse<<<(int)((nc + 31) / 32), 32, 0, P->st>>>(C.dense, (int)nc, C.inv64, C.inv32);
-    k_pack_tri<<<(int)nc, 128, 0, P->st>>>(C.inv32, (int)nc, C.tri32);
+    k_pack_tri<<<(int)nc, 128, 0, P->st>>>(C.inv32, (int)nc, C.tri32, sym);
     C.fp64_valid = true;
     count_launch(4);
   }

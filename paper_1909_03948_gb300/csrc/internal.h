@@ -274,6 +274,7 @@ template <typename T>
 void launch_stencil_apply(const hp_problem *P, const GridDesc &g, const Stencil<T> &S, const T *X, long ldx,
                           T *Y, long ldy, int s, cudaStream_t st);
 int coarse_setup(hp_problem *P, hp::OpKind op);
+bool col_holds_triangle(const hp_problem *P, OpKind op);
 // Gershgorin bound of the spectrum of diag^-1 S for a level stencil (host value, synchronises)
 int gershgorin_bound(hp_problem *P, const GridDesc &g, const Stencil<double> &S, double *out);
 
@@ -345,6 +346,7 @@ struct ColArgs {
   int nfloats, nclear, offx, offp, offs, offc, offt, tn;
 };
 bool col_fits(const ColArgs &a, bool pcg);
+bool col_holds(const ColArgs &a);  // whether a PCG from a.l0 = 0 keeps the coarse inverse's triangle on chip
 // A refused launch (or set-up of one) is left pending in cudaGetLastError, as by every launch of a
 // solve: the PCG's caller fails the solve, or the capture, on it.
 void launch_vtail(ColArgs a, int dim, bool full, int cols, cudaStream_t st);

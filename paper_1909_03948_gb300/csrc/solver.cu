@@ -2136,6 +2136,16 @@ static void col_args(const hp_problem *P, OpKind op, int vw, int s, int l0, ColA
   a->tri = op == OP_M ? nullptr : (op == OP_K ? P->cK.tri32 : P->cA.tri32);
 }
 
+// Whether a one-CTA PCG of this problem holds the coarse inverse as its lower triangle.  The square
+// matrix, computed column by column, is symmetric to rounding only; coarse_setup then mirrors it
+// from the triangle, so that a solve has the same bits in either form.
+bool col_holds_triangle(const hp_problem *P, OpKind op) {
+  if (P->lv[0].g.n > COL_MAXN) return false;
+  ColArgs a;
+  col_args(P, op, 1, 1, 0, &a);
+  return col_holds(a);
+}
+
 // first level whose cycle runs with one CTA per column: the finest that fits (at most
 // COL_MAXN nodes) and is not asked to run as TMA tiles or step by step; L if there is none
 // (and in FP64)
