@@ -2162,12 +2162,28 @@ static int col_level(const hp_problem *P, OpKind op, int tbytes, int vw) {
   return l;
 }
 
-// Whether the whole PCG of a column runs in one CTA: wherever its finest level fits.  Measured
-// per iteration on 65^2 nodes: 32 us for any number of columns up to the 152 SMs, against 36
-// launches of 1.6 us or more; one Hessian column with the prior term on 33^2 nodes went from
-// 1.38 to 0.71 ms, a block of 16 samples' solves likewise.
-static bool col_pcg_rule(const hp_problem *P, OpKind op, int tbytes, int vw) {
-  return col_level(P, op, tbytes, vw) == 0;
+// Whether the whole PCG of a column runs in one CTA.  Its finest level has to fit, and one SM has
+// to do the column's work in less time than the chain of launches takes for the block.
+// Measured, one CTA per column against launches (with the legs and the coarse end joined):
+//  * the dense coarse solve, read from L2 where it is too large to hold, at every iteration: with
+//    up to 324 nodes 0.6 to 1.0 of the launches' time up to two columns per SM, with 676 nodes
+//    0.74 to 1.1, with 784 to 1,600 nodes 1.0 to 2.1;
+//  * columns beyond two per SM come in further rounds, while the launches' time grows slowly: 65^2
+//    nodes 0.87 at 304 columns, 1.07 at 380, 1.16 at 608, 1.33 at 1,216.  With a small coarse grid
+//    (held in shared memory beside the vectors) it stays ahead: 49^2 nodes 0.73 at 456, 13^3 0.6,
+//    9^3 0.8 at 1,216;
+//  * 3D stencils over all edges, 16 coefficients per node and more nodes than three per thread:
+//    1.0 to 1.2 up to 32 columns, 0.7 to 1.0 from 60 to 304, 1.2 at 608 (13^3 nodes: 0.6 to 0.8);
+//  * the mass matrix (no cycle): 0.33 to 0.98 up to 1,216 columns, but the Chebyshev iteration is
+//    faster yet where it is taken (15^3 nodes, 608 columns: 1,119 against 851 us).
+constexpr long COL_PCGC = 700, COL_TRIC = 216;
+static bool col_pcg_rule(const hp_problem *P, OpKind op, int tbytes, int vw, int s) {
+  if (col_level(P, op, tbytes, vw) != 0) return false;
+  if (op == OP_M) return s <= 8 * NSM && !cheb_rule(P, op, tbytes, vw, s);
+  const long n = P->lv[0].g.n, nc = P->lv[P->L - 1].g.n;
+  const bool edges = P->dim == 3 && op == OP_A && n > 3072;
+  if (nc > COL_PCGC || (edges && s <= 32)) return false;
+  return s <= (nc <= COL_TRIC && !edges ? 8 : 2) * NSM;
 }
 
 // First level of the one-launch coarse end of the V-cycle (a level above the coarsest one,
@@ -2608,7 +2624,7 @@ static cudaError_t append_pcg(hp_problem *P, OpKind op, int s, double tol, int m
                               cudaGraphNode_t dep, cudaGraphNode_t *last) {
   cudaError_t e;
   if constexpr (sizeof(T) == 4) {
-    if (col_pcg_rule(P, op, 4, VW)) {
+    if (col_pcg_rule(P, op, 4, VW, s)) {
       e = cudaStreamBeginCaptureToGraph(P->cap, g, dep ? &dep : nullptr, nullptr, dep ? 1 : 0,
                                         cudaStreamCaptureModeRelaxed);
       if (e != cudaSuccess) return e;
@@ -2682,7 +2698,7 @@ static int build_graph(hp_problem *P, OpKind op, int s, double tol, int maxit, P
 
 // launches of one PCG iteration (0 when the whole PCG is one launch per solve)
 static int kernels_per_iteration(const hp_problem *P, OpKind op, int tbytes, int vw, int s) {
-  if (col_pcg_rule(P, op, tbytes, vw)) return 0;
+  if (col_pcg_rule(P, op, tbytes, vw, s)) return 0;
   if (cheb_rule(P, op, tbytes, vw, s)) return 2;
   if (op == OP_M) return 6;
   // V-cycle: per level above the one-launch coarse end (or the dense coarse solve) pre
@@ -2703,7 +2719,7 @@ static int kernels_per_iteration(const hp_problem *P, OpKind op, int tbytes, int
 // condition, or the whole PCG in one launch
 static int kernels_per_pcg(const hp_problem *P, OpKind op, int tbytes, int vw, int s) {
   if (cheb_rule(P, op, tbytes, vw, s)) return 2;
-  return col_pcg_rule(P, op, tbytes, vw) ? 1 : (op == OP_M ? 5 : 3);
+  return col_pcg_rule(P, op, tbytes, vw, s) ? 1 : (op == OP_M ? 5 : 3);
 }
 
 // after a PCG: fails the solve if a tile kernel gave up waiting for its copies
@@ -2744,7 +2760,7 @@ static int pcg(hp_problem *P, OpKind op, int s, double rtol, int maxit, int *its
     return *h_it >= maxit ? HP_ERR_NOT_CONVERGED : 0;
   }
   if constexpr (sizeof(T) == 4) {
-    if (col_pcg_rule(P, op, 4, VW)) {
+    if (col_pcg_rule(P, op, 4, VW, s)) {
       pcg_columns<VW>(P, op, s);
       HP_CUDA(cudaGetLastError());
       HP_CUDA(cudaMemcpyAsync(h_it, P->sc.iter.p, sizeof(int), cudaMemcpyDeviceToHost, st));
