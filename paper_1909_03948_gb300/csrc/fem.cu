@@ -28,6 +28,7 @@
 #include <cmath>
 #include <cstring>
 #include <mutex>
+#include <type_traits>
 #include <vector>
 
 #include "dfloat.cuh"
@@ -910,6 +911,7 @@ __global__ void k_scale_C(GridDesc g, const double *__restrict__ E, const double
 // node's coordinates cost as much as its FP64 operations), CC_Q columns per thread that share
 // the coefficients.  Bound by the FP64 pipe: 2^{D+1} + 1 operations per node and column.
 // 65^3 nodes, 120 columns: C^T 1,730 -> 945 us, C 930 -> 923 (840 us is the pipe's time).
+// The last column of an odd count is taken alone (a call for one column: C 30.4 us, computed twice 37.4).
 constexpr int CC_Q = 2;
 template <int D, bool TRANS>
 __global__ void __launch_bounds__(NT) k_cct_apply(GridDesc g, const double *__restrict__ E,
@@ -918,38 +920,42 @@ __global__ void __launch_bounds__(NT) k_cct_apply(GridDesc g, const double *__re
                                                   double yb) {
   constexpr int NC = (1 << (D + 1)) - 1;
   const int j0 = blockIdx.y * CC_Q;
-  const double *x[CC_Q];
-#pragma unroll
-  for (int k = 0; k < CC_Q; ++k) x[k] = X + ldx * min(j0 + k, s - 1);
   const unsigned np = (unsigned)g.np, n = (unsigned)g.n;
-  for (unsigned i = blockIdx.x * NT + threadIdx.x; i < n; i += gridDim.x * NT) {
-    const unsigned t = div_np(g, i), t2 = D == 2 ? 0u : div_np(g, t);
-    const int v[3] = {(int)(i - t * np), D == 2 ? (int)t : (int)(t - t2 * np), (int)t2};
-    double acc[CC_Q];
-    const double b0 = beta[i];
+  auto nodes = [&](auto nk) {  // this block's nodes for the first nk of its columns
+    constexpr int Q = decltype(nk)::value;
+    const double *x[Q];
 #pragma unroll
-    for (int k = 0; k < CC_Q; ++k) acc[k] = mulr(b0, x[k][i]);
+    for (int k = 0; k < Q; ++k) x[k] = X + ldx * (j0 + k);
+    for (unsigned i = blockIdx.x * NT + threadIdx.x; i < n; i += gridDim.x * NT) {
+      const unsigned t = div_np(g, i), t2 = D == 2 ? 0u : div_np(g, t);
+      const int v[3] = {(int)(i - t * np), D == 2 ? (int)t : (int)(t - t2 * np), (int)t2};
+      double acc[Q];
+      const double b0 = beta[i];
 #pragma unroll
-    for (int q = 1; q < NC; ++q) {
-      int sg;
-      const int m = coff_mask<D>(q, &sg);
-      // C^T: the row whose offset q points at node i is i - (sg * m)
-      const int sgn = TRANS ? -sg : sg;
-      if (!shift_ok<D>(g, v, m, sgn)) continue;
-      const unsigned r = i + (unsigned)(sgn * (int)mask_offset(g, m));
-      const double w = beta[(size_t)q * n + (TRANS ? r : i)];
+      for (int k = 0; k < Q; ++k) acc[k] = mulr(b0, x[k][i]);
 #pragma unroll
-      for (int k = 0; k < CC_Q; ++k) acc[k] = fmadd(w, x[k][r], acc[k]);
+      for (int q = 1; q < NC; ++q) {
+        int sg;
+        const int m = coff_mask<D>(q, &sg);
+        // C^T: the row whose offset q points at node i is i - (sg * m)
+        const int sgn = TRANS ? -sg : sg;
+        if (!shift_ok<D>(g, v, m, sgn)) continue;
+        const unsigned r = i + (unsigned)(sgn * (int)mask_offset(g, m));
+        const double w = beta[(size_t)q * n + (TRANS ? r : i)];
+#pragma unroll
+        for (int k = 0; k < Q; ++k) acc[k] = fmadd(w, x[k][r], acc[k]);
+      }
+      const double f = TRANS ? mulr(scale, E[i]) : scale;
+#pragma unroll
+      for (int k = 0; k < Q; ++k) {
+        double *y = Y + ldy * (j0 + k) + i;
+        const double val = mulr(f, acc[k]);
+        *y = yb == 0.0 ? val : fmadd(yb, *y, val);
+      }
     }
-    const double f = TRANS ? mulr(scale, E[i]) : scale;
-#pragma unroll
-    for (int k = 0; k < CC_Q; ++k) {
-      if (j0 + k >= s) break;
-      double *y = Y + ldy * (j0 + k) + i;
-      const double val = mulr(f, acc[k]);
-      *y = yb == 0.0 ? val : fmadd(yb, *y, val);
-    }
-  }
+  };
+  if (j0 + CC_Q <= s) nodes(std::integral_constant<int, CC_Q>{});
+  else nodes(std::integral_constant<int, 1>{});
 }
 
 // The same two stencils in double-float arithmetic on the FP32 pipe (at the solve

@@ -25,6 +25,7 @@
 #include <atomic>
 #include <cmath>
 #include <cstring>
+#include <type_traits>
 
 #include <cuda.h>
 
@@ -669,11 +670,12 @@ __global__ void __launch_bounds__(TL3_NT) k_st_tile3(const __grid_constant__ CUt
 // ---------------------------------------------------------------------------
 // FP64 stencils of column-major blocks (the refinement's residual and the operator
 // applications), one node per thread over the flattened grid, C64 columns per thread that
-// share the node's coefficients and addresses.  Bound by the FP64 pipe (2 lanes per clock and
+// share the node's coefficients and addresses (one where an odd count ends).  Bound by the FP64 pipe (2 lanes per clock and
 // SM): 15 or 17 operations per node and column over all Kuhn edges in 3D.  The row kernel gives
 // a row of 65 nodes three warps, the third with one lane, and pays for 96.  65^3 nodes, 120
 // columns: A x 1,310 -> 823 us (840 us is the pipe's time without the boundary), its residual
-// 1,545 -> 966; K's residual 829 -> 536.
+// 1,545 -> 966; K's residual 829 -> 536.  A call for one column there takes 27.6 us, 34.8 when the
+// column was computed twice (the row kernel 32.9).
 constexpr int C64 = 2;
 template <int D, bool FULL, bool RESID>
 __global__ void __launch_bounds__(NB) k_st64(GridDesc g, const double *__restrict__ diag,
@@ -683,54 +685,58 @@ __global__ void __launch_bounds__(NB) k_st64(GridDesc g, const double *__restric
   pdl_enter();
   constexpr int NF = FULL ? (1 << D) - 1 : D;
   const int j0 = blockIdx.y * C64;
-  const double *x[C64];
-#pragma unroll
-  for (int q = 0; q < C64; ++q) x[q] = X + ldx * min(j0 + q, s - 1);
   double acc[C64];
 #pragma unroll
   for (int q = 0; q < C64; ++q) acc[q] = 0.0;
   const unsigned np = (unsigned)g.np, n = (unsigned)g.n;
-  for (unsigned i = blockIdx.x * NB + threadIdx.x; i < n; i += gridDim.x * NB) {
-    const unsigned t = div_np(g, i), t2 = D == 2 ? 0u : div_np(g, t);
-    const int v[3] = {(int)(i - t * np), D == 2 ? (int)t : (int)(t - t2 * np), (int)t2};
-    double sx[C64];
-    const double dg = diag[i];
+  auto nodes = [&](auto nq) {  // this block's nodes for the first nq of its columns
+    constexpr int Q = decltype(nq)::value;
+    const double *x[Q];
 #pragma unroll
-    for (int q = 0; q < C64; ++q) sx[q] = mulr(dg, x[q][i]);
+    for (int q = 0; q < Q; ++q) x[q] = X + ldx * (j0 + q);
+    for (unsigned i = blockIdx.x * NB + threadIdx.x; i < n; i += gridDim.x * NB) {
+      const unsigned t = div_np(g, i), t2 = D == 2 ? 0u : div_np(g, t);
+      const int v[3] = {(int)(i - t * np), D == 2 ? (int)t : (int)(t - t2 * np), (int)t2};
+      double sx[Q];
+      const double dg = diag[i];
 #pragma unroll
-    for (int f = 0; f < NF; ++f) {
-      const int b = FULL ? f + 1 : (1 << f);
-      bool fw = true, bw = true;
+      for (int q = 0; q < Q; ++q) sx[q] = mulr(dg, x[q][i]);
 #pragma unroll
-      for (int a = 0; a < D; ++a)
-        if ((b >> a) & 1) {
-          fw = fw && (v[a] < g.N);
-          bw = bw && (v[a] > 0);
+      for (int f = 0; f < NF; ++f) {
+        const int b = FULL ? f + 1 : (1 << f);
+        bool fw = true, bw = true;
+#pragma unroll
+        for (int a = 0; a < D; ++a)
+          if ((b >> a) & 1) {
+            fw = fw && (v[a] < g.N);
+            bw = bw && (v[a] > 0);
+          }
+        const unsigned off = (unsigned)mask_offset(g, b);
+        const double *cf = c + (size_t)f * n;
+        if (fw) {
+          const double w = cf[i];
+#pragma unroll
+          for (int q = 0; q < Q; ++q) sx[q] = fmadd(w, x[q][i + off], sx[q]);
         }
-      const unsigned off = (unsigned)mask_offset(g, b);
-      const double *cf = c + (size_t)f * n;
-      if (fw) {
-        const double w = cf[i];
+        if (bw) {
+          const double w = cf[i - off];
 #pragma unroll
-        for (int q = 0; q < C64; ++q) sx[q] = fmadd(w, x[q][i + off], sx[q]);
+          for (int q = 0; q < Q; ++q) sx[q] = fmadd(w, x[q][i - off], sx[q]);
+        }
       }
-      if (bw) {
-        const double w = cf[i - off];
 #pragma unroll
-        for (int q = 0; q < C64; ++q) sx[q] = fmadd(w, x[q][i - off], sx[q]);
+      for (int q = 0; q < Q; ++q) {
+        double out = sx[q];
+        if (RESID) {
+          out = addr(B[ldb * (j0 + q) + i], -sx[q]);
+          acc[q] = fmadd(out, out, acc[q]);
+        }
+        Y[ldy * (j0 + q) + i] = out;
       }
     }
-#pragma unroll
-    for (int q = 0; q < C64; ++q) {
-      if (j0 + q >= s) break;
-      double out = sx[q];
-      if (RESID) {
-        out = addr(B[ldb * (j0 + q) + i], -sx[q]);
-        acc[q] = fmadd(out, out, acc[q]);
-      }
-      Y[ldy * (j0 + q) + i] = out;
-    }
-  }
+  };
+  if (j0 + C64 <= s) nodes(std::integral_constant<int, C64>{});
+  else nodes(std::integral_constant<int, 1>{});
   if (RESID) {  // per-column partials [column][block]
     __shared__ double sh[NB / 32][C64];
 #pragma unroll
