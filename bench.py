@@ -320,6 +320,14 @@ def family_bytes(fam, n, s, dim, fp32):
         return n * (3 * s * 8 + (nf + 1) * 8)
     if fam == "cg_update":    # read p, q, x, r; write x, r
         return n * 6 * s * w
+    if fam == "leg_down":     # read r, write e and the coarse right-hand side, coefficients
+        return n * (2 * s * w + (nf + 2) * w) + (n * s * w) // 2 ** dim
+    if fam == "leg_up":       # read e, r and the coarse correction, write e, coefficients
+        return n * (3 * s * w + (nf + 2) * w) + (n * s * w) // 2 ** dim
+    if fam == "columns":      # read r, write x (the rest stays on chip)
+        return n * 2 * s * w
+    if fam == "cheb_step":    # read x, the iterate before it and b, write y, coefficients of all edges
+        return n * (4 * s * w + (2 ** dim + 1) * w)
     return None
 
 
@@ -528,7 +536,8 @@ def run_ours(args, rank, world):
         cnt, ms = fams[dom]
         fp32 = args.precision == "fp32_ir" and dom != "resid64"
         bpl = family_bytes(dom, P.n, s, w.dim, fp32)
-        kind = level0_kernel_kind(w.dim, w.N, tune, fp32) if dom != "cg_update" else "vector"
+        kind = ("vector" if dom == "cg_update" else "leg" if dom.startswith("leg") else
+                "column" if dom == "columns" else level0_kernel_kind(w.dim, w.N, tune, fp32))
         in_step_s = ms / cnt / 1e3
         peak, src = measured_peak()
         warm_us = cold_us = graph_us = None

@@ -465,8 +465,12 @@ int hp_warmstart_counts(const hp_problem *P, long long *recorded, long long *gue
  * stream around each launch):  0 level-0 PCG matvec (stencil + <p,Kp>),
  * 1 level-0 Jacobi smoothing sweep, 2 level-0 V-cycle residual, 3 FP64
  * refinement residual, 4 CG vector update (+ <r,r>), 5 whole V-cycle,
- * 6 level-0 fused two-sweep pre-smoothing. */
-#define HP_PROF_NIDS 7
+ * 6 level-0 fused two-sweep pre-smoothing.  Where several steps run as one launch
+ * (smem_tail), that launch is timed in their place: 7 level-0 down leg (pre-smoothing,
+ * residual, restriction) and 8 up leg (prolongation, post-smoothing) of a 2D V-cycle
+ * instead of 1, 2 and 6; 9 the whole PCG of all columns, a CTA each, instead of
+ * 0, 1, 2, 4, 5 and 6; 10 one Chebyshev step of a 3D mass solve instead of 0 and 4. */
+#define HP_PROF_NIDS 11
 /* Turns event timing on (on != 0) or off and clears the records. */
 int hp_profile_enable(hp_problem *P, int on);
 /* Synchronises the stream and returns, per family id < nids, the number of
@@ -478,8 +482,10 @@ int hp_profile_read(hp_problem *P, int nids, int *counts, double *total_ms);
 /* Replays one level-0 kernel of the last FP32 block solve on its live workspace
  * (same columns, launch configuration and tuning), reps times back to back on the
  * problem's stream, with CUDA events around the burst: family 0 damped-Jacobi
- * sweep, 1 V-cycle residual, 2 fused two-sweep pre-smoothing.  The kernels read
- * the workspace and write a scratch level vector, so the solver state is kept.
+ * sweep, 1 V-cycle residual, 2 fused two-sweep pre-smoothing, and in 2D (up to three
+ * sweeps) 3 the down leg, 4 the up leg.  Which of them the solve itself launched is what
+ * hp_profile_read counts.  The kernels read the workspace and write scratch level
+ * vectors, so the solver state is kept.
  * us_warm (HOST, may be NULL): mean microseconds per launch back to back (data
  * largely L2-resident).  us_cold (HOST, may be NULL): each launch preceded by a
  * read of the DEVICE buffer `flush` (>= 64 MB; pass one larger than L2), minus

@@ -240,7 +240,11 @@ enum ProfId {
   PROF_CG_UPDATE = 4,  // x += a p, r -= a q, <r, r>
   PROF_VCYCLE = 5,     // whole preconditioner application
   PROF_PRESMOOTH = 6,  // level-0 fused two-sweep pre-smoothing from zero
-  PROF_COUNT = 7
+  PROF_LEG_DOWN = 7,   // level-0 pre-smoothing, residual and restriction in one launch
+  PROF_LEG_UP = 8,     // level-0 prolongation and post-smoothing in one launch
+  PROF_COLUMNS = 9,    // the whole PCG of every column in one launch
+  PROF_CHEB = 10,      // one Chebyshev step of a mass solve
+  PROF_COUNT = 11
 };
 int prof_start(hp_problem *P, int id);   // returns a record index or -1
 void prof_stop(hp_problem *P, int rec);

@@ -2301,7 +2301,9 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
         oth[l] = ea[l];
         a.rc = const_cast<T *>(rl[l + 1]);
         a.gsc = gsl[l + 1];
+        const int pr = prof_start(P, l == 0 ? PROF_LEG_DOWN : -1);
         launch_leg(a, g, S.full, false, VW, s, st);
+        prof_stop(P, pr);
         count_bytes(level_family(g.n), 4.0 * ((2.0 * s + 2.0 + S.nf) * (double)g.n + (double)s * P->lv[l + 1].g.n));
         continue;
       }
@@ -2395,7 +2397,9 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
         a.gsc = gsl[l + 1];
         const bool own_dot = l == 0 && leg_dot(g, ng);
         a.part = own_dot ? fin.part : nullptr;
+        const int pr = prof_start(P, l == 0 ? PROF_LEG_UP : -1);
         launch_leg(a, g, S.full, true, VW, s, st);
+        prof_stop(P, pr);
         count_bytes(level_family(g.n), 4.0 * ((3.0 * s + 2.0 + S.nf) * (double)g.n + (double)s * gc.n));
         if (own_dot) {
           dot_finalize(fin, leg_tiles(g), s, st);
@@ -2490,7 +2494,9 @@ static void cheb_step(hp_problem *P, int s, cudaGraphConditionalHandle h, int us
   a.gx = a.gy = a.gb = W.ldn * 4;
   a.omega = CHEB_GAMMA;
   a.ctl = cheb_ctl(P);
+  const int pr = prof_start(P, PROF_CHEB);
   launch_march(a, g, MA_CHEB, s, P->st);
+  prof_stop(P, pr);
   count_bytes(level_family(g.n), st_bytes<float, M_JACOBI>(g, S, s) + 4.0 * (double)g.n * s);
   pdl_launch(k_cheb_ctl, 1, 256, 0, P->st, P->sc.tol2col.as<double>(), s, maxit, 1, cheb_ctl(P), P->sc.active.as<int>(), h,
                                    use_handle);
@@ -2558,13 +2564,17 @@ static void pcg_body(hp_problem *P, OpKind op, int s, double tol2, cudaGraphCond
     pdl_launch(k_p_update_diag<T, VW>, nodegrid(n, ng), NB, 0, st, n, gs, r, S0.invdiag, p, P->sc.beta.as<double>());
     count_launch();
     count_bytes(BY_VECTOR, (double)sizeof(T) * (double)n * (3.0 * s + 1.0));
+    pr = prof_start(P, PROF_MATVEC);
     st_launch<T, VW, M_APPLY_DOT>(g0, S0, p, gs, nullptr, 0, q, gs, s, T(0), make_fin(P, FIN_ALPHA), st);
+    prof_stop(P, pr);
     const dim3 gu = nodegrid(n, ng);
     const Fin frr = make_fin(P, FIN_RR, tol2), fbeta = make_fin(P, FIN_BETA_NEXT);
     double *part2 = frr.part + (long)gu.x * round4(s);
+    pr = prof_start(P, PROF_CG_UPDATE);
     pdl_launch(k_cg_update_diag<T, VW>, gu, NB, 0, st, n, gs, p, q, x, r, S0.invdiag, P->sc.alpha.as<double>(), s, frr.part,
                                                part2);
     pdl_launch(k_dot_finalize2, s, NB, 0, st, frr.part, part2, gu.x, frr, fbeta);
+    prof_stop(P, pr);
     count_bytes(BY_VECTOR, (double)sizeof(T) * (double)n * (6.0 * s + 1.0));
     pdl_launch(k_pcg_cond, 1, 256, 0, st, P->sc.active.as<int>(), s, P->sc.iter.as<int>(), maxit, 1, h, use_handle);
     count_launch(3);
@@ -2767,7 +2777,10 @@ static int pcg(hp_problem *P, OpKind op, int s, double rtol, int maxit, int *its
   }
   if constexpr (sizeof(T) == 4) {
     if (col_pcg_rule(P, op, 4, VW, s)) {
+      prof_spin(P);
+      const int pr = prof_start(P, PROF_COLUMNS);
       pcg_columns<VW>(P, op, s);
+      prof_stop(P, pr);
       HP_CUDA(cudaGetLastError());
       HP_CUDA(cudaMemcpyAsync(h_it, P->sc.iter.p, sizeof(int), cudaMemcpyDeviceToHost, st));
       HP_CUDA(cudaStreamSynchronize(st));
@@ -3378,31 +3391,64 @@ __global__ void k_flush_read(const float4 *__restrict__ a, long n4, float *__res
 
 }  // namespace hp
 
-extern "C" int hp_replay_kernel(hp_problem *P, int family, int reps, void *flush, size_t flush_bytes,
-                                double *us_warm, double *us_cold) {
-  using namespace hp;
-  if (!P || reps < 1 || family < 0 || family > 2 || (us_cold && (!flush || flush_bytes < (64u << 20))))
-    return set_error(HP_ERR_INVALID, "hp_replay_kernel: family 0..2, reps >= 1, flush buffer >= 64 MB");
+namespace hp {
+
+// whether hp_replay_kernel's family can be launched on the last solve's workspace
+static int replay_ready(const hp_problem *P, int family, const char *what) {
+  if (P->w32.scap < 4 || P->L < 2 || !P->have_point)
+    return set_error(HP_ERR_STATE, std::string(what) + ": needs an FP32 multi-column solve at a point first");
+  if (family >= 3 && (P->dim != 2 || nu_at(P, 0) > LEG_MAXNU))
+    return set_error(HP_ERR_STATE, std::string(what) + ": level legs are 2D, with up to three sweeps");
+  return 0;
+}
+
+// one launch of the family on the workspace, into level vectors that every V-cycle overwrites
+static void replay_launch(hp_problem *P, int family, cudaStream_t st) {
   BlockWS<float> &W = P->w32;
-  if (W.scap < 4 || P->L < 2 || !P->have_point)
-    return set_error(HP_ERR_STATE, "hp_replay_kernel: needs an FP32 multi-column solve at a point first");
-  const int s = W.scap, VW = 4;
-  const long gs = W.ldn * VW;
-  tl_max_blocks = P->max_blocks;
-  tl_tma = P->tma_tiles;
-  tl_n0 = P->n;
+  const int s = W.scap;
+  const long gs = W.ldn * 4;
   const GridDesc &g = P->lv[0].g;
   const Stencil<float> &S = P->lv[0].K32;
   const float om = (float)P->omega;
   float *z = W.z.as<float>(), *r = W.r.as<float>(), *y = W.lb[0].as<float>();
-  auto launch = [&]() {
-    if (family == 0)
-      st_launch<float, 4, M_JACOBI>(g, S, z, gs, r, gs, y, gs, s, om, Fin{}, P->st);
-    else if (family == 1)
-      st_launch<float, 4, M_RESID>(g, S, z, gs, r, gs, y, gs, s, om, Fin{}, P->st);
-    else
-      st_launch<float, 4, M_JAC2>(g, S, r, gs, nullptr, 0, y, gs, s, om, Fin{}, P->st, om);
-  };
+  if (family == 0) {
+    st_launch<float, 4, M_JACOBI>(g, S, z, gs, r, gs, y, gs, s, om, Fin{}, st);
+  } else if (family == 1) {
+    st_launch<float, 4, M_RESID>(g, S, z, gs, r, gs, y, gs, s, om, Fin{}, st);
+  } else if (family == 2) {
+    st_launch<float, 4, M_JAC2>(g, S, r, gs, nullptr, 0, y, gs, s, om, Fin{}, st, om);
+  } else {
+    const int nu = nu_at(P, 0);
+    float w[4];
+    smooth_weights<float>(P, OP_K, 0, w);
+    LegArgs a = leg_args(S, w, nu, OP_K);
+    a.r = r;
+    a.gs = gs;
+    a.x = y;
+    a.gsc = padded(P->lv[1].g.n) * 4;
+    if (family == 3) {
+      a.rc = W.lr[1].as<float>();
+    } else {
+      a.xin = z;
+      a.ec = W.la[1].as<float>();
+      if (leg_dot(g, (s + 3) / 4) && P->sc.scap >= s) a.part = P->sc.partial.as<double>();
+    }
+    launch_leg(a, g, S.full, family == 4, 4, s, st);
+  }
+}
+
+}  // namespace hp
+
+extern "C" int hp_replay_kernel(hp_problem *P, int family, int reps, void *flush, size_t flush_bytes,
+                                double *us_warm, double *us_cold) {
+  using namespace hp;
+  if (!P || reps < 1 || family < 0 || family > 4 || (us_cold && (!flush || flush_bytes < (64u << 20))))
+    return set_error(HP_ERR_INVALID, "hp_replay_kernel: family 0..4, reps >= 1, flush buffer >= 64 MB");
+  HP_TRY(replay_ready(P, family, "hp_replay_kernel"));
+  tl_max_blocks = P->max_blocks;
+  tl_tma = P->tma_tiles;
+  tl_n0 = P->n;
+  auto launch = [&]() { replay_launch(P, family, P->st); };
   const long n4 = (long)(flush_bytes / sizeof(float4));
   HP_TRY(P->sc.tmp.ensure(64));
   float *sink = P->sc.tmp.as<float>();
@@ -3445,33 +3491,18 @@ extern "C" int hp_replay_kernel(hp_problem *P, int family, int reps, void *flush
 
 extern "C" int hp_replay_kernel_graph(hp_problem *P, int family, int reps, double *us) {
   using namespace hp;
-  if (!P || reps < 1 || reps > 100000 || family < 0 || family > 2 || !us)
-    return set_error(HP_ERR_INVALID, "hp_replay_kernel_graph: family 0..2, reps in [1, 1e5], us non-null");
-  BlockWS<float> &W = P->w32;
-  if (W.scap < 4 || P->L < 2 || !P->have_point)
-    return set_error(HP_ERR_STATE, "hp_replay_kernel_graph: needs an FP32 multi-column solve at a point first");
-  const int s = W.scap;
-  const long gs = W.ldn * 4;
+  if (!P || reps < 1 || reps > 100000 || family < 0 || family > 4 || !us)
+    return set_error(HP_ERR_INVALID, "hp_replay_kernel_graph: family 0..4, reps in [1, 1e5], us non-null");
+  HP_TRY(replay_ready(P, family, "hp_replay_kernel_graph"));
   tl_max_blocks = P->max_blocks;
   tl_tma = P->tma_tiles;
   tl_n0 = P->n;
-  const GridDesc &g = P->lv[0].g;
-  const Stencil<float> &S = P->lv[0].K32;
-  const float om = (float)P->omega;
-  float *z = W.z.as<float>(), *r = W.r.as<float>(), *y = W.lb[0].as<float>();
   HP_CUDA(cudaStreamSynchronize(P->st));
   if (!P->cap) HP_CUDA(cudaStreamCreateWithFlags(&P->cap, cudaStreamNonBlocking));
   cudaGraph_t graph = nullptr;
   cudaGraphExec_t exec = nullptr;
   HP_CUDA(cudaStreamBeginCapture(P->cap, cudaStreamCaptureModeThreadLocal));
-  for (int k = 0; k < reps; ++k) {
-    if (family == 0)
-      st_launch<float, 4, M_JACOBI>(g, S, z, gs, r, gs, y, gs, s, om, Fin{}, P->cap);
-    else if (family == 1)
-      st_launch<float, 4, M_RESID>(g, S, z, gs, r, gs, y, gs, s, om, Fin{}, P->cap);
-    else
-      st_launch<float, 4, M_JAC2>(g, S, r, gs, nullptr, 0, y, gs, s, om, Fin{}, P->cap, om);
-  }
+  for (int k = 0; k < reps; ++k) replay_launch(P, family, P->cap);
   cudaError_t ce = cudaStreamEndCapture(P->cap, &graph);
   if (ce == cudaSuccess) ce = cudaGraphInstantiate(&exec, graph, 0);
   if (graph) cudaGraphDestroy(graph);

@@ -485,7 +485,8 @@ class Problem:
         return t.as_dict(), ms.value
 
     # ---- measurement -------------------------------------------------------------
-    PROF_NAMES = ("matvec", "smooth", "resid_mg", "resid64", "cg_update", "vcycle", "presmooth")
+    PROF_NAMES = ("matvec", "smooth", "resid_mg", "resid64", "cg_update", "vcycle", "presmooth",
+                  "leg_down", "leg_up", "columns", "cheb_step")
 
     def profile_enable(self, on: bool = True):
         _check(lib().hp_profile_enable(self._h, 1 if on else 0), "hp_profile_enable")
@@ -497,7 +498,7 @@ class Problem:
         _check(lib().hp_profile_read(self._h, k, cnt, ms), "hp_profile_read")
         return {name: (cnt[i], ms[i]) for i, name in enumerate(self.PROF_NAMES)}
 
-    REPLAY_FAMILIES = ("smooth", "resid_mg", "presmooth")
+    REPLAY_FAMILIES = ("smooth", "resid_mg", "presmooth", "leg_down", "leg_up")  # the legs in 2D only
 
     def replay_kernel(self, family: str, reps: int, flush=None):
         """(us per launch back to back, us per launch from HBM or None) of a level-0
