@@ -1224,13 +1224,12 @@ int hp_laplace_sample(hp_problem *P, const double *m_map, const double *lambda, 
     }
     if (post) {
       // R x = A M^{-1} (A x) = A M^{-1} W
-      // V^T R x below magnifies this solve's error some thousandfold: at 1e-12 the error of
-      // either iteration is 7e-10 of the samples (65^3 nodes, 100 pairs).  CG keeps them equal to
-      // earlier samples of the same seed to 1e-9, the Chebyshev iteration would move them by 3e-9.
-      P->mass_cg = true;
-      const int mrc = solve_block(P, OP_M, W, ld, t, ld, cs, std::min(P->rtol, 1e-10), st);
-      P->mass_cg = false;
-      HP_TRY(mrc);
+      // V^T R x below magnifies this solve's error some thousandfold.  Against solves to 7e-15, at
+      // 1e-12, 64 samples: 8.1e-10 of the samples by CG and 6.6e-10 by the Chebyshev iteration
+      // (65^3 nodes, 100 pairs), 4.9e-10 and 4.9e-10 (57 pairs), 2.9e-10 and 2.6e-10 (49^3, 80).
+      // They are equally accurate, but apart by as much as either error, so CG stays here: a
+      // seed keeps giving the samples it gave.
+      HP_TRY(solve_block(P, OP_M, W, ld, t, ld, cs, std::min(P->rtol, 1e-10), st, true));
       HP_TRY(apply_op64(P, OP_A, t, ld, RX, ld, cs));
       if (k > 0) {
         HP_TRY(gram(P, V, ldv, k, RX, ld, cs, z, k, n));

@@ -153,7 +153,7 @@ struct hp_problem {
   cudaStream_t st = nullptr;
   cudaStream_t cap = nullptr;   // private stream used to capture CUDA graphs
   bool use_graphs = true;       // inner PCG loops as graphs with a device-side while node
-  bool mass_cg = false;   // M by CG also where the Chebyshev iteration would be taken (set around a call)
+  bool mass_cg = false;   // of the running solve_block: M by CG where the Chebyshev iteration would be taken
   std::vector<hp::PcgGraph> graphs;
   std::vector<hp::SolveGraph> sgraphs;
 
@@ -319,7 +319,7 @@ int ensure_scalars(hp_problem *P, int s);
 void drop_graphs(hp_problem *P);
 void free_scalars_host(hp_problem *P);
 int solve_block(hp_problem *P, OpKind op, const double *B, long ldb, double *X, long ldx, int s,
-                double rtol, hp_solve_stats *st);
+                double rtol, hp_solve_stats *st, bool mass_cg = false);
 int apply_op64(hp_problem *P, OpKind op, const double *X, long ldx, double *Y, long ldy, int s);
 
 // ---- column.cu ----------------------------------------------------------------

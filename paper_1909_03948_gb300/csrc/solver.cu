@@ -3357,10 +3357,12 @@ static int solve_chunk(hp_problem *P, OpKind op, const double *B, long ldb, doub
   return ir_solve<float, 1>(P, op, B, ldb, X, ldx, s, rtol, P->inner_rtol, st);
 }
 
-// Solves the s columns in chunks of the tuned width (0: all at once).
+// Solves the s columns in chunks of the tuned width (0: all at once).  mass_cg: M by CG, never by
+// the Chebyshev iteration.
 int solve_block(hp_problem *P, OpKind op, const double *B, long ldb, double *X, long ldx, int s, double rtol,
-                hp_solve_stats *st) {
+                hp_solve_stats *st, bool mass_cg) {
   if (s <= 0) return 0;
+  P->mass_cg = mass_cg;
   tl_max_blocks = P->max_blocks;
   tl_tma = P->tma_tiles;
   tl_n0 = P->n;

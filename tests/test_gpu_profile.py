@@ -65,3 +65,19 @@ def test_replay_of_legs():
                     P.replay_kernel_graph(fam, 5)
         assert torch.equal(P.state_solve(B)[0], x0)
         P.close()
+
+
+def test_samples_keep_cg():
+    """The sampling update's mass solve runs by CG, the mass solves before and after it do not."""
+    from paper_1909_03948_gb300 import Problem
+    P = Problem(3, 32, 0.1, 0.5, 0.01, np.zeros((0, 3)), rtol=1e-8)
+    B = torch.tensor(np.random.default_rng(1).standard_normal((60, P.n)), device=DEV)
+    m = torch.zeros(P.n, dtype=torch.float64, device=DEV)
+    lam, V = torch.ones(2, dtype=torch.float64, device=DEV), B[:2].clone()
+    P.profile_enable(True)
+    for call, cheb in ((lambda: P.mass_solve(B), True),
+                       (lambda: P.laplace_sample(m, lam, V, want_prior=False, seed=3, nsamples=60), False),
+                       (lambda: P.mass_solve(B), True)):
+        call()
+        assert (P.profile_read()["cheb_step"][0] > 0) == cheb
+    P.close()
