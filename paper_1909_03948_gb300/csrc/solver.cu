@@ -2192,27 +2192,30 @@ static bool col_pcg_rule(const hp_problem *P, OpKind op, int tbytes, int vw, int
   return s <= (nc <= COL_TRIC && !edges ? 8 : 2) * NSM;
 }
 
-// First level of the one-launch coarse end of the V-cycle (a level above the coarsest one,
-// whose own solve is a launch either way), or L.  It starts at COL_TAILN nodes: a larger level
-// costs one SM about what its nine launches cost (65^2 nodes: 28 us from there down, against
-// 19 launches of 1.6 us inside a CUDA graph).  The dense coarse solve has to be small too: one
-// SM takes 6.7 us for 17^2 nodes, bound by its reads of the matrix from L2, where the launch
-// over 150 CTAs takes 3 (measured over 33^2 and 17^2 nodes: no gain; over 13^3, 7^3 and 4^3
-// nodes a block of full-Newton actions on 49^3 went from 4.34 to 3.76 ms).
-constexpr long COL_TAILN = 2304, COL_TAILC = 200;
-static int tail_level(const hp_problem *P, OpKind op, int tbytes, int vw) {
-  if (P->lv[P->L - 1].g.n > COL_TAILC) return P->L;
-  int l = std::max(1, col_level(P, op, tbytes, vw));
-  while (l < P->L && P->lv[l].g.n > COL_TAILN) ++l;
-  return l + 1 < P->L ? l : P->L;
-}
-
 // Whether a level's legs run as one launch each (legs.cu): FP32, 2D, up to LEG_MAXNU sweeps
 // (the halo), neither asked to run as TMA tiles or step by step nor with the transfers fused
 // the other way.
 static bool leg_level(const hp_problem *P, OpKind op, int l, int tbytes, int vw) {
   return tbytes == 4 && P->dim == 2 && joined_level(P, l) && nu_at(P, l) <= LEG_MAXNU && !fuse_at(P, l) &&
          !tiled_level(P, op, l, vw);
+}
+
+// First level of the one-launch coarse end of the V-cycle (a level above the coarsest one,
+// whose own solve is a launch either way), or L.  Where a level's legs are one launch each there is
+// nothing to gain: 2D levels of 37^2 nodes and less took 1.04 to 1.09 times as long for one
+// column, 1.0 up to 152 and 1.1 for 608 and more, in rounds of 152 CTAs.  In 3D it replaces nine
+// launches per level: 13^3, 7^3 and 4^3 nodes of a 49^3 or 25^3 grid, stiffness and prior solves
+// 0.82 to 0.92 of the time up to 16 columns, 0.93 to 0.99 at 304, 1.0 at 1,216.
+// It starts at COL_TAILN nodes: a larger level costs one SM about what its nine launches cost
+// (65^2 nodes: 28 us from there down, against 19 launches of 1.6 us inside a CUDA graph).  The
+// dense coarse solve has to be small too: one SM takes 6.7 us for 17^2 nodes, bound by its reads
+// of the matrix from L2, where the launch over 150 CTAs takes 3.
+constexpr long COL_TAILN = 2304, COL_TAILC = 200;
+static int tail_level(const hp_problem *P, OpKind op, int tbytes, int vw) {
+  if (P->lv[P->L - 1].g.n > COL_TAILC) return P->L;
+  int l = std::max(1, col_level(P, op, tbytes, vw));
+  while (l < P->L && (P->lv[l].g.n > COL_TAILN || leg_level(P, op, l, tbytes, vw))) ++l;
+  return l + 1 < P->L ? l : P->L;
 }
 
 // Algorithmic bytes of the V-cycle's levels l0 .. L-1 as the per-level kernels would move

@@ -34,7 +34,7 @@ def run(tmp_path_factory):
     return go
 
 
-# levels run as legs (2D, for blocks and for one column), with a one-CTA coarse end (2D, 3D), a
+# levels run as legs (2D, for blocks and for one column), with a one-CTA coarse end (3D), a
 # whole PCG in one CTA, and as per-level kernels (3D)
 @pytest.mark.parametrize("dim,N,cols", [(2, 128, 5), (2, 128, 1), (2, 72, 5), (3, 24, 5), (2, 32, 3), (3, 32, 5)])
 def test_every_refused_launch_fails_its_solve(run, dim, N, cols):
