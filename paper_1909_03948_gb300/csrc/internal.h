@@ -373,6 +373,7 @@ struct LegArgs {
 };
 constexpr int LEG_MAXNU = 3;       // most sweeps of a leg
 int leg_tiles(const GridDesc &g);  // CTAs per column group (partials per column)
+constexpr int LEG_TILE = 512;      // nodes of a full one
 void launch_leg(LegArgs a, const GridDesc &g, bool full, bool up, int vw, int s, cudaStream_t st);
 
 // ---- launches that overlap the end of the kernel before them --------------------

@@ -29,6 +29,7 @@
 namespace hp {
 
 constexpr int LEG_X = 32, LEG_Y = 16;  // the last tile in a direction also takes the last node
+static_assert(LEG_X * LEG_Y == LEG_TILE, "the fill of the tiles");
 constexpr int LEG_N = 5;               // nodes per thread
 constexpr int LEG_NT = 224;            // threads at most (three sweeps: 41 columns of 5 strips)
 

@@ -2192,12 +2192,24 @@ static bool col_pcg_rule(const hp_problem *P, OpKind op, int tbytes, int vw, int
   return s <= (nc <= COL_TRIC && !edges ? 8 : 2) * NSM;
 }
 
-// Whether a level's legs run as one launch each (legs.cu): FP32, 2D, up to LEG_MAXNU sweeps
+// Whether a level's legs can run as one launch each (legs.cu): FP32, 2D, up to LEG_MAXNU sweeps
 // (the halo), neither asked to run as TMA tiles or step by step nor with the transfers fused
 // the other way.
 static bool leg_level(const hp_problem *P, OpKind op, int l, int tbytes, int vw) {
   return tbytes == 4 && P->dim == 2 && joined_level(P, l) && nu_at(P, l) <= LEG_MAXNU && !fuse_at(P, l) &&
          !tiled_level(P, op, l, vw);
+}
+
+// Whether they do for s columns: a last tile costs what a full one does, so where the tiles are
+// filled badly and there are more than two waves of CTAs, the per-step kernels are as fast or
+// faster.  Legs against those: 39^2 nodes (0.50 filled), 700 columns 1.12; 67^2 (0.58) 1.08 at 304;
+// 101^2 (0.71) 1.0 to 1.05 at 60, 1.05 to 1.09 at 152, 0.97 to 1.01 at 304, 1.01 to 1.04 at 700;
+// 77^2 (0.77) 0.95 at 304, 1.0 to 1.05 at 700; 65^2 (full) 0.86 at 608.
+static bool leg_rule(const hp_problem *P, OpKind op, int l, int tbytes, int vw, int s) {
+  if (!leg_level(P, op, l, tbytes, vw)) return false;
+  const GridDesc &g = P->lv[l].g;
+  const long tiles = leg_tiles(g);
+  return tiles * ((s + vw - 1) / vw) <= 4 * NSM || 4 * g.n >= 3l * LEG_TILE * tiles;
 }
 
 // First level of the one-launch coarse end of the V-cycle (a level above the coarsest one,
@@ -2296,7 +2308,7 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
     T w[4];
     smooth_weights<T>(P, op, l, w);
     if constexpr (sizeof(T) == 4) {
-      if (leg_level(P, op, l, 4, VW)) {
+      if (leg_rule(P, op, l, 4, VW, s)) {
         LegArgs a = leg_args(S, w, nu, op);
         a.r = rl[l];
         a.gs = gsl[l];
@@ -2390,7 +2402,7 @@ static void precondition(hp_problem *P, OpKind op, int s, const T *r0, T *z0, co
     T w[4];
     smooth_weights<T>(P, op, l, w);
     if constexpr (sizeof(T) == 4) {
-      if (leg_level(P, op, l, 4, VW)) {
+      if (leg_rule(P, op, l, 4, VW, s)) {
         LegArgs a = leg_args(S, w, nu, op);
         a.r = rl[l];
         a.gs = gsl[l];
@@ -2727,10 +2739,10 @@ static int kernels_per_iteration(const hp_problem *P, OpKind op, int tbytes, int
   int vc = 0;
   for (int l = 0; l < separate; ++l) {
     const int nu = nu_at(P, l);
-    if (leg_level(P, op, l, tbytes, vw)) vc += 2;
+    if (leg_rule(P, op, l, tbytes, vw, s)) vc += 2;
     else vc += (nu >= 2 ? nu - 1 : 1) + nu + (fuse_at(P, l) ? (nu >= 2 ? 1 : 2) : 3);
   }
-  if (separate > 0 && leg_level(P, op, 0, tbytes, vw) && !leg_dot(P->lv[0].g, (s + vw - 1) / vw)) vc += 1;
+  if (separate > 0 && leg_rule(P, op, 0, tbytes, vw, s) && !leg_dot(P->lv[0].g, (s + vw - 1) / vw)) vc += 1;
   return 7 + vc + 1 + 2 * (P->L == 1);
 }
 

@@ -67,3 +67,13 @@ def test_same_bits_after_a_change_of_precision():
     P.set_precision("fp32_ir")
     solves(P, 3, [{}, {"smem_tail": 15}])
     P.close()
+
+
+@pytest.mark.parametrize("N,cols", [(32, 330), (38, 700), (72, 250), (100, 45)])
+def test_same_bits_for_many_columns(N, cols):
+    """Column counts past the limits of the one-CTA PCG and of badly filled leg tiles (part of the
+    levels, or all, then run one launch per step)."""
+    from paper_1909_03948_gb300 import Problem
+    P = Problem(2, N, 0.1, 0.5, 0.01, np.zeros((0, 2)), rtol=RTOL)
+    solves(P, cols, [{}, {"smem_tail": 15}, {"smem_tail": 2}])
+    P.close()
