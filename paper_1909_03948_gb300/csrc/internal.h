@@ -429,6 +429,8 @@ struct MarchArgs {
   int np, s, ntx, nty, nzs;  // set by launch_march
 };
 int launch_march(MarchArgs a, const GridDesc &g, int mode, int s, cudaStream_t st);
+int march_tiles(const GridDesc &g);  // xy tiles
+constexpr int MARCH_TILE = 256;      // nodes of a full one in a plane
 
 // ---- dense.cu ---------------------------------------------------------------
 // G (s1 x s2, column-major, ldg) = X^T Y ; X: n x s1, Y: n x s2 (FP64)

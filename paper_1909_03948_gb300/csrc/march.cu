@@ -247,6 +247,11 @@ __global__ void __launch_bounds__(MA_NT, 2) k_march_full(const __grid_constant__
   }
 }
 
+static int ntx_of(const GridDesc &g) { return std::max(1, (g.np - 1 + MA_X - 1) / MA_X); }
+static int nty_of(const GridDesc &g) { return std::max(1, (g.np - 1 + MA_Y - 1) / MA_Y); }
+static_assert(MA_X * MA_Y == MARCH_TILE, "the fill of the tiles");
+int march_tiles(const GridDesc &g) { return ntx_of(g) * nty_of(g); }
+
 // CTAs per group: xy tiles times z segments -- of about 16 planes, or 8 while that leaves the
 // GPU's two CTAs per SM with fewer than two rounds
 static int march_segs(const GridDesc &g, int ng, int tiles) {
@@ -258,8 +263,8 @@ int launch_march(MarchArgs a, const GridDesc &g, int mode, int s, cudaStream_t s
   const int ng = (s + 3) / 4;
   a.np = g.np;
   a.s = s;
-  a.ntx = std::max(1, (g.np - 1 + MA_X - 1) / MA_X);
-  a.nty = std::max(1, (g.np - 1 + MA_Y - 1) / MA_Y);
+  a.ntx = ntx_of(g);
+  a.nty = nty_of(g);
   a.nzs = march_segs(g, ng, a.ntx * a.nty);
   const dim3 gr(a.ntx * a.nty * a.nzs, ng);
   switch (mode) {

@@ -1891,6 +1891,10 @@ template <typename T, int MODE> static double st_bytes(const GridDesc &g, const 
 // matvec 89 -> 57 us; 33^3 nodes, 64 columns (575,000): sweep 15.7 -> 14.2 us.
 constexpr long MARCH_MIN = 500000;
 static bool march_rule(const GridDesc &g, int ng) { return g.dim == 3 && g.n * ng >= MARCH_MIN; }
+// and on a grid that fills its xy tiles: prior solves on 37^3 nodes (0.53), 40 columns, took 2,314 us
+// against 2,185, on 41^3 (0.66) 0.86 to 0.96 of the row kernel's time.  (The Chebyshev iteration
+// is faster either way: 954 against 1,854 us for the mass solve on 37^3.)
+static bool march_filled(const GridDesc &g) { return 10l * g.np * g.np >= 6l * MARCH_TILE * march_tiles(g); }
 
 // Whether M is solved by the Chebyshev iteration: where its stencil runs as the marching kernel,
 // which takes a whole step in one launch and four passes over a block where CG's takes eleven.
@@ -1921,7 +1925,7 @@ static void st_launch(const GridDesc &g, const Stencil<T> &S, const T *X, long g
   }
   const int ng = (s + VW - 1) / VW;
   if constexpr (sizeof(T) == 4 && VW == 4 && MODE != M_APPLY) {
-    if (S.full && march_rule(g, ng)) {
+    if (S.full && march_rule(g, ng) && march_filled(g)) {
       MarchArgs a{};
       a.diag = S.diag;
       a.invdiag = S.invdiag;
