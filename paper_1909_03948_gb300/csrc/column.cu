@@ -442,8 +442,9 @@ __device__ __forceinline__ void col_prolong(const ColLevel &lf, const ColLevel &
 //   HELD: the lower triangle (row i at i (i + 1) / 2) lies in shared memory: below the
 //     diagonal block the 32 lanes read words at triangular-number distances (which all differ
 //     in their bank), above it consecutive words;
-//   else the matrix is read from L2, CO_RUN loads in flight per warp (17^2 nodes: 334 KB in
-//     9,700 clocks; with the loads under conditions, which serialised them, 30,000).
+//   else the matrix is read from L2, CO_RUN loads in flight per warp (17^2 nodes, two such runs
+//     per share and one more load: 334 KB in 9,700 clocks; with the loads under conditions,
+//     which serialised them, 30,000).
 // rp: R in share order ([share][q], k = share + 8 q), so that four values are one load.
 constexpr int CO_RUN = 18;
 template <bool HELD> __device__ __noinline__ void col_coarse(const float *inv, int tri, const ColLevel &l, int offs) {

@@ -385,9 +385,10 @@ void launch_leg(LegArgs a, const GridDesc &g, bool full, bool up, int vw, int s,
 // kernel is resident while the one before it still stores, and a non-coherent load (__ldg, or
 // what the compiler makes of a const __restrict__ parameter) is only defined, and only kept behind
 // the wait, for data that is constant over the kernel's whole life.  The stencils and the
-// coarse inverse, written when a point is set, are.  A solve is a chain of hundreds of launches of a few us: one
-// column on 257^2 nodes 1.76 -> 1.70 ms, a 3D block of 24^3 cells' full Hessian 3.71 -> 3.49 ms,
-// a gradient on 257^2 nodes 4.17 -> 3.97 ms.
+// coarse inverse, written when a point is set, are.
+// A solve is a chain of hundreds of launches of a few us.  With and without: one Hessian column on
+// 257^2 nodes 1.67 and 1.83 ms, a gradient there 4.05 and 4.26, 7 full-Newton columns on 49^3
+// nodes 4.26 and 4.47, one stiffness solve on 1,025^2 nodes 1.44 and 1.54.
 // Not for kernels of very many short CTAs: the wait costs each of them some hundred clocks
 // (k_prolong_add, 64,000 CTAs of one node per thread: 44 -> 72 us).
 template <class... P, class... A>

@@ -670,10 +670,10 @@ __global__ void __launch_bounds__(TL3_NT) k_st_tile3(const __grid_constant__ CUt
 // ---------------------------------------------------------------------------
 // FP64 stencils of column-major blocks (the refinement's residual and the operator
 // applications), one node per thread over the flattened grid, C64 columns per thread that
-// share the node's coefficients and addresses (one where an odd count ends).  Bound by the FP64 pipe (2 lanes per clock and
-// SM): 15 or 17 operations per node and column over all Kuhn edges in 3D.  The row kernel gives
-// a row of 65 nodes three warps, the third with one lane, and pays for 96.  65^3 nodes, 120
-// columns: A x 1,310 -> 823 us (840 us is the pipe's time without the boundary), its residual
+// share the node's coefficients and addresses (one where an odd count ends).  Bound by the FP64
+// pipe (2 lanes per clock and SM): 15 or 17 operations per node and column over all Kuhn edges in
+// 3D.  The row kernel gives a row of 65 nodes three warps, the third with one lane, and pays for
+// 96.  65^3 nodes, 120 columns: A x 1,310 -> 823 us (840 us is the pipe's time without the boundary), its residual
 // 1,545 -> 966; K's residual 829 -> 536.  A call for one column there takes 27.6 us, 34.8 when the
 // column was computed twice (the row kernel 32.9).
 constexpr int C64 = 2;

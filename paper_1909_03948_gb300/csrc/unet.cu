@@ -167,13 +167,14 @@ __global__ void __launch_bounds__(256) k_conv_fwd(ConvIn I, const __nv_bfloat16 
 // stages: a slab's loads to registers are under way while the MMAs of the slab before start;
 // a stage is refilled once the tcgen05.commit of the MMAs that read it has arrived on
 // its mbarrier.
-// Bound: the MMAs.  With few output channels an MMA's time is the reading of its 128 pixels (4 KB)
-// from shared memory, not its arithmetic: 63 clocks each in the 16-channel layers, of which
-// the read takes 32 or more, 87 with 32 and 64 channels.  With one thread per accumulator row, 16
-// warps per SM, the staging (load, split into terms, store) was exposed beside them: hence two
-// threads per row of up to 64 registers (four CTAs per SM), an item's place computed once per
-// tile, two values per conversion, weights by asynchronous copies.  The forward pass of 60
-// images of 264 x 264: 4.23 -> 2.92 ms (MMAs at 32 clocks: 1.2 ms).
+// Bound: the MMAs and what surrounds them.  Per MMA a 16-channel layer takes 65 to 74 clocks of an
+// SM, layers of 32 and 64 channels 84 to 127 where they fill the GPU (12 images of 264 x 264, whole
+// launches counted), with the tensor pipe 11 to 35 % busy: its arithmetic at N = 16 is 8 of
+// those clocks; reading its 128 pixels (4 KB) from shared memory would take 32.  With one thread
+// per accumulator row, 16 warps per SM, the staging (load, split into terms, store) was exposed
+// beside them: hence two threads per row of up to 64 registers (four CTAs per SM), an item's
+// place computed once per tile, two values per conversion, weights by asynchronous copies.  The
+// forward pass of 60 images of 264 x 264: 4.23 -> 2.92 ms.
 // ---------------------------------------------------------------------------
 constexpr int TC_NT = 256;   // threads per CTA: two per accumulator row (tensor-memory lane)
 constexpr int TC_TR = 16;    // tile rows
@@ -485,7 +486,10 @@ __global__ void __launch_bounds__(256) k_conv_bwd_data(const float *__restrict__
 // Bound: the FP32 pipes and the issue slots (16 images of 72^2 pixels: 3.4 G multiply-adds).
 // One block per (co, ci), reading nine inputs per pixel with their index divisions, took 7.7
 // ms for that batch's 15 layers and the bias sums 1.3 ms; the marching lanes with plain loads
-// 2.6 ms (each row waited for its loads from L2).
+// 2.6 ms (each row waited for its loads from L2).  The whole loss and gradient takes 1.47 ms, of
+// which adding the lanes in pairs and the shorter FP32 sums are 0.09.
+// GW_ROWS: a warp's loads of a set are in flight in as many registers; 18 divides the 72, 36 and
+// 18 rows of a 64^2 problem's training images, another height leaves part of its last unit idle.
 constexpr int GW_C = 8, GW_ROWS = 18, GW_WARPS = 8;
 constexpr int GW_HELD = 16;  // most sets whose FP32 sums a lane carries on
 constexpr int GW_INW = 48;   // floats per staged input row: 32 lanes and the units' halos
